@@ -18,8 +18,7 @@
 //
 // The backward pass through a layer's input is the same convolution with the kernel mirrored
 // and its channels transposed (host-packed operand), masked by the ReLU of the layer below.
-// The weight gradients are reductions over the voxels of X_shift^T dY in FP32 on the CUDA
-// cores; Adam updates FP32 master weights, which are then repacked into the BF16 operands.
+// The weight gradients contract X_shift^T dY over the voxels (wgrad_kernel); Adam updates FP32 master weights, which are then repacked into the BF16 operands.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -190,19 +189,6 @@ __device__ __forceinline__ void epilogue(const ConvArgs& a, long long v, const f
         a.jout[base + c * plane] = __ldcg(a.jres + base + c * plane) + a.scale * rr[c];
     }
   }
-}
-
-// neighbour voxel of v for tap t = (dz, dy, dx) + 1 in row-major order, -1 outside the window
-__device__ __forceinline__ long long neighbour(long long v, int t, int nx, int ny, int nz) {
-  const int dz = t / 9 - 1, dy = (t / 3) % 3 - 1, dx = t % 3 - 1;
-  const long long plane = (long long)nx * ny;
-  const int z = (int)(v / plane);
-  const int rem = (int)(v - (long long)z * plane);
-  const int y = rem / nx, x = rem - y * nx;
-  const int zz = z + dz;
-  if (zz < 0 || zz >= nz) return -1;
-  const int yy = (y + dy + ny) % ny, xx = (x + dx + nx) % nx;
-  return (long long)zz * plane + (long long)yy * nx + xx;
 }
 
 __global__ void __launch_bounds__(kThreads) conv_kernel(ConvArgs a) {
@@ -653,52 +639,234 @@ __global__ void loss_kernel(const float* j, const float* t, const float* r, __nv
     d[0] = reinterpret_cast<const uint4*>(o)[0];
     d[1] = reinterpret_cast<const uint4*>(o)[1];
   }
+  __shared__ double red[32];
   for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-  if ((threadIdx.x & 31) == 0) atomicAdd(loss, acc);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < (int)(blockDim.x >> 5); ++w) acc += red[w];
+    atomicAdd(loss, acc);
+  }
 }
 
-// dW[t][ci][co] += sum over voxels of X[v + off(t)][ci] dY[v][co]; db[co] += sum dY[v][co]
-// (tap 13 blocks).  Block = one tap x one chunk of voxels; thread = (ci, co).
-constexpr int kGradChunk = 1024;
-__global__ void __launch_bounds__(256) wgrad_kernel(const __nv_bfloat16* X, const __nv_bfloat16* dY,
-                                                    float* dW, float* db, int nx, int ny, int nz,
-                                                    int cin, int cout) {
-  __shared__ float sx[64][16];
-  __shared__ float sy[64][16];
-  __shared__ long long snb[64];
-  const int t = blockIdx.y;
-  const long long V = (long long)nx * ny * nz;
-  const long long v0 = (long long)blockIdx.x * kGradChunk;
-  const int ci = threadIdx.x >> 4, co = threadIdx.x & 15;
-  float acc = 0.0f, accb = 0.0f;
-  for (int s = 0; s < kGradChunk; s += 64) {
-    if (threadIdx.x < 64) {
-      const long long v = v0 + s + threadIdx.x;
-      snb[threadIdx.x] = v < V ? neighbour(v, t, nx, ny, nz) : -2;
+// Weight gradients dW[t][ci][co] = sum over voxels v of X[v + off(t)][ci] dY[v][co] and bias
+// gradients db[co] = sum dY[v][co] of the three layers in one launch (blockIdx.y = layer).  Per
+// tap this is a 16 x 16 product contracted over all voxels: on the tensor cores with the voxels
+// as K, straight from the channel-last rows (ldmatrix transposes both operands), FP32
+// accumulators.  The warp-level mma carries it: the outputs are 16 x 16 tiles, so a tcgen05 tile
+// (M >= 64) would have to gather several taps' shifted rows as one operand, and the tensor rate
+// is not what binds (below).  A CTA takes a run of rows (z, x-segment, y) of up to 128 voxels:
+// warp w owns the taps (dz, dy) = (w / 3 - 1, w % 3 - 1), dx = -1, 0, 1 and keeps their three
+// accumulators; the nine staged input rows serve all 27 taps, and going to the next y stages
+// only the three new rows (asynchronous copies, one row ahead of the products).  Each row's
+// products are added to the running sums in FP32, so a chain inside the tensor core is at most
+// 8 long.  Every CTA writes its partial sums; wgrad_reduce_kernel adds them in a fixed order
+// (in FP64), so gradients are reproducible bit for bit.
+// Bound: L2 and issue latency of the staging (16 KB per row and layer; the products are 1 % of
+// the tensor rate).  A training step at 128 x 128 x 32 voxels took 3.10 ms with FP32 FMA reductions
+// per tap and float atomics (2.7 ms of it here) and takes 0.43 ms.
+constexpr int kSeg = 128;                            // voxels of a row segment
+constexpr int kGradWarps = 9;
+constexpr int kGradThreads = 32 * kGradWarps;
+constexpr uint32_t kSegBytes = (uint32_t)(kSeg + 2) * 32u;
+constexpr uint32_t kGradSmem = 12u * kSegBytes + 2u * kSeg * 32u;   // [4 y][3 z] input rows, 2 dY rows
+constexpr int kPart = kTaps * kCh * kCh + kCh;       // partial sums per CTA and layer: dW, db
+
+struct GradArgs {
+  const __nv_bfloat16* x[3];    // layer inputs [V][16]
+  const __nv_bfloat16* dy[3];   // gradients of the layer outputs [V][16]
+  float* part;                  // [3][gridDim.x][kPart]
+  int nx, ny, nz;
+};
+
+// byte offset of the 16-byte half h of staged voxel xi: the halves of every other group of four
+// voxels are exchanged, so the eight rows of an ldmatrix tile start in different banks
+__device__ __forceinline__ uint32_t seg_off(int xi, int h) {
+  return (uint32_t)xi * 32u + (uint32_t)((h ^ (xi >> 2)) & 1) * 16u;
+}
+__device__ __forceinline__ void ldsm4t(uint32_t a, uint32_t (&r)[4]) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(a)
+               : "memory");
+}
+__device__ __forceinline__ void mma16816(float* d, const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+  asm volatile(
+      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
+      "{%0,%1,%2,%3};"
+      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+
+__global__ void __launch_bounds__(kGradThreads, 2) wgrad_kernel(GradArgs g) {
+  extern __shared__ __align__(128) unsigned char smem[];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int layer = blockIdx.y;
+  const __nv_bfloat16* const X = g.x[layer];
+  const __nv_bfloat16* const dY = g.dy[layer];
+  const uint32_t sx = smem_u32(smem), sy = sx + 12u * kSegBytes;
+  const int nseg = (g.nx + kSeg - 1) / kSeg;
+  const long long rows = (long long)g.nz * nseg * g.ny;
+  const long long r0 = rows * blockIdx.x / gridDim.x, r1 = rows * (blockIdx.x + 1) / gridDim.x;
+  const int pz = warp / 3, py = warp - 3 * pz;       // this warp's (dz, dy) + 1
+  // ldmatrix lane -> (voxel, half): matrices (v 0-7, c 0-7), (v 0-7, c 8-15), (v 8-15, c 0-7), ...
+  const int lv = ((lane >> 4) & 1) * 8 + (lane & 7), lh = (lane >> 3) & 1;
+  float sum[3][8], bsum[8];
+#pragma unroll
+  for (int i = 0; i < 24; ++i) sum[i >> 3][i & 7] = 0.0f;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) bsum[i] = 0.0f;
+  const uint32_t one2 = 0x3F803F80u;                 // two BF16 ones
+  const uint32_t ones[4] = {one2, one2, one2, one2};
+
+  // stage the input rows (z - 1 .. z + 1, y) of a segment with a halo voxel at each end; voxels
+  // beyond the segment are zero (so are dY's: products beyond the row add nothing)
+  auto stage_x = [&](int slot, int z, int y, int s0, int len, int kk) {
+    for (int pl = 0; pl < 3; ++pl) {
+      const int zz = z + pl - 1;
+      if (zz < 0 || zz >= g.nz) continue;            // its warps skip their products
+      const __nv_bfloat16* row = X + ((long long)zz * g.ny + y) * (long long)g.nx * kCh;
+      const uint32_t dst = sx + (uint32_t)(slot * 3 + pl) * kSegBytes;
+      for (int i = tid; i < 2 * (kk + 2); i += kGradThreads) {
+        const int xi = i >> 1, h = i & 1;
+        int x = s0 + xi - 1;
+        x = x < 0 ? x + g.nx : x >= g.nx ? x - g.nx : x;
+        const bool in = xi < len + 2;
+        cp_async16(dst + seg_off(xi, h), in ? row + (long long)x * kCh + h * 8 : X, in ? 16u : 0u);
+      }
     }
-    __syncthreads();
-    for (int e = threadIdx.x; e < 64 * 16; e += 256) {
-      const int q = e >> 4, c = e & 15;
-      const long long v = v0 + s + q;
-      const long long nb = snb[q];
-      sy[q][c] = nb > -2 ? __bfloat162float(dY[v * kCh + c]) : 0.0f;
-      sx[q][c] = nb >= 0 ? __bfloat162float(X[nb * kCh + c]) : 0.0f;
+  };
+  auto stage_y = [&](int buf, int z, int y, int s0, int len, int kk) {
+    const __nv_bfloat16* row = dY + (((long long)z * g.ny + y) * g.nx + s0) * kCh;
+    const uint32_t dst = sy + (uint32_t)buf * kSeg * 32u;
+    for (int i = tid; i < 2 * kk; i += kGradThreads) {
+      const int xi = i >> 1, h = i & 1;
+      cp_async16(dst + seg_off(xi, h), xi < len ? row + xi * kCh + h * 8 : dY, xi < len ? 16u : 0u);
     }
-    __syncthreads();
-#pragma unroll 8
-    for (int q = 0; q < 64; ++q) {
-      acc = fmaf(sx[q][ci], sy[q][co], acc);
-      accb += sy[q][co];
+  };
+
+  int base = 0, buf = 0;
+  bool staged = false;                               // this row was staged during the last one
+  for (long long r = r0; r < r1; ++r) {
+    const int y = (int)(r % g.ny);
+    const int zs = (int)(r / g.ny);
+    const int z = zs / nseg, s0 = (zs - z * nseg) * kSeg;
+    const int len = min(kSeg, g.nx - s0), kk = (len + 15) & ~15;
+    if (!staged) {
+      __syncthreads();                               // the last row's products are done
+      for (int d = 0; d < 3; ++d) {
+        int yy = y + d - 1;
+        yy = yy < 0 ? yy + g.ny : yy >= g.ny ? yy - g.ny : yy;
+        stage_x((base + d) & 3, z, yy, s0, len, kk);
+      }
+      stage_y(buf, z, y, s0, len, kk);
     }
+    cp_async_wait_all();
     __syncthreads();
+    staged = r + 1 < r1 && y + 1 < g.ny;
+    if (staged) {
+      const int yn = y + 2 >= g.ny ? y + 2 - g.ny : y + 2;
+      stage_x((base + 3) & 3, z, yn, s0, len, kk);
+      stage_y(buf ^ 1, z, y + 1, s0, len, kk);
+    }
+    if (z + pz - 1 >= 0 && z + pz - 1 < g.nz) {
+      const uint32_t xrow = sx + (uint32_t)(((base + py) & 3) * 3 + pz) * kSegBytes;
+      const uint32_t yrow = sy + (uint32_t)buf * kSeg * 32u;
+      float acc[3][8], bacc[8];
+#pragma unroll
+      for (int i = 0; i < 24; ++i) acc[i >> 3][i & 7] = 0.0f;
+#pragma unroll
+      for (int i = 0; i < 8; ++i) bacc[i] = 0.0f;
+      for (int k = 0; k < kk; k += 16) {
+        uint32_t b[4];
+        ldsm4t(yrow + seg_off(k + lv, lh), b);
+#pragma unroll
+        for (int dx = 0; dx < 3; ++dx) {
+          uint32_t a[4];
+          ldsm4t(xrow + seg_off(k + lv + dx, lh), a);
+          mma16816(acc[dx], a, b[0], b[2]);
+          mma16816(acc[dx] + 4, a, b[1], b[3]);
+        }
+        if (warp == 4) {                             // column sums of dY: the bias gradient
+          mma16816(bacc, ones, b[0], b[2]);
+          mma16816(bacc + 4, ones, b[1], b[3]);
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < 24; ++i) sum[i >> 3][i & 7] += acc[i >> 3][i & 7];
+      if (warp == 4) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) bsum[i] += bacc[i];
+      }
+    }
+    if (staged) {
+      base = (base + 1) & 3;
+      buf ^= 1;
+    }
   }
-  if (ci < cin && co < cout) atomicAdd(dW + ((size_t)t * cin + ci) * cout + co, acc);
-  if (t == 13 && ci == 0 && co < cout) atomicAdd(db + co, accb);
+  // accumulator (row, column): rows lane / 4 and + 8, columns 2 (lane % 4) + {0, 1} and + 8
+  float* out = g.part + ((size_t)layer * gridDim.x + blockIdx.x) * kPart;
+  const int row = lane >> 2, col = 2 * (lane & 3);
+#pragma unroll
+  for (int dx = 0; dx < 3; ++dx) {
+    float* t = out + (pz * 9 + py * 3 + dx) * (kCh * kCh);
+#pragma unroll
+    for (int n = 0; n < 2; ++n)
+#pragma unroll
+      for (int m = 0; m < 2; ++m)
+        *reinterpret_cast<float2*>(t + (row + 8 * m) * kCh + col + 8 * n) =
+            make_float2(sum[dx][4 * n + 2 * m], sum[dx][4 * n + 2 * m + 1]);
+  }
+  if (warp == 4 && row == 0) {
+#pragma unroll
+    for (int n = 0; n < 2; ++n)
+      *reinterpret_cast<float2*>(out + kTaps * kCh * kCh + col + 8 * n) =
+          make_float2(bsum[4 * n], bsum[4 * n + 1]);
+  }
+}
+
+// g[i] = the sum over the CTAs' partial sums, in FP64 and in a fixed order: 8 lanes of partial
+// runs per parameter.  Parameter order: W1, b1, W2, b2, W3, b3 (W[tap][ci][co])
+__global__ void __launch_bounds__(256) wgrad_reduce_kernel(const float* part, int ncta, float* g,
+                                                           int n) {
+  __shared__ double red[8][32];
+  const int lane = threadIdx.x & 31, run = threadIdx.x >> 5;
+  const int i = blockIdx.x * 32 + lane;
+  double acc = 0.0;
+  if (i < n) {
+    constexpr int cin[3] = {3, 16, 16}, cout[3] = {16, 16, 3};
+    int l = 0, o = i;
+    while (l < 2 && o >= kTaps * cin[l] * cout[l] + cout[l]) {
+      o -= kTaps * cin[l] * cout[l] + cout[l];
+      ++l;
+    }
+    const int nw = kTaps * cin[l] * cout[l];
+    int e;
+    if (o < nw) {
+      const int co = o % cout[l], tc = o / cout[l];
+      e = (tc / cin[l]) * (kCh * kCh) + (tc % cin[l]) * kCh + co;
+    } else {
+      e = kTaps * kCh * kCh + (o - nw);
+    }
+    const float* p = part + (size_t)l * ncta * kPart + e;
+#pragma unroll 4
+    for (int c = run; c < ncta; c += 8) acc += (double)p[(size_t)c * kPart];
+  }
+  red[run][lane] = acc;
+  __syncthreads();
+  if (run == 0 && i < n) {
+    double v = red[0][lane];
+#pragma unroll
+    for (int q = 1; q < 8; ++q) v += red[q][lane];
+    g[i] = (float)v;
+  }
 }
 
 // Adam (Kingma and Ba 2015) on the FP32 master parameters, bias-corrected
+// (nothing is changed when a bounded wait of the gradient gave up: *err)
 __global__ void adam_kernel(float* p, const float* g, float* m, float* v, int n, float lr,
-                            float b1, float b2, float eps, float c1, float c2) {
+                            float b1, float b2, float eps, float c1, float c2, const int* err) {
+  if (*err) return;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
     const float gi = g[i];
     const float mi = b1 * m[i] + (1.0f - b1) * gi;
@@ -709,11 +877,20 @@ __global__ void adam_kernel(float* p, const float* g, float* m, float* v, int n,
   }
 }
 
-// operand B of one layer from FP32 weights W[27][cin][cout]: K-major canonical layout,
-// B_t[n][k] = W[t][k][n] (forward) or the mirrored tap with channels swapped,
-// B_t[n][k] = W[26 - t][n][k] (backward through the input)
-__global__ void pack_weights_kernel(const float* W, __nv_bfloat16* B, int cin, int cout, int bwd) {
-  const int t = blockIdx.x;
+// operands B from the FP32 parameters, one launch: blockIdx.y = layer, + 3 for the backward
+// form.  K-major canonical layout, B_t[n][k] = W[t][k][n] (forward) or the mirrored tap with
+// channels swapped, B_t[n][k] = W[26 - t][n][k] (backward through the input)
+struct PackArgs {
+  const float* W[3];
+  __nv_bfloat16* B[6];
+};
+__global__ void pack_weights_kernel(PackArgs p) {
+  constexpr int kci[3] = {3, 16, 16}, kco[3] = {16, 16, 3};
+  const int t = blockIdx.x, l = blockIdx.y % 3;
+  const bool bwd = blockIdx.y >= 3;
+  const int cin = kci[l], cout = kco[l];
+  const float* W = p.W[l];
+  __nv_bfloat16* B = p.B[blockIdx.y];
   for (int e = threadIdx.x; e < 256; e += blockDim.x) {
     const int n = e >> 4, k = e & 15;
     float val = 0.0f;
@@ -745,8 +922,9 @@ struct gempic_denoiser {
   long long cap = 0;
   __nv_bfloat16* act[6] = {};
   float* r = nullptr;
-  double* loss = nullptr;
-  int* err = nullptr;
+  float* part = nullptr;       // partial weight gradients [3][nsm][kPart] (first gradient)
+  double* loss = nullptr;      // {loss sum, status word}: read back in one copy
+  int* err = nullptr;          // the status word, in loss[1]
 };
 
 namespace {
@@ -781,10 +959,13 @@ cudaError_t grow(gempic_denoiser* d, long long V) {
 }
 
 cudaError_t repack(gempic_denoiser* d, cudaStream_t s) {
+  PackArgs a;
   for (int l = 0; l < 3; ++l) {
-    pack_weights_kernel<<<kTaps, 256, 0, s>>>(d->p + woff(l), d->wf[l], kCin[l], kCout[l], 0);
-    pack_weights_kernel<<<kTaps, 256, 0, s>>>(d->p + woff(l), d->wb[l], kCin[l], kCout[l], 1);
+    a.W[l] = d->p + woff(l);
+    a.B[l] = d->wf[l];
+    a.B[3 + l] = d->wb[l];
   }
+  pack_weights_kernel<<<dim3(kTaps, 6), 256, 0, s>>>(a);
   return cudaGetLastError();
 }
 
@@ -928,9 +1109,11 @@ gempic_status gempic_denoiser_create(const float* params, double scale, gempic_d
     e = cudaMalloc(&d->wf[l], kTaps * 256 * sizeof(__nv_bfloat16));
     if (e == cudaSuccess) e = cudaMalloc(&d->wb[l], kTaps * 256 * sizeof(__nv_bfloat16));
   }
-  if (e == cudaSuccess) e = cudaMalloc(&d->loss, sizeof(double));
-  if (e == cudaSuccess) e = cudaMalloc(&d->err, sizeof(int));
-  if (e == cudaSuccess) e = cudaMemset(d->err, 0, sizeof(int));
+  if (e == cudaSuccess) e = cudaMalloc(&d->loss, 2 * sizeof(double));
+  if (e == cudaSuccess) e = cudaMemset(d->loss, 0, 2 * sizeof(double));
+  if (e == cudaSuccess) d->err = reinterpret_cast<int*>(d->loss + 1);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(wgrad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGradSmem);
   if (e == cudaSuccess) e = cudaMemset(d->m, 0, n * sizeof(float));
   if (e == cudaSuccess) e = cudaMemset(d->v, 0, n * sizeof(float));
   if (e == cudaSuccess) {
@@ -983,20 +1166,22 @@ gempic_status gempic_denoiser_apply(gempic_denoiser* d, const float* j_in, float
   return check_err(d, s);
 }
 
-gempic_status gempic_denoiser_grad(gempic_denoiser* d, const float* j_in, const float* j_target,
-                                   int32_t nx, int32_t ny, int32_t nz, int32_t z_margin,
-                                   double* loss, float* grad_host, void* cuda_stream) {
-  if (!d || !j_in || !j_target || !grid_ok(nx, ny, nz) || z_margin < 0 || 2 * z_margin >= nz)
-    return GEMPIC_EINVAL;
-  cudaStream_t s = (cudaStream_t)cuda_stream;
+}  // extern "C"
+
+namespace {
+
+// the loss sum and the gradient of the parameters into d->loss, d->g (device), no wait
+gempic_status gradient(gempic_denoiser* d, const float* j_in, const float* j_target, int nx, int ny,
+                       int nz, int z_margin, cudaStream_t s) {
   const long long V = (long long)nx * ny * nz;
   cudaError_t e = grow(d, V);
+  if (e == cudaSuccess && !d->part) {
+    e = cudaMalloc(&d->part, (size_t)3 * d->nsm * kPart * sizeof(float));
+    if (e != cudaSuccess) d->part = nullptr;
+  }
   if (e != cudaSuccess) return e == cudaErrorMemoryAllocation ? GEMPIC_ENOMEM : GEMPIC_ECUDA;
   const int blocks = (int)std::min<long long>((V + 255) / 256, 8LL * d->nsm);
-  const size_t n = nparams();
-  e = cudaMemsetAsync(d->g, 0, n * sizeof(float), s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(d->loss, 0, sizeof(double), s);
-  if (e != cudaSuccess) return GEMPIC_ECUDA;
+  if (cudaMemsetAsync(d->loss, 0, sizeof(double), s) != cudaSuccess) return GEMPIC_ECUDA;
   pack_input_kernel<<<blocks, 256, 0, s>>>(j_in, d->act[0], nx, ny, 0, nz, (float)(1.0 / d->scale));
   e = forward(d, nx, ny, nz, 0, nz, nullptr, nullptr, d->r, s);
   if (e != cudaSuccess) return GEMPIC_ECUDA;
@@ -1026,43 +1211,72 @@ gempic_status gempic_denoiser_grad(gempic_denoiser* d, const float* j_in, const 
     e = conv(d, b, s);
   }
   if (e != cudaSuccess) return GEMPIC_ECUDA;
-  const dim3 gg((unsigned)((V + kGradChunk - 1) / kGradChunk), kTaps);
-  const __nv_bfloat16* xs[3] = {d->act[0], d->act[1], d->act[2]};
-  const __nv_bfloat16* ds[3] = {dh1, dh2, dr};
-  for (int l = 0; l < 3; ++l)
-    wgrad_kernel<<<gg, 256, 0, s>>>(xs[l], ds[l], d->g + woff(l), d->g + boff(l), nx, ny, nz,
-                                    kCin[l], kCout[l]);
-  e = cudaGetLastError();
-  double lv = 0.0;
-  if (e == cudaSuccess) e = cudaMemcpyAsync(&lv, d->loss, sizeof(double), cudaMemcpyDeviceToHost, s);
-  if (e == cudaSuccess && grad_host)
-    e = cudaMemcpyAsync(grad_host, d->g, n * sizeof(float), cudaMemcpyDeviceToHost, s);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-  if (e != cudaSuccess) return GEMPIC_ECUDA;
-  if (loss) *loss = lv / count;
-  return check_err(d, s);
+  // two CTAs per SM over the three layers, at least one row each
+  const long long rows = (long long)nz * ny * ((nx + kSeg - 1) / kSeg);
+  const int gx = (int)std::min<long long>(rows, std::max(1, 2 * d->nsm / 3));
+  const GradArgs ga{{d->act[0], d->act[1], d->act[2]}, {dh1, dh2, dr}, d->part, nx, ny, nz};
+  wgrad_kernel<<<dim3((unsigned)gx, 3), kGradThreads, kGradSmem, s>>>(ga);
+  const int n = (int)nparams();
+  wgrad_reduce_kernel<<<(n + 31) / 32, 256, 0, s>>>(d->part, gx, d->g, n);
+  return cudaGetLastError() == cudaSuccess ? GEMPIC_OK : GEMPIC_ECUDA;
 }
 
+// wait for the stream; the loss and the status word
+gempic_status finish(gempic_denoiser* d, double count, double* loss, cudaStream_t s) {
+  double back[2] = {0.0, 0.0};
+  cudaError_t e = cudaMemcpyAsync(back, d->loss, sizeof(back), cudaMemcpyDeviceToHost, s);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  if (e != cudaSuccess) return GEMPIC_ECUDA;
+  if (loss) *loss = back[0] / count;
+  int err = 0;
+  std::memcpy(&err, &back[1], sizeof(err));
+  return err ? GEMPIC_ETIMEOUT : GEMPIC_OK;
+}
+
+bool grad_args_ok(gempic_denoiser* d, const float* j_in, const float* j_target, int nx, int ny, int nz,
+                  int z_margin) {
+  return d && j_in && j_target && grid_ok(nx, ny, nz) && z_margin >= 0 && 2 * z_margin < nz;
+}
+
+}  // namespace
+
+extern "C" {
+
+gempic_status gempic_denoiser_grad(gempic_denoiser* d, const float* j_in, const float* j_target,
+                                   int32_t nx, int32_t ny, int32_t nz, int32_t z_margin,
+                                   double* loss, float* grad_host, void* cuda_stream) {
+  if (!grad_args_ok(d, j_in, j_target, nx, ny, nz, z_margin)) return GEMPIC_EINVAL;
+  cudaStream_t s = (cudaStream_t)cuda_stream;
+  const gempic_status st = gradient(d, j_in, j_target, nx, ny, nz, z_margin, s);
+  if (st != GEMPIC_OK) return st;
+  if (grad_host && cudaMemcpyAsync(grad_host, d->g, nparams() * sizeof(float), cudaMemcpyDeviceToHost,
+                                   s) != cudaSuccess)
+    return GEMPIC_ECUDA;
+  return finish(d, 3.0 * (double)nx * ny * (nz - 2 * z_margin), loss, s);
+}
+
+// one wait per step: Adam and the repacking are queued behind the gradient and change nothing
+// when a bounded wait in it gave up
 gempic_status gempic_denoiser_train_step(gempic_denoiser* d, const float* j_in,
                                          const float* j_target, int32_t nx, int32_t ny,
                                          int32_t nz, int32_t z_margin, double lr, double* loss,
                                          void* cuda_stream) {
   if (!(lr > 0) || !std::isfinite(lr)) return GEMPIC_EINVAL;
-  gempic_status st = gempic_denoiser_grad(d, j_in, j_target, nx, ny, nz, z_margin, loss, nullptr,
-                                          cuda_stream);
-  if (st != GEMPIC_OK) return st;
+  if (!grad_args_ok(d, j_in, j_target, nx, ny, nz, z_margin)) return GEMPIC_EINVAL;
   cudaStream_t s = (cudaStream_t)cuda_stream;
-  d->step++;
+  gempic_status st = gradient(d, j_in, j_target, nx, ny, nz, z_margin, s);
+  if (st != GEMPIC_OK) return st;
+  const long long step = d->step + 1;
   const float b1 = 0.9f, b2 = 0.999f;
-  const float c1 = (float)(1.0 - std::pow(0.9, (double)d->step));
-  const float c2 = (float)(1.0 - std::pow(0.999, (double)d->step));
+  const float c1 = (float)(1.0 - std::pow(0.9, (double)step));
+  const float c2 = (float)(1.0 - std::pow(0.999, (double)step));
   const int n = (int)nparams();
   adam_kernel<<<(n + 255) / 256, 256, 0, s>>>(d->p, d->g, d->m, d->v, n, (float)lr, b1, b2, 1e-8f,
-                                               c1, c2);
-  cudaError_t e = cudaGetLastError();
-  if (e == cudaSuccess) e = repack(d, s);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-  return e == cudaSuccess ? GEMPIC_OK : GEMPIC_ECUDA;
+                                               c1, c2, d->err);
+  if (cudaGetLastError() != cudaSuccess || repack(d, s) != cudaSuccess) return GEMPIC_ECUDA;
+  st = finish(d, 3.0 * (double)nx * ny * (nz - 2 * z_margin), loss, s);
+  if (st == GEMPIC_OK) d->step = step;
+  return st;
 }
 
 void gempic_denoiser_destroy(gempic_denoiser* d) {
@@ -1078,8 +1292,8 @@ void gempic_denoiser_destroy(gempic_denoiser* d) {
   for (auto* a : d->act)
     if (a) cudaFree(a);
   if (d->r) cudaFree(d->r);
+  if (d->part) cudaFree(d->part);
   if (d->loss) cudaFree(d->loss);
-  if (d->err) cudaFree(d->err);
   cudaGetLastError();
   delete d;
 }
