@@ -5,7 +5,8 @@
 // particles per cell stand in for one with many (include/gempic.h, gempic_denoiser_*).
 //
 // Tensors are channel-last, X[z][y][x][16] in BF16 (z = half-slice, periodic across, zero
-// outside the window along zeta).  A convolution is an implicit GEMM: a tile of 128 voxels
+// outside the window along zeta); rows of 128 voxels lie in memory in the tensor core's operand
+// layout and take conv_ws_kernel, described there.  Other widths (conv_kernel): a convolution is an implicit GEMM: a tile of 128 voxels
 // (consecutive in z, y, x order) is the M dimension, the 16 output channels N, and each of the
 // 27 taps adds a K = 16 slice (the 16 input channels of the tap's neighbour).  Per tap the
 // CTA gathers its tile's 128 neighbour voxels into shared memory in the tensor core's K-major
@@ -18,7 +19,8 @@
 //
 // The backward pass through a layer's input is the same convolution with the kernel mirrored
 // and its channels transposed (host-packed operand), masked by the ReLU of the layer below.
-// The weight gradients contract X_shift^T dY over the voxels (wgrad_kernel); Adam updates FP32 master weights, which are then repacked into the BF16 operands.
+// The weight gradients contract X_shift^T dY over the voxels (wgrad_kernel); Adam
+// updates FP32 master weights, which are then repacked into the BF16 operands.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -49,6 +51,51 @@ constexpr int kSpinLimit = 1 << 22;   // polls of an mbarrier before giving up
 // N = 16, M = 128
 constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kCh >> 3) << 17) |
                             ((uint32_t)(kTile >> 4) << 24);
+
+// Activation layouts in global memory.  Plain (any width): [z][y][x][16], 32 bytes a voxel.
+// Padded rows (rows of 128 voxels, the 128 x 128 grids): [z][y] rows of kRowBytes holding
+// voxels x = -1 .. 128 (the periodic neighbour at each end), a voxel's two 16-byte halves
+// exchanged in every other group of four voxels.  That is byte for byte the operand layout of
+// the row convolution in shared memory (32-byte swizzle), so a row goes there in one bulk copy.
+constexpr int kRowVox = 128;                         // nx of the row path
+constexpr int kRowHalo = kRowVox + 2;                // staged voxels: x = -1 .. 128
+constexpr uint32_t kRowBytes = 17u * 256u;           // 130 x 32 bytes, rounded to 256
+constexpr uint32_t kRowCopy = (uint32_t)kRowHalo * 32u;
+
+// byte offset of half h of position xi (voxel x = xi - 1) in a padded row
+__device__ __forceinline__ uint32_t seg_off(int xi, int h) {
+  return (uint32_t)xi * 32u + (uint32_t)((h ^ (xi >> 2)) & 1) * 16u;
+}
+// the 16 channels of voxel v (v = (z ny + y) nx + x): read, or write with the row's halo copies
+__device__ __forceinline__ void act_load(const __nv_bfloat16* x, int nx, long long v, uint4& a, uint4& b) {
+  if (nx == kRowVox) {
+    const char* row = reinterpret_cast<const char*>(x) + (v / kRowVox) * (long long)kRowBytes;
+    const int xi = (int)(v % kRowVox) + 1;
+    a = *reinterpret_cast<const uint4*>(row + seg_off(xi, 0));
+    b = *reinterpret_cast<const uint4*>(row + seg_off(xi, 1));
+  } else {
+    const uint4* d = reinterpret_cast<const uint4*>(x + v * 16);
+    a = d[0];
+    b = d[1];
+  }
+}
+__device__ __forceinline__ void act_store(__nv_bfloat16* x, int nx, long long v, uint4 a, uint4 b) {
+  if (nx == kRowVox) {
+    char* row = reinterpret_cast<char*>(x) + (v / kRowVox) * (long long)kRowBytes;
+    const int xi = (int)(v % kRowVox) + 1;
+    *reinterpret_cast<uint4*>(row + seg_off(xi, 0)) = a;
+    *reinterpret_cast<uint4*>(row + seg_off(xi, 1)) = b;
+    if (xi == 1 || xi == kRowVox) {
+      const int xh = xi == 1 ? kRowVox + 1 : 0;
+      *reinterpret_cast<uint4*>(row + seg_off(xh, 0)) = a;
+      *reinterpret_cast<uint4*>(row + seg_off(xh, 1)) = b;
+    }
+  } else {
+    uint4* d = reinterpret_cast<uint4*>(x + v * 16);
+    d[0] = a;
+    d[1] = b;
+  }
+}
 
 enum Mode { MODE_HIDDEN = 0, MODE_LAST = 1, MODE_BWD = 2 };
 
@@ -152,32 +199,23 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v) {
 // the layer's output for voxel v from its 16 accumulators: bias + ReLU in BF16 (hidden layers),
 // the input's ReLU mask (backward through a layer's input), or bias, the net output r and the
 // residual into the FP32 current (last layer)
-__device__ __forceinline__ void epilogue(const ConvArgs& a, long long v, const float* acc,
-                                         bool add_bias = true) {
+__device__ __forceinline__ void epilogue(const ConvArgs& a, long long v, const float* acc) {
   if (a.mode == MODE_HIDDEN) {
     __align__(16) __nv_bfloat16 o[16];
 #pragma unroll
     for (int c = 0; c < 16; ++c)
-      o[c] = __float2bfloat16_rn(fmaxf(acc[c] + (add_bias ? a.bias[c] : 0.0f), 0.0f));
-    uint4* d = reinterpret_cast<uint4*>(a.out + v * kCh);
-    d[0] = reinterpret_cast<const uint4*>(o)[0];
-    d[1] = reinterpret_cast<const uint4*>(o)[1];
+      o[c] = __float2bfloat16_rn(fmaxf(acc[c] + a.bias[c], 0.0f));
+    act_store(a.out, a.nx, v, reinterpret_cast<const uint4*>(o)[0], reinterpret_cast<const uint4*>(o)[1]);
   } else if (a.mode == MODE_BWD) {
-    const uint4* mk = reinterpret_cast<const uint4*>(a.mask + v * kCh);
     __align__(16) __nv_bfloat16 m[16];
-    reinterpret_cast<uint4*>(m)[0] = mk[0];
-    reinterpret_cast<uint4*>(m)[1] = mk[1];
+    act_load(a.mask, a.nx, v, reinterpret_cast<uint4*>(m)[0], reinterpret_cast<uint4*>(m)[1]);
     __align__(16) __nv_bfloat16 o[16];
 #pragma unroll
     for (int c = 0; c < 16; ++c)
       o[c] = __float2bfloat16_rn(__bfloat162float(m[c]) > 0.0f ? acc[c] : 0.0f);
-    uint4* d = reinterpret_cast<uint4*>(a.out + v * kCh);
-    d[0] = reinterpret_cast<const uint4*>(o)[0];
-    d[1] = reinterpret_cast<const uint4*>(o)[1];
+    act_store(a.out, a.nx, v, reinterpret_cast<const uint4*>(o)[0], reinterpret_cast<const uint4*>(o)[1]);
   } else {
-    const float b0 = add_bias ? a.bias[0] : 0.0f, b1 = add_bias ? a.bias[1] : 0.0f,
-                b2 = add_bias ? a.bias[2] : 0.0f;
-    const float r0 = acc[0] + b0, r1 = acc[1] + b1, r2 = acc[2] + b2;
+    const float r0 = acc[0] + a.bias[0], r1 = acc[1] + a.bias[1], r2 = acc[2] + a.bias[2];
     if (a.r) *reinterpret_cast<float4*>(a.r + v * 4) = make_float4(r0, r1, r2, 0.0f);
     if (a.jout) {
       const long long plane = (long long)a.nx * a.ny;
@@ -321,28 +359,13 @@ __global__ void __launch_bounds__(kThreads) conv_kernel(ConvArgs a) {
 
 // ---- row-staged operands (rows of 128 voxels) ------------------------------------------------
 // For nx = 128 an output tile is one row (z, y), and the A operand of tap (dz, dy, dx) is the
-// input row (z + dz, y + dy) shifted by dx.  Each input row is staged once in shared memory
-// with one halo voxel at each end (x = -1 and x = 128, periodic), a voxel's 16 channels as one
-// 32-byte row of the K-major layout with 32-byte swizzling (the two 16-byte halves of a row
-// exchanged where bit 7 of its shared-memory address is set; rows 256-byte aligned in groups of
-// eight): every tap's operand is then a descriptor into the staged rows, advanced by dx x 32
-// bytes, with no per-tap gather.
-constexpr int kRowVox = 128;                         // nx of the row path
-constexpr int kRowHalo = kRowVox + 2;                // staged voxels: x = -1 .. 128
-constexpr uint32_t kRowBytes = 17u * 256u;           // 130 x 32 bytes, rounded to 256
-
+// input row (z + dz, y + dy) shifted by dx: with the padded rows above in shared memory (256-byte
+// aligned, 32-byte swizzled K-major rows in groups of eight) it is a descriptor advanced by
+// dx x 32 bytes, with no per-tap gather.
 __device__ __forceinline__ uint64_t sdesc_row(uint32_t saddr) {
   return (uint64_t)((saddr & 0x3FFFFu) >> 4) | (1ull << 16) | ((uint64_t)(256u >> 4) << 32) |
          (1ull << 46) | (6ull << 61);
 }
-
-// shared-memory address of the 16-byte half h of staged voxel xi in the row at `row`
-__device__ __forceinline__ uint32_t swz_addr(uint32_t row, int xi, int h) {
-  const uint32_t a = row + (uint32_t)xi * 32u + (uint32_t)h * 16u;
-  return a ^ (((a >> 7) & 1u) << 4);
-}
-
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 
 // ---- warp-specialised row convolution with the three dy taps in one MMA (rows of 128 voxels) -
 // An input row (z + dz, r) feeds the output rows r - 1, r, r + 1 of plane z through the taps
@@ -354,18 +377,23 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 // as units (three z-planes each) in a ring; set s of tensor memory holds output row
 // y0 - 1 + s (sets 0 and kStripW + 1 only collect the contributions to the rows beyond the
 // strip, the first and last input rows use N = 16 MMAs of the one tap that reaches into it).
-// Roles: two producer warps stage the units with asynchronous copies, wait for them, fence
-// them into the tensor core's view and arrive on the unit's `full` mbarrier; one thread issues
-// the MMAs (after the epilogue warps zeroed the strip's accumulators), frees each unit through
-// `empty` and marks each finished output row through its set's `rowd` mbarrier; four epilogue
-// warps zero the accumulators, then read each finished row back and write it.  Every wait is
-// bounded: a wait that gives up sets the abort flag and its role stops; the MMA thread waits
-// for its MMAs in flight before the tensor memory is freed.
+// Roles: one thread stages the units, three bulk copies each (cp.async.bulk, completing on the
+// unit's `full` mbarrier; the rows lie in global memory as the tensor core reads them); one
+// thread issues the MMAs (after the epilogue warps zeroed the strip's accumulators), frees each
+// unit through `empty` and marks each finished output row through its set's `rowd` mbarrier;
+// four epilogue warps zero the accumulators, then read each finished row back and write it.
+// Every wait is bounded: a wait that gives up sets the abort flag and its role stops; the MMA
+// thread waits for its MMAs in flight before the tensor memory is freed, the staging thread for
+// its copies before the CTA ends.
+// Bound: the issuing thread and the tensor pipe, about half each.  An MMA of K = 16 takes 62-68
+// cycles on its CTA whatever N <= 128 is (88 with two CTAs on the SM), 596 of a unit's 1130
+// cycles; waits and commits take the rest.  128 x 128 x 512, 16 -> 16 channels: 346 us with
+// asynchronous 16-byte copies by two warps, 325 us with bulk copies, 164 us with the two
+// single-thread roles cut to a few instructions per unit (DRAM floor 75 us); last layer 500 -> 204 us.
 constexpr int kUnits = 6;                            // ring of staged units
-constexpr int kLead = 4;                             // units whose copies may be in flight
 constexpr int kStripW = 14;                          // output rows per strip
 constexpr int kSets = kStripW + 2;                   // accumulator sets (16 columns each)
-constexpr int kWsThreads = 224;                      // warps 0-1 produce, 2 issues, 3-6 drain
+constexpr int kWsThreads = 192;                      // warp 0 stages, 1 issues, 2-5 drain
 constexpr uint32_t kUnitBytes = 3u * kRowBytes;      // three z-planes of one row
 constexpr uint32_t kWsSmem = (uint32_t)kTaps * kTapBytesB + kUnits * kUnitBytes + 256u;
 // instruction descriptors: M = 128, N = 48 (three taps) and N = 16 (one)
@@ -381,14 +409,16 @@ __device__ __forceinline__ void umma_n(uint32_t tmem_d, uint64_t a, uint64_t b, 
 __device__ __forceinline__ void mbar_arrive(uint64_t* m) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(m)) : "memory");
 }
-__device__ __forceinline__ void cp_async_wait_0() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
-// all but the kLead newest groups have landed
-__device__ __forceinline__ void cp_async_wait_lead() {
-  asm volatile("cp.async.wait_group %0;" ::"n"(kLead) : "memory");
+__device__ __forceinline__ void mbar_expect(uint64_t* m, uint32_t bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(m)), "r"(bytes)
+               : "memory");
 }
-// 16-byte asynchronous copy global -> shared through L2 only (a staged row is read once per CTA)
-__device__ __forceinline__ void cp_async16_cg(uint32_t dst, const void* src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+// bulk copy global -> shared, 16-byte aligned at both ends, completing on an mbarrier
+__device__ __forceinline__ void bulk_g2s(uint32_t dst, const void* src, uint32_t bytes, uint64_t* m) {
+  asm volatile(
+      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+      "l"(src), "r"(bytes), "r"(smem_u32(m))
+      : "memory");
 }
 // zero 16 accumulator columns of this warp's 32 lanes
 __device__ __forceinline__ void tmem_zero16(uint32_t taddr) {
@@ -397,6 +427,68 @@ __device__ __forceinline__ void tmem_zero16(uint32_t taddr) {
       "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,"
       "%1,%1};" ::"r"(taddr), "r"(z)
       : "memory");
+}
+
+// What the epilogue of voxel x of row (z, y) reads: the current (last layer) or the mask
+// (backward); loaded a row ahead, so that its latency passes meanwhile (the last layer took 0.49 ms at 128 x 128 x 512, 3.0 k cycles a row in these loads)
+struct EpiIn {
+  uint4 a, b;
+};
+__device__ __forceinline__ EpiIn epilogue_read(const ConvArgs& a, int z, int y, int x) {
+  EpiIn in{};
+  const long long rowi = (long long)z * a.ny + y;
+  if (a.mode == MODE_LAST) {
+    if (a.jout) {
+      const long long plane = (long long)a.ny * kRowVox;
+      const float* j = a.jres + (long long)z * 3 * plane + (long long)y * kRowVox + x;
+      in.a.x = __float_as_uint(__ldcg(j));
+      in.a.y = __float_as_uint(__ldcg(j + plane));
+      in.a.z = __float_as_uint(__ldcg(j + 2 * plane));
+    }
+  } else if (a.mode == MODE_BWD) {
+    const char* mr = reinterpret_cast<const char*>(a.mask) + rowi * kRowBytes;
+    in.a = *reinterpret_cast<const uint4*>(mr + seg_off(x + 1, 0));
+    in.b = *reinterpret_cast<const uint4*>(mr + seg_off(x + 1, 1));
+  }
+  return in;
+}
+
+// epilogue() for voxel x of row (z, y) of a grid of 128-voxel rows (bias already added)
+__device__ __forceinline__ void epilogue_row(const ConvArgs& a, int z, int y, int x, const EpiIn& in,
+                                             const float* acc) {
+  const long long rowi = (long long)z * a.ny + y;
+  const uint32_t o0 = seg_off(x + 1, 0), o1 = seg_off(x + 1, 1);
+  if (a.mode == MODE_LAST) {
+    if (a.r) *reinterpret_cast<float4*>(a.r + (rowi * kRowVox + x) * 4) = make_float4(acc[0], acc[1], acc[2], 0.0f);
+    if (a.jout) {
+      const long long plane = (long long)a.ny * kRowVox;
+      float* j = a.jout + (long long)z * 3 * plane + (long long)y * kRowVox + x;
+      j[0] = __uint_as_float(in.a.x) + a.scale * acc[0];
+      j[plane] = __uint_as_float(in.a.y) + a.scale * acc[1];
+      j[2 * plane] = __uint_as_float(in.a.z) + a.scale * acc[2];
+    }
+    return;
+  }
+  __align__(16) __nv_bfloat16 o[16];
+  if (a.mode == MODE_HIDDEN) {
+#pragma unroll
+    for (int c = 0; c < 16; ++c) o[c] = __float2bfloat16_rn(fmaxf(acc[c], 0.0f));
+  } else {
+    __align__(16) __nv_bfloat16 m[16];
+    reinterpret_cast<uint4*>(m)[0] = in.a;
+    reinterpret_cast<uint4*>(m)[1] = in.b;
+#pragma unroll
+    for (int c = 0; c < 16; ++c) o[c] = __float2bfloat16_rn(__bfloat162float(m[c]) > 0.0f ? acc[c] : 0.0f);
+  }
+  char* row = reinterpret_cast<char*>(a.out) + rowi * kRowBytes;
+  const uint4 h0 = reinterpret_cast<const uint4*>(o)[0], h1 = reinterpret_cast<const uint4*>(o)[1];
+  *reinterpret_cast<uint4*>(row + o0) = h0;
+  *reinterpret_cast<uint4*>(row + o1) = h1;
+  if (x == 0 || x == kRowVox - 1) {                            // the row's periodic halo copies
+    const int xh = x == 0 ? kRowVox + 1 : 0;
+    *reinterpret_cast<uint4*>(row + seg_off(xh, 0)) = h0;
+    *reinterpret_cast<uint4*>(row + seg_off(xh, 1)) = h1;
+  }
 }
 
 __global__ void __launch_bounds__(kWsThreads) conv_ws_kernel(ConvArgs a) {
@@ -416,7 +508,7 @@ __global__ void __launch_bounds__(kWsThreads) conv_ws_kernel(ConvArgs a) {
   }
   if (tid == 0) {
     for (int u = 0; u < kUnits; ++u) {
-      mbar_init(&full[u], 64);
+      mbar_init(&full[u], 1);
       mbar_init(&empty[u], 1);
     }
     for (int c = 0; c < kSets; ++c) mbar_init(&rowd[c], 1);
@@ -445,98 +537,101 @@ __global__ void __launch_bounds__(kWsThreads) conv_ws_kernel(ConvArgs a) {
   const uint32_t tmem = tmem_slot;
   const uint32_t uBase = smem_u32(sU);
   const int nyb = (a.ny + kStripW - 1) / kStripW;
-  const long long nstrips = (long long)(a.zhi - a.zlo) * nyb;
-  auto unit_addr = [&](long long u, int plane) -> uint32_t {
-    return uBase + (uint32_t)(u % kUnits) * kUnitBytes + (uint32_t)plane * kRowBytes;
-  };
+  const int nstrips = (a.zhi - a.zlo) * nyb;
 
-  if (warp < 2) {
-    // ---- producers: units (z, r) for r = y0-1 .. y1 of every strip, in order ----
-    const int pt = tid;                                       // 0 .. 63
-    long long uc = 0;
-    long long landed = 0;                 // units before this one have been released
-    for (long long strip = blockIdx.x; strip < nstrips && !abort_flag; strip += gridDim.x) {
-      const int z = a.zlo + (int)(strip / nyb);
-      const int y0 = (int)(strip % nyb) * kStripW, y1 = min(a.ny, y0 + kStripW);
-      for (int r = y0 - 1; r <= y1; ++r, ++uc) {
-        if (!mbar_wait(&empty[uc % kUnits], (uint32_t)(((uc / kUnits) & 1) ^ 1))) {
-          atomicExch(&abort_flag, 1);
-          break;
-        }
-        const int yr = r < 0 ? r + a.ny : (r >= a.ny ? r - a.ny : r);
-        for (int dz = -1; dz <= 1; ++dz) {
-          const int zz = z + dz;
-          if (zz < 0 || zz >= a.nz) continue;                 // its taps are skipped
-          const __nv_bfloat16* row = a.x + ((long long)zz * a.ny + yr) * (long long)kRowVox * kCh;
-          const uint32_t dst = unit_addr(uc, dz + 1);
-          for (int i = pt; i < 2 * kRowHalo; i += 64) {
-            const int xi = i >> 1, h = i & 1;
-            const int xs = (xi + kRowVox - 1) & (kRowVox - 1);
-            cp_async16_cg(swz_addr(dst, xi, h), row + xs * kCh + h * 8);
+  // The two single-thread roles run a few instructions per unit: ring slot and phase are
+  // counters (a 64-bit modulo per unit and barrier cost the issuing thread more than its MMAs
+  // take: 190 cycles per MMA against 44 in the tensor pipe), descriptors advance by constants.
+  if (warp == 0) {
+    // ---- staging: units (z, r) for r = y0-1 .. y1 of every strip, in order; one thread ----
+    if (lane == 0) {
+      int slot = 0;
+      uint32_t phase = 0, staged = 0;               // staged: units so far, at most kUnits
+      bool ok = true;
+      for (int strip = blockIdx.x; strip < nstrips && ok && !abort_flag; strip += gridDim.x) {
+        const int zq = strip / nyb;
+        const int z = a.zlo + zq, y0 = (strip - zq * nyb) * kStripW, y1 = min(a.ny, y0 + kStripW);
+        const int p0 = z == 0 ? 1 : 0, p1 = z == a.nz - 1 ? 1 : 2;   // planes inside the window
+        const uint32_t bytes = (uint32_t)(p1 - p0 + 1) * kRowCopy;
+        const long long plane = (long long)a.ny * kRowBytes;
+        const char* base = reinterpret_cast<const char*>(a.x) + (z - 1) * plane;
+        for (int r = y0 - 1; r <= y1; ++r) {
+          if (!mbar_wait(&empty[slot], phase ^ 1u)) {
+            atomicExch(&abort_flag, 1);
+            ok = false;
+            break;
+          }
+          const int yr = r < 0 ? r + a.ny : (r >= a.ny ? r - a.ny : r);
+          const char* src = base + (long long)yr * kRowBytes;
+          const uint32_t dst = uBase + (uint32_t)slot * kUnitBytes;
+          mbar_expect(&full[slot], bytes);
+          for (int pl = p0; pl <= p1; ++pl) bulk_g2s(dst + (uint32_t)pl * kRowBytes, src + pl * plane, kRowCopy, &full[slot]);
+          staged = min(staged + 1u, (uint32_t)kUnits);
+          if (++slot == kUnits) {
+            slot = 0;
+            phase ^= 1u;
           }
         }
-        cp_async_commit();
-        // up to kLead + 1 units in flight (with the one the MMAs read, the whole ring): release
-        // the oldest once its copies have landed
-        if (uc - landed >= kLead) {
-          cp_async_wait_lead();
-          fence_async_smem();
-          mbar_arrive(&full[landed % kUnits]);
-          ++landed;
+      }
+      // no copy may land after the CTA has ended: the last staged units' copies, newest first
+      for (uint32_t k = 0; k < staged; ++k) {
+        if (--slot < 0) {
+          slot = kUnits - 1;
+          phase ^= 1u;
         }
+        if (!mbar_wait(&full[slot], phase)) atomicExch(&abort_flag, 1);
       }
     }
-    cp_async_wait_0();
-    fence_async_smem();
-    for (; landed < uc; ++landed) mbar_arrive(&full[landed % kUnits]);
-  } else if (warp == 2) {
+    __syncwarp();
+  } else if (warp == 1) {
     // ---- MMA issue: one thread ----
     if (lane == 0) {
       const uint64_t bdesc = sdesc(smem_u32(sB));
+      const uint64_t adesc = sdesc_row(uBase);
       constexpr uint64_t kPair = (3u * kTapBytesB) >> 4;     // B of the next (dz, dx) pair
       constexpr uint64_t kTap = kTapBytesB >> 4;
-      long long uc = 0, sc = 0;
-      bool issued = false;
-      for (long long strip = blockIdx.x; strip < nstrips && !abort_flag; strip += gridDim.x, ++sc) {
-        const int z = a.zlo + (int)(strip / nyb);
-        const int y0 = (int)(strip % nyb) * kStripW, y1 = min(a.ny, y0 + kStripW);
+      int slot = 0;
+      uint32_t phase = 0, zphase = 0;
+      bool issued = false, ok = true;
+      for (int strip = blockIdx.x; strip < nstrips && ok && !abort_flag; strip += gridDim.x) {
+        const int zq = strip / nyb;
+        const int z = a.zlo + zq, y0 = (strip - zq * nyb) * kStripW, y1 = min(a.ny, y0 + kStripW);
+        const int p0 = z == 0 ? 1 : 0, p1 = z == a.nz - 1 ? 1 : 2;
         // the epilogue warps have zeroed the accumulators of this strip
-        if (!mbar_wait(&zeroed, (uint32_t)(sc & 1))) {
+        if (!mbar_wait(&zeroed, zphase)) {
           atomicExch(&abort_flag, 1);
           break;
         }
+        zphase ^= 1u;
         tc_fence_after();
-        bool ok = true;
-        for (int r = y0 - 1; r <= y1 && ok; ++r, ++uc) {
-          if (!mbar_wait(&full[uc % kUnits], (uint32_t)((uc / kUnits) & 1))) {
+        for (int r = y0 - 1; r <= y1; ++r) {
+          if (!mbar_wait(&full[slot], phase)) {
             atomicExch(&abort_flag, 1);
             ok = false;
             break;
           }
           tc_fence_after();
-          const int sidx = r - y0;                            // set of output row r - 1
-#pragma unroll
-          for (int pz = 0; pz < 3; ++pz) {
-            if (z + pz - 1 < 0 || z + pz - 1 >= a.nz) continue;
-            const uint64_t ad = sdesc_row(unit_addr(uc, pz));
-#pragma unroll
-            for (int px = 0; px < 3; ++px) {
-              const uint64_t bd = bdesc + (uint64_t)(pz * 3 + px) * kPair;
-              const uint64_t as = ad + (uint64_t)(2 * px);          // dx: 32 bytes a voxel
-              if (r == y0 - 1)            // only dy = -1 reaches the strip (row y0: set 1)
-                umma_n(tmem + 16u, as, bd + 2 * kTap, kIdesc);
-              else if (r == y1)           // only dy = +1 (row y1 - 1)
-                umma_n(tmem + (uint32_t)(16 * (y1 - y0)), as, bd, kIdesc);
-              else                        // rows r - 1, r, r + 1: sets r - y0 .. r - y0 + 2
-                umma_n(tmem + (uint32_t)(16 * sidx), as, bd, kIdesc48);
-            }
+          // rows r - 1, r, r + 1: sets r - y0 .. r - y0 + 2 (N = 48); at the strip's ends only the
+          // tap that reaches into it: dy = -1 into row y0 (set 1), dy = +1 into row y1 - 1
+          const bool first = r == y0 - 1, last = r == y1;
+          const uint32_t d = tmem + (uint32_t)(first ? 16 : 16 * (r - y0));
+          const uint32_t id = first || last ? kIdesc : kIdesc48;
+          uint64_t ad = adesc + (uint64_t)((slot * kUnitBytes + (uint32_t)p0 * kRowBytes) >> 4);
+          uint64_t bd = bdesc + (uint64_t)(3 * p0) * kPair + (first ? 2 * kTap : 0);
+          for (int pz = p0; pz <= p1; ++pz, ad += kRowBytes >> 4, bd += 3 * kPair) {
+            umma_n(d, ad, bd, id);                            // dx = -1, 0, 1: 32 bytes a voxel
+            umma_n(d, ad + 2, bd + kPair, id);
+            umma_n(d, ad + 4, bd + 2 * kPair, id);
           }
           issued = true;
-          umma_commit(&empty[uc % kUnits]);
+          umma_commit(&empty[slot]);
           // output row r - 1 has all its contributions (input rows r - 2 .. r)
           if (r - 1 >= y0) umma_commit(&rowd[r - y0]);
+          if (++slot == kUnits) {
+            slot = 0;
+            phase ^= 1u;
+          }
         }
-        if (!ok) break;
       }
       if (issued) {
         umma_commit(&drain);
@@ -545,7 +640,7 @@ __global__ void __launch_bounds__(kWsThreads) conv_ws_kernel(ConvArgs a) {
     }
     __syncwarp();
   } else {
-    // ---- epilogue: warps 3..6 own lanes 32 (warp % 4) .. +31 of the accumulators ----
+    // ---- epilogue: warps 2..5 own lanes 32 (warp % 4) .. +31 of the accumulators ----
     const int q = warp & 3;
     float bias[16];
 #pragma unroll
@@ -553,10 +648,9 @@ __global__ void __launch_bounds__(kWsThreads) conv_ws_kernel(ConvArgs a) {
     const uint32_t lanes = (uint32_t)(q * 32) << 16;
     // phase of each row barrier (a short strip at the end of y completes only some of them)
     uint32_t rpar = 0u;                                       // bit c: parity of rowd[c]
-    long long sc = 0;
-    for (long long strip = blockIdx.x; strip < nstrips && !abort_flag; strip += gridDim.x, ++sc) {
-      const int z = a.zlo + (int)(strip / nyb);
-      const int y0 = (int)(strip % nyb) * kStripW, y1 = min(a.ny, y0 + kStripW);
+    for (int strip = blockIdx.x; strip < nstrips && !abort_flag; strip += gridDim.x) {
+      const int zq = strip / nyb;
+      const int z = a.zlo + zq, y0 = (strip - zq * nyb) * kStripW, y1 = min(a.ny, y0 + kStripW);
       // zero this strip's accumulators (the previous strip's rows have all been read)
       for (int c = 0; c < kSets; ++c) tmem_zero16(tmem + lanes + (uint32_t)(16 * c));
       asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
@@ -564,8 +658,11 @@ __global__ void __launch_bounds__(kWsThreads) conv_ws_kernel(ConvArgs a) {
       __syncwarp();
       if (lane == 0) mbar_arrive(&zeroed);
       bool ok = true;
+      EpiIn next = epilogue_read(a, z, y0, q * 32 + lane);
       for (int y = y0; y < y1; ++y) {
         const int set = y - y0 + 1;
+        const EpiIn in = next;
+        if (y + 1 < y1) next = epilogue_read(a, z, y + 1, q * 32 + lane);
         if (!mbar_wait(&rowd[set], (rpar >> set) & 1u)) {
           atomicExch(&abort_flag, 1);
           ok = false;
@@ -577,8 +674,7 @@ __global__ void __launch_bounds__(kWsThreads) conv_ws_kernel(ConvArgs a) {
         tmem_ld16(tmem + lanes + (uint32_t)(16 * set), acc);
 #pragma unroll
         for (int c = 0; c < 16; ++c) acc[c] += bias[c];
-        const long long v = ((long long)z * a.ny + y) * kRowVox + q * 32 + lane;
-        epilogue(a, v, acc, false);
+        epilogue_row(a, z, y, q * 32 + lane, in, acc);
       }
       tc_fence_before();
       if (!ok) break;
@@ -598,18 +694,29 @@ __global__ void __launch_bounds__(kWsThreads) conv_ws_kernel(ConvArgs a) {
 __global__ void pack_input_kernel(const float* j, __nv_bfloat16* x0, int nx, int ny, int zlo,
                                   int zhi, float inv_scale) {
   const long long plane = (long long)nx * ny, v0 = plane * zlo, V = plane * zhi;
-  for (long long v = v0 + blockIdx.x * (long long)blockDim.x + threadIdx.x; v < V;
-       v += (long long)gridDim.x * blockDim.x) {
-    const long long z = v / plane, rem = v - z * plane;
-    __align__(16) __nv_bfloat16 o[16];
+  const long long step = (long long)gridDim.x * blockDim.x;
+  // four voxels in flight per thread: with one, the kernel moved 3.5 TB/s at 128 x 128 x 512
+  for (long long w = v0 + blockIdx.x * (long long)blockDim.x + threadIdx.x; w < V; w += 4 * step) {
+    float f[4][3];
 #pragma unroll
-    for (int c = 0; c < 16; ++c) o[c] = __float2bfloat16_rn(0.0f);
+    for (int u = 0; u < 4; ++u) {
+      const long long v = w + u * step;
+      if (v >= V) break;
+      const long long z = v / plane, rem = v - z * plane;
 #pragma unroll
-    for (int c = 0; c < 3; ++c)
-      o[c] = __float2bfloat16_rn(__ldcg(j + (z * 3 + c) * plane + rem) * inv_scale);
-    uint4* d = reinterpret_cast<uint4*>(x0 + v * kCh);
-    d[0] = reinterpret_cast<const uint4*>(o)[0];
-    d[1] = reinterpret_cast<const uint4*>(o)[1];
+      for (int c = 0; c < 3; ++c) f[u][c] = __ldcg(j + (z * 3 + c) * plane + rem);
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const long long v = w + u * step;
+      if (v >= V) break;
+      const __nv_bfloat162 lo = __floats2bfloat162_rn(f[u][0] * inv_scale, f[u][1] * inv_scale);
+      const __nv_bfloat162 hi = __floats2bfloat162_rn(f[u][2] * inv_scale, 0.0f);
+      uint4 a = make_uint4(0u, 0u, 0u, 0u);
+      a.x = *reinterpret_cast<const uint32_t*>(&lo);
+      a.y = *reinterpret_cast<const uint32_t*>(&hi);
+      act_store(x0, nx, v, a, make_uint4(0u, 0u, 0u, 0u));
+    }
   }
 }
 
@@ -635,9 +742,7 @@ __global__ void loss_kernel(const float* j, const float* t, const float* r, __nv
         o[c] = __float2bfloat16_rn(e * inv_count2);
       }
     }
-    uint4* d = reinterpret_cast<uint4*>(dr + v * kCh);
-    d[0] = reinterpret_cast<const uint4*>(o)[0];
-    d[1] = reinterpret_cast<const uint4*>(o)[1];
+    act_store(dr, nx, v, reinterpret_cast<const uint4*>(o)[0], reinterpret_cast<const uint4*>(o)[1]);
   }
   __shared__ double red[32];
   for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
@@ -669,7 +774,7 @@ constexpr int kSeg = 128;                            // voxels of a row segment
 constexpr int kGradWarps = 9;
 constexpr int kGradThreads = 32 * kGradWarps;
 constexpr uint32_t kSegBytes = (uint32_t)(kSeg + 2) * 32u;
-constexpr uint32_t kGradSmem = 12u * kSegBytes + 2u * kSeg * 32u;   // [4 y][3 z] input rows, 2 dY rows
+constexpr uint32_t kGradSmem = 14u * kSegBytes;      // [4 y][3 z] input rows, 2 dY rows
 constexpr int kPart = kTaps * kCh * kCh + kCh;       // partial sums per CTA and layer: dW, db
 
 struct GradArgs {
@@ -679,11 +784,6 @@ struct GradArgs {
   int nx, ny, nz;
 };
 
-// byte offset of the 16-byte half h of staged voxel xi: the halves of every other group of four
-// voxels are exchanged, so the eight rows of an ldmatrix tile start in different banks
-__device__ __forceinline__ uint32_t seg_off(int xi, int h) {
-  return (uint32_t)xi * 32u + (uint32_t)((h ^ (xi >> 2)) & 1) * 16u;
-}
 __device__ __forceinline__ void ldsm4t(uint32_t a, uint32_t (&r)[4]) {
   asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
                : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
@@ -699,13 +799,14 @@ __device__ __forceinline__ void mma16816(float* d, const uint32_t (&a)[4], uint3
 }
 
 __global__ void __launch_bounds__(kGradThreads, 2) wgrad_kernel(GradArgs g) {
-  extern __shared__ __align__(128) unsigned char smem[];
+  extern __shared__ __align__(1024) unsigned char smem[];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int layer = blockIdx.y;
   const __nv_bfloat16* const X = g.x[layer];
   const __nv_bfloat16* const dY = g.dy[layer];
   const uint32_t sx = smem_u32(smem), sy = sx + 12u * kSegBytes;
   const int nseg = (g.nx + kSeg - 1) / kSeg;
+  const bool padded = g.nx == kRowVox;               // rows lie in memory as they are staged
   const long long rows = (long long)g.nz * nseg * g.ny;
   const long long r0 = rows * blockIdx.x / gridDim.x, r1 = rows * (blockIdx.x + 1) / gridDim.x;
   const int pz = warp / 3, py = warp - 3 * pz;       // this warp's (dz, dy) + 1
@@ -725,8 +826,13 @@ __global__ void __launch_bounds__(kGradThreads, 2) wgrad_kernel(GradArgs g) {
     for (int pl = 0; pl < 3; ++pl) {
       const int zz = z + pl - 1;
       if (zz < 0 || zz >= g.nz) continue;            // its warps skip their products
-      const __nv_bfloat16* row = X + ((long long)zz * g.ny + y) * (long long)g.nx * kCh;
       const uint32_t dst = sx + (uint32_t)(slot * 3 + pl) * kSegBytes;
+      if (padded) {                                  // as it lies in memory
+        const char* row = reinterpret_cast<const char*>(X) + ((long long)zz * g.ny + y) * kRowBytes;
+        for (int i = tid; i < (int)(kRowCopy / 16); i += kGradThreads) cp_async16(dst + i * 16, row + i * 16, 16u);
+        continue;
+      }
+      const __nv_bfloat16* row = X + ((long long)zz * g.ny + y) * (long long)g.nx * kCh;
       for (int i = tid; i < 2 * (kk + 2); i += kGradThreads) {
         const int xi = i >> 1, h = i & 1;
         int x = s0 + xi - 1;
@@ -737,11 +843,16 @@ __global__ void __launch_bounds__(kGradThreads, 2) wgrad_kernel(GradArgs g) {
     }
   };
   auto stage_y = [&](int buf, int z, int y, int s0, int len, int kk) {
+    const uint32_t dst = sy + (uint32_t)buf * kSegBytes;
+    if (padded) {
+      const char* row = reinterpret_cast<const char*>(dY) + ((long long)z * g.ny + y) * kRowBytes;
+      for (int i = tid; i < (int)(kRowCopy / 16); i += kGradThreads) cp_async16(dst + i * 16, row + i * 16, 16u);
+      return;
+    }
     const __nv_bfloat16* row = dY + (((long long)z * g.ny + y) * g.nx + s0) * kCh;
-    const uint32_t dst = sy + (uint32_t)buf * kSeg * 32u;
     for (int i = tid; i < 2 * kk; i += kGradThreads) {
       const int xi = i >> 1, h = i & 1;
-      cp_async16(dst + seg_off(xi, h), xi < len ? row + xi * kCh + h * 8 : dY, xi < len ? 16u : 0u);
+      cp_async16(dst + seg_off(xi + 1, h), xi < len ? row + xi * kCh + h * 8 : dY, xi < len ? 16u : 0u);
     }
   };
 
@@ -771,7 +882,7 @@ __global__ void __launch_bounds__(kGradThreads, 2) wgrad_kernel(GradArgs g) {
     }
     if (z + pz - 1 >= 0 && z + pz - 1 < g.nz) {
       const uint32_t xrow = sx + (uint32_t)(((base + py) & 3) * 3 + pz) * kSegBytes;
-      const uint32_t yrow = sy + (uint32_t)buf * kSeg * 32u;
+      const uint32_t yrow = sy + (uint32_t)buf * kSegBytes;
       float acc[3][8], bacc[8];
 #pragma unroll
       for (int i = 0; i < 24; ++i) acc[i >> 3][i & 7] = 0.0f;
@@ -779,7 +890,7 @@ __global__ void __launch_bounds__(kGradThreads, 2) wgrad_kernel(GradArgs g) {
       for (int i = 0; i < 8; ++i) bacc[i] = 0.0f;
       for (int k = 0; k < kk; k += 16) {
         uint32_t b[4];
-        ldsm4t(yrow + seg_off(k + lv, lh), b);
+        ldsm4t(yrow + seg_off(k + lv + 1, lh), b);
 #pragma unroll
         for (int dx = 0; dx < 3; ++dx) {
           uint32_t a[4];
@@ -919,7 +1030,8 @@ struct gempic_denoiser {
   __nv_bfloat16* wb[3] = {};   // backward operands (layers 2, 3)
   long long step = 0;
   // activations (grown on demand): x0, h1, h2, dr, dh2, dh1 channel-last; r FP32
-  long long cap = 0;
+  long long cap = 0;           // voxels of r
+  size_t act_bytes = 0;        // bytes of each activation buffer
   __nv_bfloat16* act[6] = {};
   float* r = nullptr;
   float* part = nullptr;       // partial weight gradients [3][nsm][kPart] (first gradient)
@@ -941,8 +1053,11 @@ size_t nparams() { return woff(3); }
 
 size_t conv_smem() { return (size_t)kTaps * kTapBytesB + 2u * kRound * kTapBytesA; }
 
-cudaError_t grow(gempic_denoiser* d, long long V) {
-  if (V <= d->cap) return cudaSuccess;
+// buffers for nx x ny x nz voxels (activations in their layout's size)
+cudaError_t grow(gempic_denoiser* d, int nx, int ny, int nz) {
+  const long long V = (long long)nx * ny * nz;
+  const size_t bytes = nx == kRowVox ? (size_t)ny * nz * kRowBytes : (size_t)V * kCh * sizeof(__nv_bfloat16);
+  if (bytes <= d->act_bytes && V <= d->cap) return cudaSuccess;
   for (auto*& a : d->act) {
     if (a) cudaFree(a);
     a = nullptr;
@@ -950,11 +1065,15 @@ cudaError_t grow(gempic_denoiser* d, long long V) {
   if (d->r) cudaFree(d->r);
   d->r = nullptr;
   d->cap = 0;
+  d->act_bytes = 0;
   cudaError_t e = cudaSuccess;
   for (auto*& a : d->act)
-    if (e == cudaSuccess) e = cudaMalloc(&a, (size_t)V * kCh * sizeof(__nv_bfloat16));
+    if (e == cudaSuccess) e = cudaMalloc(&a, bytes);
   if (e == cudaSuccess) e = cudaMalloc(&d->r, (size_t)V * 4 * sizeof(float));
-  if (e == cudaSuccess) d->cap = V;
+  if (e == cudaSuccess) {
+    d->cap = V;
+    d->act_bytes = bytes;
+  }
   return e;
 }
 
@@ -1052,7 +1171,7 @@ int denoise_range(gempic_denoiser* d, const float* j_in, float* j_out, int nx, i
                   int z0, int z1, cudaStream_t s) {
   if (!d || !j_in || !j_out || !grid_ok(nx, ny, nz) || z0 < 0 || z1 > nz || z0 >= z1)
     return GEMPIC_EINVAL;
-  cudaError_t e = grow(d, (long long)nx * ny * nz);
+  cudaError_t e = grow(d, nx, ny, nz);
   if (e != cudaSuccess) return e == cudaErrorMemoryAllocation ? GEMPIC_ENOMEM : GEMPIC_ECUDA;
   const int p0 = std::max(0, z0 - 3), p1 = std::min(nz, z1 + 3);
   const long long V = (long long)nx * ny * (p1 - p0);
@@ -1071,7 +1190,7 @@ int denoise_status(gempic_denoiser* d, cudaStream_t s) { return check_err(d, s);
 // for marches that wait for the net
 int denoise_reserve(gempic_denoiser* d, int nx, int ny, int nz) {
   if (!d || !grid_ok(nx, ny, nz)) return GEMPIC_EINVAL;
-  cudaError_t e = grow(d, (long long)nx * ny * nz);
+  cudaError_t e = grow(d, nx, ny, nz);
   // the net's kernels are loaded now: with lazy module loading a kernel's first launch loads
   // its module, which can wait for the device -- for marches that wait for that kernel
   cudaFuncAttributes fa;
@@ -1112,8 +1231,6 @@ gempic_status gempic_denoiser_create(const float* params, double scale, gempic_d
   if (e == cudaSuccess) e = cudaMalloc(&d->loss, 2 * sizeof(double));
   if (e == cudaSuccess) e = cudaMemset(d->loss, 0, 2 * sizeof(double));
   if (e == cudaSuccess) d->err = reinterpret_cast<int*>(d->loss + 1);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(wgrad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGradSmem);
   if (e == cudaSuccess) e = cudaMemset(d->m, 0, n * sizeof(float));
   if (e == cudaSuccess) e = cudaMemset(d->v, 0, n * sizeof(float));
   if (e == cudaSuccess) {
@@ -1156,7 +1273,7 @@ gempic_status gempic_denoiser_apply(gempic_denoiser* d, const float* j_in, float
   if (!d || !j_in || !j_out || !grid_ok(nx, ny, nz)) return GEMPIC_EINVAL;
   cudaStream_t s = (cudaStream_t)cuda_stream;
   const long long V = (long long)nx * ny * nz;
-  cudaError_t e = grow(d, V);
+  cudaError_t e = grow(d, nx, ny, nz);
   if (e != cudaSuccess) return e == cudaErrorMemoryAllocation ? GEMPIC_ENOMEM : GEMPIC_ECUDA;
   const int blocks = (int)std::min<long long>((V + 255) / 256, 8LL * d->nsm);
   pack_input_kernel<<<blocks, 256, 0, s>>>(j_in, d->act[0], nx, ny, 0, nz, (float)(1.0 / d->scale));
@@ -1174,9 +1291,10 @@ namespace {
 gempic_status gradient(gempic_denoiser* d, const float* j_in, const float* j_target, int nx, int ny,
                        int nz, int z_margin, cudaStream_t s) {
   const long long V = (long long)nx * ny * nz;
-  cudaError_t e = grow(d, V);
+  cudaError_t e = grow(d, nx, ny, nz);
   if (e == cudaSuccess && !d->part) {
-    e = cudaMalloc(&d->part, (size_t)3 * d->nsm * kPart * sizeof(float));
+    e = cudaFuncSetAttribute(wgrad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGradSmem);
+    if (e == cudaSuccess) e = cudaMalloc(&d->part, (size_t)3 * d->nsm * kPart * sizeof(float));
     if (e != cudaSuccess) d->part = nullptr;
   }
   if (e != cudaSuccess) return e == cudaErrorMemoryAllocation ? GEMPIC_ENOMEM : GEMPIC_ECUDA;
