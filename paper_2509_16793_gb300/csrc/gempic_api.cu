@@ -34,6 +34,11 @@ struct gempic_sim {
   Params p{};                      // launch template
   int eb = 8;                      // bytes per real
   int pmax = 1;                    // concurrent marches
+  // 2-D: launch shapes with the particles of a march on 1, 2, 4, 8 CTAs (shape 0 is p's; a shape
+  // that does not apply has maxcl 0); empty: only p's
+  struct Shape { Params p; int maxcl; };
+  std::vector<Shape> shapes;
+  int nrank_last = 1;              // CTAs per march of the last launch (diagnostic partials)
   cudaStream_t stream = nullptr;
   long long k = 0;                 // s-steps completed
   bool initialized = false;
@@ -73,6 +78,8 @@ struct gempic_sim {
 };
 
 namespace {
+
+constexpr int kMaxSplit = 8;       // CTAs that share the particles of a 2-D march at most
 
 bool pow2(int v) { return v > 0 && (v & (v - 1)) == 0; }
 int ilog2(int v) {
@@ -122,7 +129,7 @@ gempic_status check_device_error(gempic_sim* s) {
 cudaError_t ensure_diag_cap(gempic_sim* s, int n) {
   if (n <= s->diag_cap) return cudaSuccess;
   double *d = nullptr, *o = nullptr, *r = nullptr, *gr = nullptr;
-  cudaError_t e = dalloc(s, &d, (size_t)n * gempic::kNDiag * s->p.C * sizeof(double));
+  cudaError_t e = dalloc(s, &d, (size_t)n * gempic::kNDiag * (s->shapes.empty() ? s->p.C : kMaxSplit) * sizeof(double));
   if (e != cudaSuccess) return e;
   e = dalloc(s, &o, (size_t)n * s->p.nz * sizeof(double));
   if (e != cudaSuccess) return e;
@@ -243,6 +250,7 @@ gempic_status ensure_initialized(gempic_sim* s) {
   q.snapshot = 0;
   e = gempic::launch_march(prec, q, s->stream);
   s->launches++;
+  s->nrank_last = s->p.C;
   if (e != cudaSuccess) return cuda_fail(s, e);
   st = check_device_error(s);
   if (st != GEMPIC_OK) return st;
@@ -298,6 +306,7 @@ void batch_advance(gempic_sim* s, int n) {
   s->k += n;
   s->launches++;
   s->denoised_last = false;
+  s->nrank_last = s->p.C;
 }
 
 int batch_precision(const gempic_sim* s) { return s->cfg.precision; }
@@ -321,7 +330,73 @@ const char* gempic_strerror(gempic_status s) {
   return "unknown status";
 }
 
-gempic_status gempic_create(const gempic_config* cfg, gempic_sim** out) {
+}  // extern "C"
+
+namespace {
+
+// threads per CTA: one spectral mode per thread at least, and one fresh particle per thread up
+// to 512 (FP64: 256, the size of the kernel that keeps its state in registers).  With four
+// particles per thread a small slice ran on 4 warps: 95 k cycles a slice at 16 x 16 (FP32, 2 per
+// cell, with one-warp transforms) where 16 warps are free.
+int pick_threads(int precision, int M, int fresh) {
+  const int most = precision == 64 ? 256 : 512;
+  return std::min(512, std::max(std::max(M, 128), (std::min(most, fresh) + 31) / 32 * 32));
+}
+
+// cycles of one slice of a 2-D march on S CTAs, from the phase timers: the push (FP64 bound by
+// the SM's two lanes, FP32 by issue) divides, transforms and solve do not, and the summation
+// over the CTAs adds two cluster barriers and S reads per current
+double slice_cycles_2d(const Params& p, int eb, int S) {
+  const double np = (double)p.nx * p.ppc_sum / S;
+  const double push = eb == 8 ? 260.0 * np + 4000.0 : 8.0 * np + 3000.0;
+  const double fixed = eb == 8 ? 10000.0 + 160.0 * p.nx : 12000.0 + 16.0 * p.nx;
+  return push + fixed + (S > 1 ? 2500.0 + 2.0 * S * p.nx * 3 / p.nthreads * 8.0 : 0.0);
+}
+
+// The launch of n s-steps: parameters with the shape and the number of marches in flight.  2-D
+// grids choose how many CTAs share a march by the modelled time of the wavefront: march c starts
+// when march c - 1 is a few slices ahead (kLag) and march c - P has finished.  Many s-steps fill
+// the chip with marches of one CTA; few s-steps (or one) leave SMs to share a march's particles.
+Params plan_launch(const gempic_sim* s, int n) {
+  constexpr double kLag = 4.0;
+  const Params* best = &s->p;
+  int bestP = std::min(s->pmax, n);
+  double best_t = -1.0;
+  for (const gempic_sim::Shape& c : s->shapes) {
+    const int P = std::min(std::min(s->pmax, n), c.maxcl);
+    if (P < 1) continue;
+    std::vector<double> end((size_t)P, 0.0);
+    double start = -kLag;
+    for (int i = 0; i < n; ++i) {
+      start = std::max(start + kLag, end[i % P]);
+      end[i % P] = start + c.p.nz;
+      if (i >= 4 * P && i % P == P - 1) {              // steady: the remaining waves alike
+        const double wave = std::max(P * kLag, (double)c.p.nz);
+        start += wave * ((n - 1 - i) / P);
+        break;
+      }
+    }
+    const double t = (start + c.p.nz) * slice_cycles_2d(c.p, s->eb, c.p.split);
+    if (best_t < 0 || t < best_t) {
+      best_t = t;
+      best = &c.p;
+      bestP = P;
+    }
+  }
+  Params q = s->p;
+  if (best != &s->p) {
+    // the shape: split, threads and shared-memory layout; everything else is the simulation's
+    const Params& b = *best;
+    q.split = b.split;
+    q.nthreads = b.nthreads;
+    q.pcap = b.pcap;
+    gempic::smem_layout(q, s->eb);
+  }
+  q.P = bestP;
+  return q;
+}
+
+gempic_status create_sim(const gempic_config* cfg, gempic_sim** out, bool one_cta) {
   if (!cfg || !out) return GEMPIC_EINVAL;
   *out = nullptr;
   const gempic_grid& g = cfg->grid;
@@ -394,6 +469,7 @@ gempic_status gempic_create(const gempic_config* cfg, gempic_sim** out) {
 
   Params& p = s->p;
   p.resid = (cfg->flags & GEMPIC_FLAG_RESIDUAL) ? 1 : 0;   // sizes shared memory
+  p.split = 1;
   p.nx = g.nx;
   p.ny = g.ny;
   p.nz = g.nzeta;
@@ -429,7 +505,7 @@ gempic_status gempic_create(const gempic_config* cfg, gempic_sim** out) {
     return GEMPIC_ECUDA;
   }
   const int nxh = g.nx / 2;
-  int C = cfg->cluster_ctas;
+  const int C = cfg->cluster_ctas;
   bool chosen = false;
   for (int cand = (C > 0 ? C : 1); cand <= (C > 0 ? C : 16); cand *= 2) {
     if (g.ny % cand || nxh % cand) continue;
@@ -439,22 +515,29 @@ gempic_status gempic_create(const gempic_config* cfg, gempic_sim** out) {
     const int RB = g.ny / cand, KB = nxh / cand, M = KB * g.ny;
     if (M > 512) continue;
     const int fresh = RB * g.nx * ppc_sum;
-    int NT = std::max(M, fresh / 4);
-    NT = std::min(512, std::max(128, (NT + 31) / 32 * 32));
+    // a larger cluster than the slice needs shortens the march: the push and the transforms divide
+    // by the CTAs, the barriers do not grow.  ms per s-step of one march, 96 slices, 2 per cell,
+    // C = 1, 2, 4, 8, 16: 16 x 16 FP32 1.31 1.11 1.10 1.05 -; 32 x 32 FP32 3.19 1.69 1.24 1.07 1.09;
+    // 64 x 64 FP32 - - 2.98 1.65 1.27; 32 x 32 FP64 - 21.1 11.4 6.9 5.1.  Clusters of 16 leave room
+    // for 7 to 14 marches where those of 8 leave 15 or more (64 x 64 FP32 with 48 s-steps in a call:
+    // 0.133 ms per s-step with 8, 0.174 with 16), so they want more work per CTA
+    if (chosen && fresh < (cand <= 8 ? 64 : cfg->precision == 64 ? 128 : 512)) break;
+    Params t = p;
+    t.C = cand;
+    t.RB = RB;
+    t.KB = KB;
+    t.logRB = ilog2(RB);
+    t.logKB = ilog2(KB);
+    t.M = M;
+    t.nthreads = pick_threads(cfg->precision, M, fresh);
+    bool fits = false;
     // streaming slots beyond the fresh layer hold stored particles that rejoin the march;
     // by default as many as the shared-memory budget allows, up to max(256, fresh)
     int head = cfg->particle_headroom > 0 ? cfg->particle_headroom : std::max(256, fresh);
-    p.C = cand;
-    p.RB = RB;
-    p.KB = KB;
-    p.logRB = ilog2(RB);
-    p.logKB = ilog2(KB);
-    p.M = M;
-    p.nthreads = NT;
     for (;;) {
-      p.pcap = fresh + head;
-      if (gempic::smem_layout(p, s->eb) <= smem_optin) {
-        chosen = true;
+      t.pcap = fresh + head;
+      if (gempic::smem_layout(t, s->eb) <= smem_optin) {
+        fits = true;
         break;
       }
       if (cfg->particle_headroom > 0 || head <= 32) break;
@@ -462,12 +545,15 @@ gempic_status gempic_create(const gempic_config* cfg, gempic_sim** out) {
     }
     // many particles per cell: a fresh layer larger than the shared memory keeps as many
     // slots there as fit and continues in the overflow slots in global memory
-    for (int pc = (fresh / 256) * 256; !chosen && cfg->particle_headroom <= 0 && pc >= 512;
+    for (int pc = (fresh / 256) * 256; !fits && cfg->particle_headroom <= 0 && pc >= 512;
          pc -= 256) {
-      p.pcap = pc;
-      if (gempic::smem_layout(p, s->eb) <= smem_optin) chosen = true;
+      t.pcap = pc;
+      if (gempic::smem_layout(t, s->eb) <= smem_optin) fits = true;
     }
-    if (chosen) break;
+    if (!fits) continue;
+    p = t;
+    chosen = true;
+    if (one_cta) break;
   }
   if (!chosen) {
     delete s;
@@ -493,7 +579,41 @@ gempic_status gempic_create(const gempic_config* cfg, gempic_sim** out) {
     delete s;
     return GEMPIC_ECUDA;
   }
-  s->pmax = cfg->pipeline_depth > 0 ? cfg->pipeline_depth : std::max(1, std::min(maxcl, 16));
+  if (g.ny == 1 && C == 0 && !one_cta && !p.resid) {
+    // 2-D: the shapes a launch chooses from (plan_launch)
+    int nsm = 0;
+    e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    for (int S = 1; S <= kMaxSplit && e == cudaSuccess; S *= 2) {
+      gempic_sim::Shape sh{p, 0};
+      Params& t = sh.p;
+      if (S > 1) {
+        const int share = (g.nx * ppc_sum + S - 1) / S;
+        if (share < 64) break;
+        t.split = S;
+        t.nthreads = pick_threads(cfg->precision, t.M, share);
+        int head = cfg->particle_headroom > 0 ? cfg->particle_headroom : std::max(256, share);
+        bool fits = false;
+        for (; !fits; head -= 32) {
+          t.pcap = share + head;
+          fits = gempic::smem_layout(t, s->eb) <= smem_optin;
+          if (!fits && (cfg->particle_headroom > 0 || head <= 32)) break;
+        }
+        if (!fits) continue;
+      }
+      e = gempic::max_active_clusters(cfg->precision, t, &sh.maxcl);
+      sh.maxcl = std::min(sh.maxcl, nsm / S);          // one CTA per SM
+      if (e == cudaSuccess) s->shapes.push_back(sh);
+    }
+    if (e != cudaSuccess) {
+      delete s;
+      return GEMPIC_ECUDA;
+    }
+  }
+  // marches in flight: a march trails the one before it by about four slices, so up to a quarter
+  // of the window's slices march at once.  2-D marches take one CTA each, and 16 of them (the
+  // limit of the clustered 3-D marches) left 136 of 152 SMs idle
+  const int deepest = s->shapes.empty() ? 16 : std::min(64, std::max(16, g.nzeta / 4));
+  s->pmax = cfg->pipeline_depth > 0 ? cfg->pipeline_depth : std::max(1, std::min(maxcl, deepest));
   if (s->pmax > std::max(1, maxcl)) s->pmax = std::max(1, maxcl);
   p.ring = s->pmax + 2;
 
@@ -583,7 +703,13 @@ gempic_status gempic_create(const gempic_config* cfg, gempic_sim** out) {
     // overflow particle slots: bands that gain particles (radial expulsion, rejoining stored
     // particles) spill beyond their shared-memory capacity into these
     p.gcap = std::max(1024, g.nx * (g.ny / p.C) * std::max(ppc_sum, 1) * 2);
-    ALLOC(p.pover, (size_t)std::max(s->pmax, 1) * p.C * p.gcap * (4 + 7 * eb));
+    {
+      // one area per CTA of a launch (2-D: every shape's marches x CTAs)
+      size_t ctas = (size_t)std::max(s->pmax, 1) * p.C;
+      for (const gempic_sim::Shape& sh : s->shapes)
+        ctas = std::max(ctas, (size_t)std::min(s->pmax, sh.maxcl) * sh.p.split);
+      ALLOC(p.pover, ctas * p.gcap * (4 + 7 * eb));
+    }
     if (p.snapshot) ALLOC(p.snap, (size_t)9 * g.nzeta * nperp * eb);
     if (cfg->flags & GEMPIC_FLAG_CURRENT) {
       ALLOC(s->jcap, (size_t)3 * g.nzeta * nperp * eb);
@@ -603,6 +729,21 @@ fail:
   delete s;
   cudaGetLastError();
   return e == cudaErrorMemoryAllocation ? GEMPIC_ENOMEM : GEMPIC_ECUDA;
+}
+
+}  // namespace
+
+namespace gempic {
+// a member of a batch: the smallest cluster that holds a slice, one launch shape
+gempic_status batch_member(const gempic_config* cfg, gempic_sim** out) {
+  return create_sim(cfg, out, true);
+}
+}  // namespace gempic
+
+extern "C" {
+
+gempic_status gempic_create(const gempic_config* cfg, gempic_sim** out) {
+  return create_sim(cfg, out, false);
 }
 
 gempic_status gempic_add_particles(gempic_sim* s, int64_t n, const double* x, const double* y,
@@ -694,15 +835,16 @@ static gempic_status denoised_chain(gempic_sim* s, int n) {
   // at most 7 marches in flight: the first pass of s-step i+4 reuses the current buffers of
   // s-step i only after it starts, i.e. after march 2i+8-P, the second pass of s-step i or later,
   // has finished with them.  The net runs on the SMs the marches leave free: unless the
-  // configuration sets the depth, the marches take at most two thirds of them (on GB300 at
-  // 128 x 128 x 512, 1 ppc, the chain's time per s-step against its depth was 11.5, 7.7, 6.8,
-  // 5.5, 5.3 and 7.3 ms for 2 to 7 clusters of 16 CTAs: 6 leaves 56 SMs to the net).
+  // configuration sets the depth, the marches take at most three quarters of them (on GB300 at
+  // 128 x 128 x 512, 1 ppc, 7 s-steps, the chain's time per s-step against its depth is 7.5, 6.7,
+  // 5.3, 5.2 and 4.1 ms for 3 to 7 clusters of 16 CTAs; with the net twice as slow 7 of them
+  // starved it, 7.3 ms against 5.3 with 6).
   int dev = 0, nsm = 0;
   e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return cuda_fail(s, e);
   const int want = s->cfg.pipeline_depth > 0 ? s->cfg.pipeline_depth
-                                             : std::max(1, 2 * nsm / (3 * s->p.C));
+                                             : std::max(1, 3 * nsm / (4 * s->p.C));
   const int P = std::min(std::min(std::min(s->pmax, 2 * n), 7), want);
   const long long k0 = s->k;
   unsigned long long* done = s->dn_host;
@@ -812,6 +954,7 @@ static gempic_status denoised_chain(gempic_sim* s, int n) {
   if (e != cudaSuccess) return cuda_fail(s, e);
   s->last_launch_k0 = k0;
   s->last_launch_n = 2 * n;
+  s->nrank_last = s->p.C;
   s->denoised_last = true;
   s->jcap_last = s->dn_jcap[(k0 + n - 1) & 3];
   s->k += n;
@@ -833,13 +976,13 @@ gempic_status gempic_step_async(gempic_sim* s, int32_t n) {
   s->denoised_last = false;
   cudaError_t e = ensure_diag_cap(s, n);
   if (e != cudaSuccess) return cuda_fail(s, e);
-  Params q = s->p;
+  Params q = plan_launch(s, n);
   q.k0 = s->k;
   q.nsteps = n;
-  q.P = std::min(s->pmax, n);
   q.inject = q.nspecies > 0 ? 1 : 0;
   q.delta_field = s->p.delta;
   e = gempic::launch_march(s->cfg.precision, q, s->stream);
+  s->nrank_last = q.C * q.split;
   s->launches++;
   if (e != cudaSuccess) return cuda_fail(s, e);
   s->last_launch_k0 = s->k;
@@ -946,14 +1089,15 @@ gempic_status gempic_step_host(gempic_sim* s, int32_t n, const void* state_in, v
 // the FP64 diagnostic sums of march `sl` of the last launch: the per-CTA partials added
 static cudaError_t diag_sums(gempic_sim* s, int sl, double* v) {
   const Params& p = s->p;
-  std::vector<double> d((size_t)gempic::kNDiag * p.C);
-  cudaError_t e = cudaMemcpyAsync(d.data(), p.diag_out + (size_t)sl * gempic::kNDiag * p.C,
+  const int nr = s->nrank_last;
+  std::vector<double> d((size_t)gempic::kNDiag * nr);
+  cudaError_t e = cudaMemcpyAsync(d.data(), p.diag_out + (size_t)sl * gempic::kNDiag * nr,
                                   d.size() * sizeof(double), cudaMemcpyDeviceToHost, s->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
   if (e != cudaSuccess) return e;
   for (int i = 0; i < gempic::kNDiag; ++i) {
     v[i] = 0.0;
-    for (int r = 0; r < p.C; ++r) v[i] += d[(size_t)i * p.C + r];
+    for (int r = 0; r < nr; ++r) v[i] += d[(size_t)i * nr + r];
   }
   return cudaSuccess;
 }
@@ -1195,6 +1339,7 @@ gempic_status gempic_step_streamed(gempic_sim* s, int32_t n, void* host, size_t 
   if (e != cudaSuccess) return cuda_fail(s, e);
   s->last_launch_k0 = s->k;
   s->last_launch_n = n;
+  s->nrank_last = s->p.C;
   s->denoised_last = false;
   s->k += n;
   if (result != GEMPIC_OK) {

@@ -26,6 +26,7 @@
 #include "gempic_internal.h"
 
 namespace gempic {
+gempic_status batch_member(const gempic_config* cfg, gempic_sim** out);
 gempic_status batch_prepare(gempic_sim* s, int nthreads, int nsteps, Params* out);
 void batch_advance(gempic_sim* s, int n);
 int batch_precision(const gempic_sim* s);
@@ -85,7 +86,7 @@ double time_class(const gempic_config& cfg, int nt, cudaStream_t stream) {
   c.pipeline_depth = 1;
   c.beam = nullptr;
   gempic_sim* sim = nullptr;
-  if (gempic_create(&c, &sim) != GEMPIC_OK) return -1.0;
+  if (gempic::batch_member(&c, &sim) != GEMPIC_OK) return -1.0;
   double ms = -1.0;
   gempic::Params q;
   if (gempic::batch_prepare(sim, nt, 1, &q) == GEMPIC_OK && gempic_step(sim, 1) == GEMPIC_OK) {
@@ -212,7 +213,7 @@ gempic_status gempic_batch_create(const gempic_config* cfgs, int32_t n, gempic_b
     c.cuda_stream = b->stream;
     c.pipeline_depth = kBatchDepth;
     gempic_sim* sim = nullptr;
-    st = gempic_create(&c, &sim);
+    st = gempic::batch_member(&c, &sim);
     if (st == GEMPIC_OK) b->sims.push_back(sim);
   }
   if (st == GEMPIC_OK) st = autotune(b, cfgs, n);

@@ -34,7 +34,9 @@ struct PartStore {
 struct Params {
   // grid and decomposition
   int nx, ny, nz;                 // transverse nodes, slices
-  int C, RB, KB, M;               // CTAs per cluster, rows per CTA, kx per CTA, modes per CTA
+  int C, RB, KB, M;               // CTAs per slice, rows per CTA, kx per CTA, modes per CTA
+  int split;                      // 2-D: CTAs that share a march's particles (1: not split); the
+                                  // cluster has C split CTAs
   int FR, JR, JOFF;               // field rows per CTA (own + halo above), current rows (own +
                                   // halo below/above), row offset of own row 0 in the currents
   int lognx, logny, logRB, logKB;
@@ -71,7 +73,7 @@ struct Params {
   int gcap;                       // further slots per CTA in global memory (overflow)
   int bcap, ring;                 // stored bucket capacity, ring of s-levels
   int wait_spin_limit;            // bounded wait: polls before giving up
-  int nwork;                      // FFT work rows per CTA
+  int nwork;                      // work rows of the inverse row transform
   int mig_cap;                    // migrating particles a CTA can receive per slice
   // shared-memory layout (byte offsets)
   int o_f0, o_f1, o_j, o_recv, o_sr, o_sc, o_workB, o_workD, o_tw, o_inbox, o_outbox, o_part, o_misc, o_dd,
@@ -85,7 +87,7 @@ struct Params {
   PartStore rq;                   // rejoin queues
   void* jbeam;                    // [ring][nz][3][ny][nx]
   int* jflag;                     // [ring][nz]
-  double* diag_out;               // [nsteps][kNDiag][C]
+  double* diag_out;               // [nsteps][kNDiag][C split]
   double* onaxis;                 // [nsteps][nz]
   void* snap;                     // [9][nz][ny][nx]
   // denoised s-step (two passes): the first marches the particles with the plain deposit,
@@ -97,7 +99,7 @@ struct Params {
   const void* jext;               // [nz][3][ny][nx] current replacing the deposit
   void* state_out;                // new level written here instead of over the old one
   int skip_stored, fields_only;
-  void* pover;                    // overflow particle slots [P*C][int cell; 7 reals][gcap]
+  void* pover;                    // overflow particle slots [CTA][int cell; 7 reals][gcap]
   unsigned long long* timers;     // phase timers (builds with GEMPIC_PHASE_TIMERS only)
   // state streamed through host memory (gempic_step_streamed): the old level is read from
   // `state`, the new one written to `state_out`, both in the public layout; the blocks go out

@@ -180,6 +180,11 @@ __device__ __forceinline__ double ldc(uint32_t a, double) {
   asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(a));
   return v;
 }
+__device__ __forceinline__ int ldc_s32(uint32_t a) {
+  int v;
+  asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(v) : "r"(a));
+  return v;
+}
 __device__ __forceinline__ void red_local(uint32_t a, float v) {
   asm volatile("red.shared.add.f32 [%0], %1;" ::"r"(a), "f"(v));
 }
@@ -230,36 +235,34 @@ __device__ __forceinline__ Cx<T> twiddle(const Cx<T>* tw, int N, int m, bool inv
   return w;
 }
 
-// radix-2, any N = 2^logN (used for N < 32 and N > 256)
+// Radix-2 transforms of `rows` consecutive rows of N = 2^logN values by the whole CTA (any N; used
+// for N < 32, N > 256 and for the FP64 rows of 2-D grids).  A 2-D slice has only two rows to
+// transform forward and three back, and rows of 8 or 16 values leave most lanes of a warp idle:
+// with one row per warp the two transforms of a 512-point FP32 slice took 35 of 68 k cycles, each
+// stage a chain of eight dependent passes of one warp; here every stage is one pass of all the
+// CTA's threads.  The butterflies and twiddles are those of the one-warp transform.
+// Input in bit-reversed positions (bitrev); every thread of the CTA calls it.
+__device__ __forceinline__ int bitrev(int i, int logN) {
+  return logN ? (int)(__brev((unsigned)i) >> (32 - logN)) : 0;
+}
 template <typename T>
-__device__ void warp_fft_r2(Cx<T>* d, int logN, const Cx<T>* tw, bool inverse) {
-  const int N = 1 << logN;
-  const int lane = threadIdx.x & 31;
-  for (int i = lane; i < N; i += 32) {
-    const int r = (int)(__brev((unsigned)i) >> (32 - logN));
-    if (i < r) {
-      Cx<T> t = d[i];
-      d[i] = d[r];
-      d[r] = t;
-    }
-  }
-  __syncwarp();
+__device__ void block_fft_r2(Cx<T>* d, int rows, int logN, const Cx<T>* tw, bool inverse) {
+  const int total = rows << (logN - 1);
+  __syncthreads();
   for (int s = 1; s <= logN; ++s) {
     const int half = 1 << (s - 1);
-    const int tstride = N >> s;
-    for (int b = lane; b < N / 2; b += 32) {
-      const int grp = b >> (s - 1);
+    for (int b = threadIdx.x; b < total; b += blockDim.x) {
       const int j = b & (half - 1);
-      const int i0 = grp * (half << 1) + j;
+      const int i0 = ((b >> (s - 1)) << s) + j;
       const int i1 = i0 + half;
-      Cx<T> w = tw[j * tstride];
+      Cx<T> w = tw[j << (logN - s)];
       if (inverse) w.im = -w.im;
       const Cx<T> t = w * d[i1];
       const Cx<T> u = d[i0];
       d[i0] = u + t;
       d[i1] = u - t;
     }
-    __syncwarp();
+    __syncthreads();
   }
 }
 
@@ -522,10 +525,12 @@ struct Sm {
   T* F[2];          // [6][FR][nx] real-space fields (Ex,Ey,Ez,Bx,By,Bz)
   T* J;             // [3][JR][nx] current accumulators (jx on x-edges, jy (3-D: y-edges), jz)
   int* Jint;        // [3][JR][nx] fixed-point accumulators of the push phase (FP32; aliases SR)
-  T* recv;          // [3][3][nx] halo currents received: rows 0, 1 (from below), RB-1 (above)
+  T* recv;          // [3][3][nx] halo currents received: rows 0, 1 (from below), RB-1 (above);
+                    // a split march: [3][nx] the summed currents of the slice
   Cx<T>* SR;        // [6][FR][nx/2] row spectra received for the inverse transform
   Cx<T>* SC;        // [6][KB][ny] column spectra (forward: 3 currents; inverse: 6 fields)
-  Cx<T>* workB;     // [nwork][nx] row FFT work of the forward transform (aliases SR)
+  Cx<T>* workB;     // [2 RB][nx] row FFT work or staging of the forward transform (aliases SR,
+                    // its own region when a march is split: other CTAs still read Jint)
   Cx<T>* workD;     // [nwork][nx] row FFT work of the inverse transform (aliases SC)
   Cx<T>* twx;       // [nx/2]
   Cx<T>* twy;       // [max(ny/2,1)]
@@ -711,7 +716,7 @@ __device__ __forceinline__ void st_cx(const cg::cluster_group& cl, Cx<T>* local,
 // element (comp, k, yl), yl fastest, goes to its kx owner: a warp's 32 stores go to one CTA.
 template <typename T, int R>
 __device__ void forward_rows_reg(const cg::cluster_group& cl, const Params& p, const Sm<T>& s,
-                                 int me, bool stagger) {
+                                 const T* J, int me, bool stagger) {
   constexpr int N = 32 * R, NH = N / 2, SP = 17;
   constexpr int LR = R == 1 ? 0 : R == 2 ? 1 : R == 4 ? 2 : 3;
   const int warp = threadIdx.x >> 5, l = threadIdx.x & 31;
@@ -719,11 +724,11 @@ __device__ void forward_rows_reg(const cg::cluster_group& cl, const Params& p, c
   const int ntask = 2 * p.RB;
   const int k1 = bitrev5(l);
   const int src0 = bitrev5((32 - k1) & 31);
-  Cx<T>* stg = s.SR;      // [3][R][RB][SP]
+  Cx<T>* stg = s.workB;   // [3][R][RB][SP]
   for (int task = warp; task < ntask; task += nwarps) {
     const int yl = task >> 1, pr = task & 1;
-    const T* A = s.J + ((size_t)(pr == 0 ? 0 : 2) * p.JR + yl + p.JOFF) * N;
-    const T* B = s.J + ((size_t)1 * p.JR + yl + p.JOFF) * N;
+    const T* A = J + ((size_t)(pr == 0 ? 0 : 2) * p.JR + yl + p.JOFF) * N;
+    const T* B = J + ((size_t)1 * p.JR + yl + p.JOFF) * N;
     Cx<T> a[R];
 #pragma unroll
     for (int r = 0; r < R; ++r) a[r] = cx<T>(A[l + 32 * r], pr == 0 ? B[l + 32 * r] : T(0));
@@ -834,16 +839,17 @@ __device__ void forward_rows_128(const cg::cluster_group& cl, const Params& p, c
 // carried per-mode state at every length
 template <typename T>
 __device__ __noinline__ void forward_rows_r8(const cg::cluster_group& cl, const Params& p,
-                                             const Sm<T>& s, int me, bool stagger) {
-  forward_rows_reg<T, 8>(cl, p, s, me, stagger);
+                                             const Sm<T>& s, const T* J, int me, bool stagger) {
+  forward_rows_reg<T, 8>(cl, p, s, J, me, stagger);
 }
 
 // SH = 1: the kernel instantiated for 128 x 128 grids with an even band (only the length-128
 // transforms are compiled in; with the other lengths present the compiler schedules them
 // markedly worse)
+// J: the slice's currents (s.J, or the sum over the CTAs of a split march)
 template <typename T, int SH>
 __device__ void forward_rows(const cg::cluster_group& cl, const Params& p, const Sm<T>& s,
-                             int me, bool stagger) {
+                             const T* J, int me, bool stagger) {
   if constexpr (SH == 1) {
     forward_rows_128(cl, p, s, me, stagger);
   } else {
@@ -851,41 +857,44 @@ __device__ void forward_rows(const cg::cluster_group& cl, const Params& p, const
     forward_rows_128(cl, p, s, me, stagger);
     return;
   }
-  switch (p.lognx) {
-    case 5: forward_rows_reg<T, 1>(cl, p, s, me, stagger); return;
-    case 6: forward_rows_reg<T, 2>(cl, p, s, me, stagger); return;
-    case 7: forward_rows_reg<T, 4>(cl, p, s, me, stagger); return;
-    case 8: forward_rows_r8<T>(cl, p, s, me, stagger); return;
-    default: break;
+  // FP64 rows of 2-D grids: two rows on two warps are bound by the FP64 chain of a warp; the
+  // whole CTA takes them at every length
+  if (sizeof(T) == 4 || p.ny > 1) {
+    switch (p.lognx) {
+      case 5: forward_rows_reg<T, 1>(cl, p, s, J, me, stagger); return;
+      case 6: forward_rows_reg<T, 2>(cl, p, s, J, me, stagger); return;
+      case 7: forward_rows_reg<T, 4>(cl, p, s, J, me, stagger); return;
+      case 8: forward_rows_r8<T>(cl, p, s, J, me, stagger); return;
+      default: break;
+    }
   }
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int nxh = p.nx / 2;
   const int ntask = 2 * p.RB;                 // (row, pair): pair 0 = jx + i jy, 1 = jz
-  if (warp >= p.nwork) return;
-  for (int task = warp; task < ntask; task += p.nwork) {
-    Cx<T>* w = s.workB + (size_t)warp * p.nx;
+  Cx<T>* w = s.workB;
+  for (int i = threadIdx.x; i < ntask << p.lognx; i += blockDim.x) {
+    const int task = i >> p.lognx, x = i & (p.nx - 1);
     const int yl = task >> 1, pr = task & 1;
-    const T* a = s.J + ((size_t)(pr == 0 ? 0 : 2) * p.JR + yl + p.JOFF) * p.nx;
-    const T* b = s.J + ((size_t)1 * p.JR + yl + p.JOFF) * p.nx;
-    for (int x = lane; x < p.nx; x += 32) w[x] = cx<T>(a[x], pr == 0 ? b[x] : T(0));
-    __syncwarp();
-    warp_fft_r2(w, p.lognx, s.twx, false);
-    const int y = (me << p.logRB) + yl;
-    for (int k = lane; k < nxh; k += 32) {
-      const Cx<T> zk = w[k];
-      const Cx<T> zm = conjg(w[(p.nx - k) & (p.nx - 1)]);
-      Cx<T> X = T(0.5) * (zk + zm);                     // spectrum of the real part
-      const Cx<T> Y = T(0.5) * mul_i(zm - zk);          // spectrum of the imaginary part
-      const int rd = k >> p.logKB, kxl = k & (p.KB - 1);
-      if (pr == 0) {
-        if (stagger) X = X * s.shx[k];
-        st_cx(cl, s.SC + ((size_t)0 * p.KB + kxl) * p.ny + y, rd, me, X);
-        st_cx(cl, s.SC + ((size_t)1 * p.KB + kxl) * p.ny + y, rd, me, Y);
-      } else {
-        st_cx(cl, s.SC + ((size_t)2 * p.KB + kxl) * p.ny + y, rd, me, X);
-      }
+    const T* a = J + ((size_t)(pr == 0 ? 0 : 2) * p.JR + yl + p.JOFF) * p.nx;
+    const T* b = J + ((size_t)1 * p.JR + yl + p.JOFF) * p.nx;
+    w[(task << p.lognx) + bitrev(x, p.lognx)] = cx<T>(a[x], pr == 0 ? b[x] : T(0));
+  }
+  block_fft_r2(w, ntask, p.lognx, s.twx, false);
+  for (int i = threadIdx.x; i < ntask * nxh; i += blockDim.x) {
+    const int task = i >> (p.lognx - 1), k = i & (nxh - 1);
+    const int pr = task & 1, y = (me << p.logRB) + (task >> 1);
+    const Cx<T>* wr = w + (task << p.lognx);
+    const Cx<T> zk = wr[k];
+    const Cx<T> zm = conjg(wr[(p.nx - k) & (p.nx - 1)]);
+    Cx<T> X = T(0.5) * (zk + zm);                     // spectrum of the real part
+    const Cx<T> Y = T(0.5) * mul_i(zm - zk);          // spectrum of the imaginary part
+    const int rd = k >> p.logKB, kxl = k & (p.KB - 1);
+    if (pr == 0) {
+      if (stagger) X = X * s.shx[k];
+      st_cx(cl, s.SC + ((size_t)0 * p.KB + kxl) * p.ny + y, rd, me, X);
+      st_cx(cl, s.SC + ((size_t)1 * p.KB + kxl) * p.ny + y, rd, me, Y);
+    } else {
+      st_cx(cl, s.SC + ((size_t)2 * p.KB + kxl) * p.ny + y, rd, me, X);
     }
-    __syncwarp();
   }
   }
 }
@@ -947,17 +956,30 @@ __device__ void column_ffts(const Params& p, const Sm<T>& s, int c0, int c1, boo
       column_ffts_128(p, s, c0, c1, inverse);
       return;
     }
+    const int ntask = (c1 - c0) << p.logKB;
+    if (!reg_fft_len(p.logny)) {
+      // all columns at once, in place: bit reversal, then the CTA-wide stages
+      Cx<T>* d = s.SC + ((size_t)c0 * p.KB) * p.ny;
+      for (int i = threadIdx.x; i < ntask << p.logny; i += blockDim.x) {
+        const int q = i & (p.ny - 1), r = bitrev(q, p.logny);
+        if (q < r) {
+          const Cx<T> t = d[i];
+          d[i] = d[i - q + r];
+          d[i - q + r] = t;
+        }
+      }
+      block_fft_r2(d, ntask, p.logny, s.twy, inverse);
+      return;
+    }
     const int warp = threadIdx.x >> 5;
     const int nwarps = blockDim.x >> 5;
-    const int ntask = (c1 - c0) << p.logKB;
     for (int task = warp; task < ntask; task += nwarps) {
       const int c = c0 + (task >> p.logKB), kxl = task & (p.KB - 1);
       Cx<T>* d = s.SC + ((size_t)c * p.KB + kxl) * p.ny;
       switch (p.logny) {
         case 5: col_fft_reg<T, 1>(d, s.twy, inverse); break;
         case 6: col_fft_reg<T, 2>(d, s.twy, inverse); break;
-        case 8: col_fft_r8<T>(d, s.twy, inverse); break;
-        default: warp_fft_r2(d, p.logny, s.twy, inverse); break;
+        default: col_fft_r8<T>(d, s.twy, inverse); break;
       }
     }
   }
@@ -1099,44 +1121,45 @@ __device__ void inverse_rows(const Params& p, const Sm<T>& s, T* Fdst, T& fe) {
   if constexpr (SH == 1) {
     inverse_rows_128<T>(p, s, Fdst, fe);
   } else {
-    switch (p.lognx) {
-      case 5: inverse_rows_reg<T, 1>(p, s, Fdst, fe); return;
-      case 6: inverse_rows_reg<T, 2>(p, s, Fdst, fe); return;
-      case 7: inverse_rows_128<T>(p, s, Fdst, fe); return;
-      case 8: inverse_rows_r8<T>(p, s, Fdst, fe); return;
-      default: break;
+    if (sizeof(T) == 4 || p.ny > 1) {
+      switch (p.lognx) {
+        case 5: inverse_rows_reg<T, 1>(p, s, Fdst, fe); return;
+        case 6: inverse_rows_reg<T, 2>(p, s, Fdst, fe); return;
+        case 7: inverse_rows_128<T>(p, s, Fdst, fe); return;
+        case 8: inverse_rows_r8<T>(p, s, Fdst, fe); return;
+        default: break;
+      }
     }
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int nxh = p.nx / 2;
     const T scale = T(1.0 / ((double)p.nx * (double)p.ny));
     const int ntask = 3 * p.FR;
-    for (int task = (warp < p.nwork ? warp : ntask); task < ntask; task += p.nwork) {
-      Cx<T>* w = s.workD + (size_t)warp * p.nx;
-      const int yl = task / 3, pr = task - 3 * yl;
-      const Cx<T>* X = s.SR + ((size_t)(2 * pr) * p.FR + yl) * nxh;
-      const Cx<T>* Y = s.SR + ((size_t)(2 * pr + 1) * p.FR + yl) * nxh;
-      for (int k = lane; k < nxh; k += 32) {
-        Cx<T> x = X[k], y = Y[k];
+    Cx<T>* w = s.workD;
+    for (int t0 = 0; t0 < ntask; t0 += p.nwork) {         // as many rows as the work area holds
+      const int nt = min(p.nwork, ntask - t0);
+      for (int i = threadIdx.x; i < nt * nxh; i += blockDim.x) {
+        const int task = t0 + (i >> (p.lognx - 1)), k = i & (nxh - 1);
+        const int yl = task / 3, pr = task - 3 * yl;
+        const Cx<T> x = s.SR[((size_t)(2 * pr) * p.FR + yl) * nxh + k];
+        const Cx<T> y = s.SR[((size_t)(2 * pr + 1) * p.FR + yl) * nxh + k];
+        Cx<T>* wr = w + ((i >> (p.lognx - 1)) << p.lognx);
         if (k == 0) {
-          w[0] = cx<T>(x.re, y.re);                         // real DC of each field
+          wr[0] = cx<T>(x.re, y.re);                        // real DC of each field
+          wr[bitrev(nxh, p.lognx)] = cx<T>(T(0), T(0));     // Nyquist projected out
         } else {
-          w[k] = cx<T>(x.re - y.im, x.im + y.re);           // X + i Y
-          w[p.nx - k] = cx<T>(x.re + y.im, y.re - x.im);    // conj(X) + i conj(Y)
+          wr[bitrev(k, p.lognx)] = cx<T>(x.re - y.im, x.im + y.re);          // X + i Y
+          wr[bitrev(p.nx - k, p.lognx)] = cx<T>(x.re + y.im, y.re - x.im);   // conj(X) + i conj(Y)
         }
       }
-      if (lane == 0) w[nxh] = cx<T>(T(0), T(0));            // Nyquist projected out
-      __syncwarp();
-      warp_fft_r2(w, p.lognx, s.twx, true);
-      T* a = Fdst + ((size_t)(2 * pr) * p.FR + yl) * p.nx;
-      T* b = Fdst + ((size_t)(2 * pr + 1) * p.FR + yl) * p.nx;
-      const bool own = yl < p.RB;
-      for (int x = lane; x < p.nx; x += 32) {
-        const T va = w[x].re * scale, vb = w[x].im * scale;
-        a[x] = va;
-        b[x] = vb;
-        if (own) fe += va * va + vb * vb;
+      block_fft_r2(w, nt, p.lognx, s.twx, true);
+      for (int i = threadIdx.x; i < nt << p.lognx; i += blockDim.x) {
+        const int task = t0 + (i >> p.lognx), x = i & (p.nx - 1);
+        const int yl = task / 3, pr = task - 3 * yl;
+        const T va = w[i].re * scale, vb = w[i].im * scale;
+        Fdst[((size_t)(2 * pr) * p.FR + yl) * p.nx + x] = va;
+        Fdst[((size_t)(2 * pr + 1) * p.FR + yl) * p.nx + x] = vb;
+        if (yl < p.RB) fe += va * va + vb * vb;
       }
-      __syncwarp();
+      if (t0 + nt < ntask) __syncthreads();
     }
   }
 }
@@ -1717,10 +1740,10 @@ struct Ovf {
 };
 
 template <typename T>
-__device__ __forceinline__ Ovf<T> ovf_view(const Params& p, int cid, int me) {
+__device__ __forceinline__ Ovf<T> ovf_view(const Params& p, int cta) {
   Ovf<T> o;
   const size_t g = (size_t)p.gcap;
-  char* b = (char*)p.pover + ((size_t)cid * p.C + me) * g * (4 + 7 * sizeof(T));
+  char* b = (char*)p.pover + (size_t)cta * g * (4 + 7 * sizeof(T));
   o.cell = (int*)b;
   T* t = (T*)(b + 4 * g);
   o.fx = t;
@@ -1813,14 +1836,15 @@ __device__ __forceinline__ void warp_diag_add(double* dwarp, int slot, V v) {
 
 template <typename T>
 __device__ void stored_phase(const Params& p, const Sm<T>& s, const T* Fn, const T* Fn1,
-                             int s1, int s2, int n, int me, int cnt_raw, bool varh) {
-  // s1, s2: ring slots of the stored sets at levels k+1 and k+2
+                             int s1, int s2, int n, int me, int rank, int nrank, int cnt_raw,
+                             bool varh) {
+  // s1, s2: ring slots of the stored sets at levels k+1 and k+2; rank of nrank CTAs
   T dkin = T(0);
   int dsto = 0, dlost = 0;
   const int cnt = min(cnt_raw, p.bcap);
   const T D = s.cst[K_D], h = s.cst[K_H], invh = s.cst[K_INVH];
   const int mx = p.nx - 1, my = p.ny - 1;
-  for (int e0 = me * blockDim.x + threadIdx.x; e0 < cnt; e0 += p.C * blockDim.x) {
+  for (int e0 = rank * blockDim.x + threadIdx.x; e0 < cnt; e0 += nrank * blockDim.x) {
     T fz;
     PState<T> P = store_read<T>(p.st, p, ((size_t)s1 * p.nz + n) * p.bcap + e0, fz);
     const T g = gamma_of(P.u);
@@ -2062,7 +2086,19 @@ __device__ void march(const Params& p, const Sm<T>& s, const cg::cluster_group& 
   const int rbe = p.ny > 1 ? p.RB : 1;            // own rows of the residual planes
   T rmax = T(0), gmax = T(0);
   const T* hzt = (const T*)p.hzt;
-  const int me = (int)cl.block_rank();
+  // A split march (2-D: one row, C = 1): the p.split CTAs of its cluster share the particles.
+  // Each holds the whole slice and transforms and solves it on its own (the same arithmetic on
+  // the same sums); only the particles, their deposits and the stored set are divided, and the
+  // deposits summed over the cluster after B1.  CTA 0 alone writes the state, publishes and
+  // reports the fields.  A 2-D slice is one CTA's work otherwise, which leaves the chip idle
+  // where few s-steps are in flight, and its FP64 push is bound by the SM's two FP64 lanes
+  // (130 of 200 k cycles a slice at 128 cells, 4 per cell).
+  const bool spl = SH != 1 && p.split > 1;
+  const int rank = (int)cl.block_rank();
+  const int me = spl ? 0 : rank;
+  const int part = spl ? rank : 0;
+  const int nrank = spl ? p.split : p.C;
+  const bool lead = rank == 0;
   const int tid = threadIdx.x;
   const int NT = blockDim.x;
   // march index: k, or 2k + pass in a denoised chain; the previous march of the launch is
@@ -2078,7 +2114,7 @@ __device__ void march(const Params& p, const Sm<T>& s, const cg::cluster_group& 
   const int s2 = (int)(((k + 2) % p.ring + p.ring) % p.ring);
   const T h = s.cst[K_H], Dl = s.cst[K_DF];
   const long long sl = item - item0;                // march index within this launch
-  const Ovf<T> ov = ovf_view<T>(p, cid, me);        // overflow particle slots of this CTA
+  const Ovf<T> ov = ovf_view<T>(p, cid * nrank + rank);   // overflow particle slots of this CTA
   const int fplane = p.FR * p.nx;                   // elements of one field component
   const int jplane = p.JR * p.nx;                   // elements of one current component
   TIMER_DECL
@@ -2088,7 +2124,7 @@ __device__ void march(const Params& p, const Sm<T>& s, const cg::cluster_group& 
 
   // reset the next level's stored buckets and rejoin queues (free: their last reader, the
   // march of step k+1-ring, has completed)
-  for (int b = me * NT + tid; b < nz; b += p.C * NT) {
+  for (int b = rank * NT + tid; b < nz; b += nrank * NT) {
     p.st.cnt[(size_t)s2 * nz + b] = 0;
     p.rq.cnt[(size_t)s2 * nz + b] = 0;
   }
@@ -2107,12 +2143,14 @@ __device__ void march(const Params& p, const Sm<T>& s, const cg::cluster_group& 
   __syncthreads();
   if (p.inject && !dn2) {
     const int per_row = p.nlayer >> p.logny;        // particles per transverse row
-    const int nmine = per_row * p.RB;
+    // a split march: this CTA's share of the row
+    const int i0 = spl ? (int)((long long)per_row * part / p.split) : 0;
+    const int nmine = spl ? (int)((long long)per_row * (part + 1) / p.split) - i0 : per_row * p.RB;
     for (int i = tid; i < nmine; i += NT) {
       // storage order: segments of nx particles with fixed (row, species, k); inside a segment
       // position j holds cell ix = 5 j mod nx, so the 32 lanes of a warp deposit into cells 5
       // apart (disjoint stencils, distinct shared-memory banks)
-      const int seg = i >> p.lognx, j = i & (p.nx - 1);
+      const int seg = (i + i0) >> p.lognx, j = (i + i0) & (p.nx - 1);
       const int yl = seg / p.ppc_sum;
       int kk = seg - yl * p.ppc_sum;
       int sp = 0;
@@ -2312,7 +2350,7 @@ __device__ void march(const Params& p, const Sm<T>& s, const cg::cluster_group& 
       // stored particles that rejoin the march at this slice (partial first step), taken by
       // the CTA that owns their row
       const int nq = (p.fields_only || dn2) ? 0 : min(s.misc[M_RQN], p.bcap);
-      for (int e = tid; e < nq; e += NT) {
+      for (int e = spl ? tid * p.split + part : tid; e < nq; e += spl ? NT * p.split : NT) {
         const size_t ge = ((size_t)s1 * nz + n) * p.bcap + e;
         if ((((ldcg(p.rq.cell + ge) >> 10) & 1023) >> p.logRB) != me) continue;
         T fz;
@@ -2489,7 +2527,7 @@ __device__ void march(const Params& p, const Sm<T>& s, const cg::cluster_group& 
     }
 #endif
     // publish: iteration n+1 complete (its stored phase and this push have been issued)
-    if (p.P > 1 && me == 0 && tid == 0 && n + 1 <= nz - 1)
+    if (p.P > 1 && lead && tid == 0 && n + 1 <= nz - 1)
       st_release_u64(p.progress + cid, prog_value(item, nz, nz - (n + 1)));
     // denoised chain: the first pass's current of half-slices >= n + 1 is written
     if (dn1 && me == 0 && tid == 0) {
@@ -2509,8 +2547,22 @@ __device__ void march(const Params& p, const Sm<T>& s, const cg::cluster_group& 
     if (tid == NT - 32) s.misc[M_STN] = ldcg(p.st.cnt + (size_t)s1 * nz + n);
     TIMER_MARK(PH_B1);
     // own rows: fixed-point accumulators (FP32) and the received halo currents (rows 0, 1
-    // from the band below, RB - 1 from the band above); element mapping as in the beam add
-    if constexpr (sizeof(T) == 4) {
+    // from the band below, RB - 1 from the band above); element mapping as in the beam add.
+    // A split march sums the CTAs' accumulators instead (exact in fixed point), into recv: every
+    // CTA of the cluster reads them until B2
+    T* const Jf = spl ? s.recv : s.J;
+    if (spl) {
+      for (int i = tid; i < 3 * p.nx; i += NT) {
+        T v = T(0);
+        int q = 0;
+        for (int r = 0; r < p.split; ++r) {
+          v += ldc(cluster_addr(sh_addr(s.J + i), r), T(0));
+          if constexpr (sizeof(T) == 4) q += ldc_s32(cluster_addr(sh_addr(s.Jint + i), r));
+        }
+        if constexpr (sizeof(T) == 4) v += T(q) * s.cst[K_JINV];
+        Jf[i] = v;
+      }
+    } else if constexpr (sizeof(T) == 4) {
       const T jinv = s.cst[K_JINV];
       for (int i = 4 * tid; i < 3 * p.RB * p.nx; i += 4 * NT) {
         const int c = i >> (p.logRB + p.lognx);
@@ -2633,8 +2685,8 @@ __device__ void march(const Params& p, const Sm<T>& s, const cg::cluster_group& 
         const int c = i >> (p.logRB + p.lognx);
         const int rem = i & ((p.RB << p.lognx) - 1);
         const size_t g = (size_t)c * p.nx * p.ny + ((size_t)me << p.logRB) * p.nx + rem;
-        s.J[((size_t)c * p.JR + p.JOFF) * p.nx + rem] += ldcg(jb + g);
-        jb[g] = T(0);
+        Jf[((size_t)c * p.JR + p.JOFF) * p.nx + rem] += ldcg(jb + g);
+        if (!spl) jb[g] = T(0);                     // (a split march: after B2)
       }
     }
     if (snap_step || cap_step) {
@@ -2644,7 +2696,7 @@ __device__ void march(const Params& p, const Sm<T>& s, const cg::cluster_group& 
       for (int i = tid; i < 3 * p.RB * p.nx; i += NT) {
         const int c = i >> (p.logRB + p.lognx);
         const int rem = i & ((p.RB << p.lognx) - 1);
-        const T v = s.J[((size_t)c * p.JR + p.JOFF) * p.nx + rem];
+        const T v = Jf[((size_t)c * p.JR + p.JOFF) * p.nx + rem];
         if (snap_step) sn[(((size_t)(6 + c) * nz + n) * p.ny + (me << p.logRB)) * p.nx + rem] = v;
         // the current of the s-step in [nzeta][3][ny][nx] (the denoiser's layout)
         if (cap_step) jc[(((size_t)n * 3 + c) * p.ny + (me << p.logRB)) * p.nx + rem] = v;
@@ -2658,20 +2710,24 @@ __device__ void march(const Params& p, const Sm<T>& s, const cg::cluster_group& 
       for (int i = tid; i < 3 * p.RB * p.nx; i += NT) {
         const int c = i >> (p.logRB + p.lognx);
         const int rem = i & ((p.RB << p.lognx) - 1);
-        s.J[((size_t)c * p.JR + p.JOFF) * p.nx + rem] =
+        Jf[((size_t)c * p.JR + p.JOFF) * p.nx + rem] =
             ldcg(je + (((size_t)n * 3 + c) * p.ny + (me << p.logRB)) * p.nx + rem);
       }
     }
     if (beam_slice || snap_step || cap_step || jext) __syncthreads();
     TIMER_MARK(PH_BEAM);
     // ---------------- B: row FFTs of the currents, transposed to the kx owners ------------
-    forward_rows<T, SH>(cl, p, s, me, true);
+    forward_rows<T, SH>(cl, p, s, Jf, me, true);
     TIMER_MARK(PH_FWD);
     // streamed state: block n-1 of the input, read after the solve below
     if constexpr (CANON)
       if (p.io_chunk && tid == 0 && me == 0 && n >= 1) wait_input(p, k, n - 1, s.misc + M_IOSEEN);
     cl.sync();                                                      // B2
-    if (tid == 0 && me == 0) p.jflag[(size_t)s1 * nz + n] = 0;
+    if (tid == 0 && lead) p.jflag[(size_t)s1 * nz + n] = 0;
+    if (spl && lead && beam_slice) {
+      T* jb = (T*)p.jbeam + (((size_t)s1 * nz + n) * 3) * (size_t)p.nx * p.ny;
+      for (int i = tid; i < 3 * p.nx; i += NT) jb[i] = T(0);
+    }
     TIMER_MARK(PH_B2);
     // ---------------- C: column FFTs, per-mode solve, inverse column FFTs ------------------
     if constexpr (sizeof(T) == 4) {
@@ -2695,14 +2751,16 @@ __device__ void march(const Params& p, const Sm<T>& s, const cg::cluster_group& 
         S1.Ry = S1.Ry - (T(0.25) * Dl) * (Jy - jpy);
       }
       // new level, block n+1 = {R, E_z, B_z at slice n+1; j at n+1/2}
-      if (blk_ok(n + 1, 0)) {
+      if (part == 0 && blk_ok(n + 1, 0)) {
         stw[blk(n + 1, 0)] = S1.Rx;
         stw[blk(n + 1, 1)] = S1.Ry;
         stw[blk(n + 1, 2)] = S1.Ez;
         stw[blk(n + 1, 3)] = S1.Bz;
       }
-      stw[blk(n + 1, 4)] = Jx;
-      stw[blk(n + 1, 5)] = Jy;
+      if (part == 0) {
+        stw[blk(n + 1, 4)] = Jx;
+        stw[blk(n + 1, 5)] = Jy;
+      }
       // old level at slice n; j^0 at n -/+ 1/2
       const Cx<T> j0mx = n > 0 ? o[4] : j0px;
       const Cx<T> j0my = n > 0 ? o[5] : j0py;
@@ -2728,10 +2786,12 @@ __device__ void march(const Params& p, const Sm<T>& s, const cg::cluster_group& 
       j0px = j0mx;
       j0py = j0my;
       if (n == 0) {
-        stw[blk(0, 0)] = S0.Rx;
-        stw[blk(0, 1)] = S0.Ry;
-        stw[blk(0, 2)] = S0.Ez;
-        stw[blk(0, 3)] = S0.Bz;
+        if (part == 0) {
+          stw[blk(0, 0)] = S0.Rx;
+          stw[blk(0, 1)] = S0.Ry;
+          stw[blk(0, 2)] = S0.Ez;
+          stw[blk(0, 3)] = S0.Bz;
+        }
       } else {
 #pragma unroll
         for (int c = 0; c < 6; ++c)
@@ -2747,7 +2807,11 @@ __device__ void march(const Params& p, const Sm<T>& s, const cg::cluster_group& 
     TIMER_MARK(PH_SCAT);
     if (waits && tid == 0 && me == 0)
       wait_for(p, pcid, prog_value(item - 1, nz, min(nz, nz - n + 3)));   // down to n-3
-    cl.sync();                                                      // B3
+    // (2-D: the spectra and the fields of a slice stay in the CTA, B3 and B4 order its threads)
+    if (SH != 1 && p.ny == 1)
+      __syncthreads();
+    else
+      cl.sync();                                                    // B3
     // the predecessor is now known to be done down to slice n-3: counters of slice n-1,
     // loaded by the last warp (no inverse-transform task) so that no transform waits on them
     if (tid == NT - 32 && n > 0) {
@@ -2759,7 +2823,7 @@ __device__ void march(const Params& p, const Sm<T>& s, const cg::cluster_group& 
     {
       T fs = T(0);
       inverse_rows<T, SH>(p, s, Fnew, fs);
-      fe += (double)(varh ? fs * hn : fs);
+      if (part == 0) fe += (double)(varh ? fs * hn : fs);
     }
     TIMER_MARK(PH_INV);
     if constexpr (sizeof(T) == 4) {
@@ -2768,7 +2832,10 @@ __device__ void march(const Params& p, const Sm<T>& s, const cg::cluster_group& 
       for (int i = 4 * tid; i < 3 * jplane; i += 4 * NT)
         *reinterpret_cast<int4*>(s.Jint + i) = make_int4(0, 0, 0, 0);
     }
-    cl.sync();                                                      // B4: fields of slice n
+    if (SH != 1 && p.ny == 1)
+      __syncthreads();
+    else
+      cl.sync();                                                    // B4: fields of slice n
     TIMER_MARK(PH_B4);
     if (resid) {
       // Gauss residual on plane n: d_x L_x + d_y L_y - (rho - j_z), L_x = E_x - B_y,
@@ -2808,10 +2875,10 @@ __device__ void march(const Params& p, const Sm<T>& s, const cg::cluster_group& 
     }
     if (p.diag) {
       const int yc = p.ny / 2;
-      if (tid == 0 && (yc >> p.logRB) == me)
+      if (tid == 0 && part == 0 && (yc >> p.logRB) == me)
         p.onaxis[sl * nz + n] = (double)Fnew[((size_t)2 * p.FR + (yc & (p.RB - 1))) * p.nx + nxh];
     }
-    if (snap_step) {
+    if (snap_step && part == 0) {
       T* sn = (T*)p.snap;
       for (int i = tid; i < 6 * p.RB * p.nx; i += NT) {
         const int c = i >> (p.logRB + p.lognx);
@@ -2823,7 +2890,7 @@ __device__ void march(const Params& p, const Sm<T>& s, const cg::cluster_group& 
     // ---------------- E: stored particles of cell (zeta_n, zeta_{n+1}] along s -------------
     // (most cells hold no stored particle: the call is skipped, uniformly over the CTA)
     if (s.misc[M_STN] > 0 && !p.skip_stored && !dn1)
-      stored_phase(p, s, Fnew, Fcur, s1, s2, n, me, s.misc[M_STN], varh);
+      stored_phase(p, s, Fnew, Fcur, s1, s2, n, me, rank, nrank, s.misc[M_STN], varh);
     TIMER_MARK(PH_E);
     T* t = Fcur;
     Fcur = Fnew;
@@ -2833,7 +2900,7 @@ __device__ void march(const Params& p, const Sm<T>& s, const cg::cluster_group& 
   __syncthreads();
   if (tid == 0) __threadfence();
   cl.sync();
-  if (p.P > 1 && me == 0 && tid == 0) st_release_u64(p.progress + cid, prog_value(item, nz, nz));
+  if (p.P > 1 && lead && tid == 0) st_release_u64(p.progress + cid, prog_value(item, nz, nz));
   if constexpr (CANON)
     if (p.io_chunk && me == 0 && tid == 0) st_release_sys_u64(p.io_done + cid, prog_value(k, nz, nz));
   if (dn1 && me == 0 && tid == 0) st_release_sys_u64(p.dn_done + cid, prog_value(item, nz, nz));
@@ -2869,7 +2936,7 @@ __device__ void march(const Params& p, const Sm<T>& s, const cg::cluster_group& 
       const double hv = tid == DG_FIELD ? 0.5 * p.hx * p.hy * hw
                         : tid == DG_FLUX ? p.hx * p.hy * hw
                                          : 1.0;
-      p.diag_out[((size_t)sl * kNDiag + tid) * p.C + me] = v * hv;
+      p.diag_out[((size_t)sl * kNDiag + tid) * nrank + rank] = v * hv;
       // watchdog: a NaN or infinity anywhere in the slice fields or in a particle's momentum
       // reaches these FP64 sums
       if ((tid == DG_FIELD || tid == DG_KIN) && !isfinite(v)) atomicOr(p.err, ERR_NONFINITE);
@@ -2886,7 +2953,7 @@ __device__ __forceinline__ void march_launch(const Params& p) {
   load_tables(p, s);
   if (threadIdx.x < kNDiag) s.dacc[threadIdx.x] = 0.0;
   __syncthreads();
-  const int cid = (int)(blockIdx.x / p.C);
+  const int cid = (int)(blockIdx.x / (p.C * p.split));
   // a chain's march index is 2k + pass
   for (long long it = cid; it < p.nsteps; it += p.P) {
     const long long item = DN ? 2 * p.k0 + it : p.k0 + it;
@@ -3019,7 +3086,7 @@ __global__ void __launch_bounds__(512, 1)
       s.J[((size_t)c * p.JR + yl + p.JOFF) * p.nx + x] = (c == 2) ? T(2.0 * E) : T(0);
     }
     __syncthreads();
-    forward_rows<T, SH>(cl, p, s, me, false);
+    forward_rows<T, SH>(cl, p, s, s.J, me, false);
     cl.sync();
     column_ffts<T, SH>(p, s, 2, 3, false);
     __syncthreads();
@@ -3138,7 +3205,6 @@ int smem_layout(Params& p, int eb) {
   p.JR = p.ny > 1 ? p.RB + 3 : 1;
   p.JOFF = p.ny > 1 ? 1 : 0;
   p.mig_cap = p.ny > 1 ? 128 : 0;
-  p.nwork = std::min(p.nthreads / 32, 3 * p.FR);
   const int nxh = p.nx / 2;
   const int nyh = p.ny > 1 ? p.ny / 2 : 1;
   int o = 0;
@@ -3149,19 +3215,19 @@ int smem_layout(Params& p, int eb) {
   p.o_j = o;
   o += align16(3 * p.JR * p.nx * eb);
   p.o_recv = o;
-  o += align16((p.ny > 1 ? 9 : 1) * p.nx * eb);
+  o += align16((p.ny > 1 ? 9 : p.split > 1 ? 3 : 1) * p.nx * eb);
   p.o_sr = o;
-  const int sr_bytes = align16(6 * p.FR * nxh * 2 * eb);
-  o += sr_bytes;
+  o += align16(6 * p.FR * nxh * 2 * eb);
   p.o_sc = o;
   const int sc_bytes = align16(6 * p.KB * p.ny * 2 * eb);
   o += sc_bytes;
-  // row-FFT work rows live in SR (forward transform) and SC (inverse) when they fit
-  const int work = align16(p.nwork * p.nx * 2 * eb);
-  p.o_workB = work <= sr_bytes ? p.o_sr : o;
-  if (work > sr_bytes) o += work;
-  p.o_workD = work <= sc_bytes ? p.o_sc : o;
-  if (work > sc_bytes) o += work;
+  // row-FFT work rows live in SR (forward transform: 2 RB rows of its 3 FR) and SC (inverse: as
+  // many of the 3 FR rows at a time as fit, 3 RB); a split march's other CTAs read the
+  // accumulators in SR until B2, so its forward work has a region of its own
+  p.o_workB = p.split > 1 ? o : p.o_sr;
+  if (p.split > 1) o += align16(2 * p.RB * p.nx * 2 * eb);
+  p.o_workD = p.o_sc;
+  p.nwork = std::min(3 * p.FR, sc_bytes / (p.nx * 2 * eb));
   p.o_tw = o;
   o += align16((nxh + nyh + nxh + p.ny) * 2 * eb + (nxh + p.ny + 32) * eb);
   p.o_inbox = o;
@@ -3228,12 +3294,12 @@ cudaError_t configure_kernels(int precision, int smem, int) {
 static cudaLaunchConfig_t make_cfg(const Params& p, int nclusters, cudaStream_t s,
                                    cudaLaunchAttribute* attr) {
   cudaLaunchConfig_t c = {};
-  c.gridDim = dim3((unsigned)(nclusters * p.C), 1, 1);
+  c.gridDim = dim3((unsigned)(nclusters * p.C * p.split), 1, 1);
   c.blockDim = dim3((unsigned)p.nthreads, 1, 1);
   c.dynamicSmemBytes = (size_t)p.smem_bytes;
   c.stream = s;
   attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = (unsigned)p.C;
+  attr[0].val.clusterDim.x = (unsigned)(p.C * p.split);
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
   c.attrs = attr;

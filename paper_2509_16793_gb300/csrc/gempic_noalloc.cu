@@ -91,6 +91,7 @@ extern "C" gempic_status gempic_step_noalloc(const gempic_config* cfg, int64_t s
     if (st != GEMPIC_OK) return st;
   }
   const int ppc_sum = p.ppc_sum;
+  p.split = 1;
   p.nx = g.nx;
   p.ny = g.ny;
   p.nz = g.nzeta;
