@@ -33,9 +33,9 @@ struct gempic_sim {
   std::vector<double> hz, zp;      // variable zeta-step: slab thicknesses, plane positions
   Params p{};                      // launch template
   int eb = 8;                      // bytes per real
-  int pmax = 1;                    // concurrent marches
-  // 2-D: launch shapes with the particles of a march on 1, 2, 4, 8 CTAs (shape 0 is p's; a shape
-  // that does not apply has maxcl 0); empty: only p's
+  int pmax = 1;                    // concurrent marches of p's launch shape
+  // launch shapes that a call of several s-steps chooses from (plan_launch); empty: only p's.
+  // 2-D: the particles of a march on 1, 2, 4, 8 CTAs; FP32 128 x 128: one or two CTAs per SM
   struct Shape { Params p; int maxcl; };
   std::vector<Shape> shapes;
   int nrank_last = 1;              // CTAs per march of the last launch (diagnostic partials)
@@ -129,7 +129,7 @@ gempic_status check_device_error(gempic_sim* s) {
 cudaError_t ensure_diag_cap(gempic_sim* s, int n) {
   if (n <= s->diag_cap) return cudaSuccess;
   double *d = nullptr, *o = nullptr, *r = nullptr, *gr = nullptr;
-  cudaError_t e = dalloc(s, &d, (size_t)n * gempic::kNDiag * (s->shapes.empty() ? s->p.C : kMaxSplit) * sizeof(double));
+  cudaError_t e = dalloc(s, &d, (size_t)n * gempic::kNDiag * std::max(s->p.C, s->p.ny == 1 ? kMaxSplit : 1) * sizeof(double));
   if (e != cudaSuccess) return e;
   e = dalloc(s, &o, (size_t)n * s->p.nz * sizeof(double));
   if (e != cudaSuccess) return e;
@@ -353,17 +353,23 @@ double slice_cycles_2d(const Params& p, int eb, int S) {
   return push + fixed + (S > 1 ? 2500.0 + 2.0 * S * p.nx * 3 / p.nthreads * 8.0 : 0.0);
 }
 
+// the same of a 128 x 128 FP32 march: 54 k cycles with an SM to itself per CTA, 82 k with two
+// CTAs per SM and 14 marches in flight
+double slice_cycles_128(const Params& p) { return p.dense ? 82000.0 : 54000.0; }
+
 // The launch of n s-steps: parameters with the shape and the number of marches in flight.  2-D
 // grids choose how many CTAs share a march by the modelled time of the wavefront: march c starts
 // when march c - 1 is a few slices ahead (kLag) and march c - P has finished.  Many s-steps fill
 // the chip with marches of one CTA; few s-steps (or one) leave SMs to share a march's particles.
 Params plan_launch(const gempic_sim* s, int n) {
   constexpr double kLag = 4.0;
+  const int depth = s->cfg.pipeline_depth;
   const Params* best = &s->p;
   int bestP = std::min(s->pmax, n);
   double best_t = -1.0;
   for (const gempic_sim::Shape& c : s->shapes) {
-    const int P = std::min(std::min(s->pmax, n), c.maxcl);
+    int P = std::min(n, c.maxcl);
+    if (depth > 0) P = std::min(P, depth);
     if (P < 1) continue;
     std::vector<double> end((size_t)P, 0.0);
     double start = -kLag;
@@ -376,7 +382,7 @@ Params plan_launch(const gempic_sim* s, int n) {
         break;
       }
     }
-    const double t = (start + c.p.nz) * slice_cycles_2d(c.p, s->eb, c.p.split);
+    const double t = (start + c.p.nz) * (c.p.ny > 1 ? slice_cycles_128(c.p) : slice_cycles_2d(c.p, s->eb, c.p.split));
     if (best_t < 0 || t < best_t) {
       best_t = t;
       best = &c.p;
@@ -388,8 +394,10 @@ Params plan_launch(const gempic_sim* s, int n) {
     // the shape: split, threads and shared-memory layout; everything else is the simulation's
     const Params& b = *best;
     q.split = b.split;
+    q.dense = b.dense;
     q.nthreads = b.nthreads;
     q.pcap = b.pcap;
+    q.gcap = b.gcap;
     gempic::smem_layout(q, s->eb);
   }
   q.P = bestP;
@@ -615,7 +623,36 @@ gempic_status create_sim(const gempic_config* cfg, gempic_sim** out, bool one_ct
   const int deepest = s->shapes.empty() ? 16 : std::min(64, std::max(16, g.nzeta / 4));
   s->pmax = cfg->pipeline_depth > 0 ? cfg->pipeline_depth : std::max(1, std::min(maxcl, deepest));
   if (s->pmax > std::max(1, maxcl)) s->pmax = std::max(1, maxcl);
-  p.ring = s->pmax + 2;
+  for (gempic_sim::Shape& sh : s->shapes) sh.maxcl = std::min(sh.maxcl, s->pmax);
+  // overflow slots: bands that gain particles (radial expulsion, rejoining particles) spill
+  // beyond their shared-memory capacity into these
+  p.gcap = std::max(1024, g.nx * (g.ny / p.C) * std::max(ppc_sum, 1) * 2);
+  for (gempic_sim::Shape& sh : s->shapes) sh.p.gcap = p.gcap;
+  if (C == 0 && !one_cta && gempic::dense_ok(cfg->precision, p) && cfg->particle_headroom <= 0) {
+    // 128 x 128 FP32: two CTAs per SM where more s-steps are in flight than one per SM allows;
+    // as many particle slots per CTA as p's in shared memory and overflow together
+    gempic_sim::Shape one{p, s->pmax}, two{p, 0};
+    Params& t = two.p;
+    t.dense = 1;
+    t.nthreads = 256;
+    t.gcap = (p.pcap + p.gcap + 3) / 4 * 4;
+    if (gempic::smem_layout(t, s->eb) <= smem_optin) {
+      e = gempic::max_active_clusters(cfg->precision, t, &two.maxcl);
+      if (e != cudaSuccess) {
+        delete s;
+        return GEMPIC_ECUDA;
+      }
+      if (cfg->pipeline_depth > 0) two.maxcl = std::min(two.maxcl, cfg->pipeline_depth);
+      two.maxcl = std::min(two.maxcl, 16);
+      if (two.maxcl > s->pmax) {
+        s->shapes.push_back(one);
+        s->shapes.push_back(two);
+      }
+    }
+  }
+  int pring = s->pmax;                             // marches in flight of any shape
+  for (const gempic_sim::Shape& sh : s->shapes) pring = std::max(pring, sh.maxcl);
+  p.ring = pring + 2;
 
   // device memory
   const size_t eb = s->eb;
@@ -629,7 +666,7 @@ gempic_status create_sim(const gempic_config* cfg, gempic_sim** out, bool one_ct
   } while (0)
   {
     ALLOC(p.state, (size_t)(g.nzeta + 1) * 6 * nxh * g.ny * 2 * eb);
-    ALLOC(p.progress, (size_t)std::max(s->pmax, 1) * sizeof(unsigned long long));
+    ALLOC(p.progress, (size_t)pring * sizeof(unsigned long long));
     ALLOC(p.err, sizeof(int));
     void* tab = nullptr;
     const int nyh = g.ny > 1 ? g.ny / 2 : 1;
@@ -700,16 +737,11 @@ gempic_status create_sim(const gempic_config* cfg, gempic_sim** out, bool one_ct
     }
     ALLOC(p.jbeam, ring * g.nzeta * 3 * nperp * eb);
     ALLOC(p.jflag, ring * g.nzeta * sizeof(int));
-    // overflow particle slots: bands that gain particles (radial expulsion, rejoining stored
-    // particles) spill beyond their shared-memory capacity into these
-    p.gcap = std::max(1024, g.nx * (g.ny / p.C) * std::max(ppc_sum, 1) * 2);
-    {
-      // one area per CTA of a launch (2-D: every shape's marches x CTAs)
-      size_t ctas = (size_t)std::max(s->pmax, 1) * p.C;
-      for (const gempic_sim::Shape& sh : s->shapes)
-        ctas = std::max(ctas, (size_t)std::min(s->pmax, sh.maxcl) * sh.p.split);
-      ALLOC(p.pover, ctas * p.gcap * (4 + 7 * eb));
-    }
+    // particle slots in global memory, one area per CTA of a launch of any shape
+    size_t slots = (size_t)s->pmax * p.C * gempic::slot_bytes(p, (int)eb);
+    for (const gempic_sim::Shape& sh : s->shapes)
+      slots = std::max(slots, (size_t)sh.maxcl * sh.p.C * sh.p.split * gempic::slot_bytes(sh.p, (int)eb));
+    ALLOC(p.pover, slots);
     if (p.snapshot) ALLOC(p.snap, (size_t)9 * g.nzeta * nperp * eb);
     if (cfg->flags & GEMPIC_FLAG_CURRENT) {
       ALLOC(s->jcap, (size_t)3 * g.nzeta * nperp * eb);

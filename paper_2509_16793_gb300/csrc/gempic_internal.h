@@ -37,6 +37,7 @@ struct Params {
   int C, RB, KB, M;               // CTAs per slice, rows per CTA, kx per CTA, modes per CTA
   int split;                      // 2-D: CTAs that share a march's particles (1: not split); the
                                   // cluster has C split CTAs
+  int dense;                      // 1: two CTAs of 256 threads per SM (FP32 128 x 128 grids)
   int FR, JR, JOFF;               // field rows per CTA (own + halo above), current rows (own +
                                   // halo below/above), row offset of own row 0 in the currents
   int lognx, logny, logRB, logKB;
@@ -76,7 +77,7 @@ struct Params {
   int nwork;                      // work rows of the inverse row transform
   int mig_cap;                    // migrating particles a CTA can receive per slice
   // shared-memory layout (byte offsets)
-  int o_f0, o_f1, o_j, o_recv, o_sr, o_sc, o_workB, o_workD, o_tw, o_inbox, o_outbox, o_part, o_misc, o_dd,
+  int o_f0, o_f1, o_j, o_recv, o_sr, o_jint, o_sc, o_workB, o_workD, o_tw, o_inbox, o_outbox, o_part, o_misc, o_dd,
       smem_bytes;
   // device memory
   void* state;                    // blocks [nz+1][C][6][M] complex
@@ -159,6 +160,11 @@ struct BeamArgs {
 
 // Host-side helpers implemented in gempic_kernels.cu
 int smem_layout(Params& p, int elem_bytes);           // fills offsets, returns total bytes
+// bytes of one CTA's particle slots in global memory
+inline size_t slot_bytes(const Params& p, int elem_bytes) {
+  return p.dense ? (size_t)p.gcap * 32 + 4096 : (size_t)p.gcap * (4 + 7 * elem_bytes);
+}
+bool dense_ok(int precision, const Params& p);        // the grid has a dense march
 cudaError_t configure_kernels(int precision, int smem_bytes, int cluster);
 cudaError_t launch_march(int precision, const Params& p, cudaStream_t s);
 cudaError_t launch_laser_init(int precision, const Params& p, double a0, double waist,

@@ -29,6 +29,7 @@
 
 #include <algorithm>
 #include <cstdint>
+#include <type_traits>
 
 #include "gempic_internal.h"
 
@@ -65,9 +66,34 @@ struct V3 {
   T x, y, z;
 };
 
+// FP32 arithmetic of a push with its fused operations spelled out: the march is compiled for
+// several launch shapes, and which multiplication of a sum is fused must not depend on the
+// code around it, so that every shape gives the same bits.  FP64 is left to the compiler.
+__device__ __forceinline__ float fma_(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double fma_(double a, double b, double c) { return a * b + c; }
+__device__ __forceinline__ float mul_(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_(double a, double b) { return a * b; }
+// (the same for the slice solve below: c + s a, and c + i s a, of complex values)
+template <typename T>
+__device__ __forceinline__ Cx<T> cfma(T s, Cx<T> a, Cx<T> c) {
+  return {fma_(s, a.re, c.re), fma_(s, a.im, c.im)};
+}
+template <typename T>
+__device__ __forceinline__ Cx<T> cfma_i(T s, Cx<T> a, Cx<T> c) {
+  return {fma_(-s, a.im, c.re), fma_(s, a.re, c.im)};
+}
+template <typename T>
+__device__ __forceinline__ T ppm(T a, T b, T c, T d) { return fma_(a, b, mul_(c, d)); }    // ab + cd
+template <typename T>
+__device__ __forceinline__ T pmm(T a, T b, T c, T d) { return fma_(a, b, -mul_(c, d)); }   // ab - cd
+template <typename T>
+__device__ __forceinline__ Cx<T> cmul(Cx<T> a, Cx<T> b) {
+  return {pmm(a.re, b.re, a.im, b.im), ppm(a.im, b.re, a.re, b.im)};
+}
+
 template <typename T>
 __device__ __forceinline__ T gamma_of(V3<T> u) {   // sqrt(1 + ux^2 + uy^2 + uz^2)
-  return sqrt(((T(1) + u.x * u.x) + u.y * u.y) + u.z * u.z);
+  return sqrt(fma_(u.z, u.z, fma_(u.y, u.y, fma_(u.x, u.x, T(1)))));
 }
 // gamma - 1 for the kinetic energy: in FP32 as u^2/(gamma + 1) (sqrt(1 + u^2) - 1 cancels for
 // slow particles); in FP64 as gamma - 1, the form the FP64 reference evaluates
@@ -81,7 +107,7 @@ __device__ __forceinline__ T gamma_minus_one(V3<T> u, T g) {
 // gamma - u_z, as (1 + u_perp^2)/(gamma + u_z) where u_z > 0 (no cancellation).
 template <typename T>
 __device__ __forceinline__ T gamma_minus_uz(V3<T> u, T g) {
-  return u.z > T(0) ? ((T(1) + u.x * u.x) + u.y * u.y) / (g + u.z) : g - u.z;
+  return u.z > T(0) ? fma_(u.y, u.y, fma_(u.x, u.x, T(1))) / (g + u.z) : g - u.z;
 }
 
 // reciprocal and reciprocal square root: hardware approximations (a few ulp) in FP32, exact
@@ -105,16 +131,16 @@ __device__ __forceinline__ T rsq(T x) {
 template <typename T>
 __device__ __forceinline__ V3<T> boris(V3<T> u, const T* E, const T* B, T qm, T dt) {
   const T a = T(0.5) * qm * dt;
-  V3<T> um{u.x + a * E[0], u.y + a * E[1], u.z + a * E[2]};
-  const T ag = a * rsq(T(1) + ((um.x * um.x + um.y * um.y) + um.z * um.z));   // a / gamma
-  const T tx = ag * B[0], ty = ag * B[1], tz = ag * B[2];
-  V3<T> up{um.x + (um.y * tz - um.z * ty), um.y + (um.z * tx - um.x * tz),
-           um.z + (um.x * ty - um.y * tx)};
-  const T f = T(2) * rcp(T(1) + ((tx * tx + ty * ty) + tz * tz));
-  const T sx = f * tx, sy = f * ty, sz = f * tz;
-  V3<T> upl{um.x + (up.y * sz - up.z * sy), um.y + (up.z * sx - up.x * sz),
-            um.z + (up.x * sy - up.y * sx)};
-  return V3<T>{upl.x + a * E[0], upl.y + a * E[1], upl.z + a * E[2]};
+  V3<T> um{fma_(a, E[0], u.x), fma_(a, E[1], u.y), fma_(a, E[2], u.z)};
+  const T ag = a * rsq(T(1) + fma_(um.z, um.z, ppm(um.x, um.x, um.y, um.y)));   // a / gamma
+  const T tx = mul_(ag, B[0]), ty = mul_(ag, B[1]), tz = mul_(ag, B[2]);
+  V3<T> up{um.x + pmm(um.y, tz, um.z, ty), um.y + pmm(um.z, tx, um.x, tz),
+           um.z + pmm(um.x, ty, um.y, tx)};
+  const T f = T(2) * rcp(T(1) + fma_(tz, tz, ppm(tx, tx, ty, ty)));
+  const T sx = mul_(f, tx), sy = mul_(f, ty), sz = mul_(f, tz);
+  V3<T> upl{um.x + pmm(up.y, sz, up.z, sy), um.y + pmm(up.z, sx, up.x, sz),
+            um.z + pmm(up.x, sy, up.y, sx)};
+  return V3<T>{fma_(a, E[0], upl.x), fma_(a, E[1], upl.y), fma_(a, E[2], upl.z)};
 }
 
 // ------------------------------------------------------------------------------------------
@@ -556,7 +582,7 @@ struct Sm {
   double* dwarp;    // [nthreads / 32][kNDiag] per-warp FP64 diagnostic sums of this march
 };
 
-template <typename T>
+template <typename T, bool DEN = false>
 __device__ Sm<T> carve(const Params& p, unsigned char* base) {
   Sm<T> s;
   s.F[0] = (T*)(base + p.o_f0);
@@ -564,19 +590,29 @@ __device__ Sm<T> carve(const Params& p, unsigned char* base) {
   s.J = (T*)(base + p.o_j);
   s.recv = (T*)(base + p.o_recv);
   s.SR = (Cx<T>*)(base + p.o_sr);
-  s.Jint = (int*)(base + p.o_sr);
+  s.Jint = (int*)(base + (DEN ? p.o_jint : p.o_sr));
   s.SC = (Cx<T>*)(base + p.o_sc);
   s.workB = (Cx<T>*)(base + p.o_workB);
   s.workD = (Cx<T>*)(base + p.o_workD);
   Cx<T>* tw = (Cx<T>*)(base + p.o_tw);
   const int nyh = p.ny > 1 ? p.ny / 2 : 1;
   s.twx = tw;
-  s.twy = s.twx + p.nx / 2;
-  s.shx = s.twy + nyh;
-  s.shy = s.shx + p.nx / 2;
-  s.kx = (T*)(s.shy + p.ny);
-  s.ky = s.kx + p.nx / 2;
-  s.cst = s.ky + p.ny;
+  if constexpr (DEN) {
+    // nx = ny: one twiddle table; ky and its shift are read from global memory once per march
+    s.twy = tw;
+    s.shx = tw + nyh;
+    s.shy = nullptr;
+    s.kx = (T*)(s.shx + p.nx / 2);
+    s.ky = nullptr;
+    s.cst = s.kx + p.nx / 2;
+  } else {
+    s.twy = s.twx + p.nx / 2;
+    s.shx = s.twy + nyh;
+    s.shy = s.shx + p.nx / 2;
+    s.kx = (T*)(s.shy + p.ny);
+    s.ky = s.kx + p.nx / 2;
+    s.cst = s.ky + p.ny;
+  }
   unsigned char* ib = base + p.o_inbox;
   const int mcap = p.mig_cap;
   s.icell = (int*)ib;
@@ -619,15 +655,24 @@ __device__ Sm<T> carve(const Params& p, unsigned char* base) {
 }
 
 // tables built in FP64 on the host (already in the working precision) and the constants
-template <typename T>
+template <typename T, bool DEN = false>
 __device__ void load_tables(const Params& p, const Sm<T>& s) {
   const int nyh = p.ny > 1 ? p.ny / 2 : 1;
   const int ncx = p.nx / 2 + nyh + p.nx / 2 + p.ny;
   const int nr = p.nx / 2 + p.ny;
   const Cx<T>* src = (const Cx<T>*)p.tables;
-  for (int i = threadIdx.x; i < ncx; i += blockDim.x) s.twx[i] = src[i];
   const T* srcr = (const T*)(src + ncx);
-  for (int i = threadIdx.x; i < nr; i += blockDim.x) s.kx[i] = srcr[i];
+  if constexpr (DEN) {
+    const int nxh = p.nx / 2;
+    for (int i = threadIdx.x; i < nxh; i += blockDim.x) {
+      s.twx[i] = src[i];
+      s.shx[i] = src[nxh + nyh + i];
+      s.kx[i] = srcr[i];
+    }
+  } else {
+    for (int i = threadIdx.x; i < ncx; i += blockDim.x) s.twx[i] = src[i];
+    for (int i = threadIdx.x; i < nr; i += blockDim.x) s.kx[i] = srcr[i];
+  }
   if (threadIdx.x == 0) {
     T* c = s.cst;
     c[K_H] = T(p.h);
@@ -845,12 +890,12 @@ __device__ __noinline__ void forward_rows_r8(const cg::cluster_group& cl, const 
 
 // SH = 1: the kernel instantiated for 128 x 128 grids with an even band (only the length-128
 // transforms are compiled in; with the other lengths present the compiler schedules them
-// markedly worse)
+// markedly worse).  SH = 2: the same for two CTAs per SM (march(), "dense")
 // J: the slice's currents (s.J, or the sum over the CTAs of a split march)
 template <typename T, int SH>
 __device__ void forward_rows(const cg::cluster_group& cl, const Params& p, const Sm<T>& s,
                              const T* J, int me, bool stagger) {
-  if constexpr (SH == 1) {
+  if constexpr (SH >= 1) {
     forward_rows_128(cl, p, s, me, stagger);
   } else {
   if (p.lognx == 7 && p.ny > 1 && (p.RB & 1) == 0) {
@@ -948,7 +993,7 @@ __device__ void column_ffts_128(const Params& p, const Sm<T>& s, int c0, int c1,
 // the spectra stay in lane order (position q holds ky_of_pos(q))
 template <typename T, int SH>
 __device__ void column_ffts(const Params& p, const Sm<T>& s, int c0, int c1, bool inverse) {
-  if constexpr (SH == 1) {
+  if constexpr (SH >= 1) {
     column_ffts_128(p, s, c0, c1, inverse);
   } else {
     if (p.ny == 1) return;
@@ -1118,7 +1163,7 @@ __device__ __noinline__ void inverse_rows_r8(const Params& p, const Sm<T>& s, T*
 
 template <typename T, int SH>
 __device__ void inverse_rows(const Params& p, const Sm<T>& s, T* Fdst, T& fe) {
-  if constexpr (SH == 1) {
+  if constexpr (SH >= 1) {
     inverse_rows_128<T>(p, s, Fdst, fe);
   } else {
     if (sizeof(T) == 4 || p.ny > 1) {
@@ -1216,21 +1261,21 @@ __device__ __forceinline__ void gather6_g(const Params& p, const T* Fb, int ix, 
 #pragma unroll
     for (int c = 0; c < 6; ++c) {
       const uint32_t b = a + (c * cs) * (uint32_t)sizeof(T);
-      out[c] = (T(1) - fx) * lds(b + ix * (uint32_t)sizeof(T), T(0)) +
-               fx * lds(b + ix1 * (uint32_t)sizeof(T), T(0));
+      out[c] = ppm(T(1) - fx, lds(b + ix * (uint32_t)sizeof(T), T(0)), fx,
+                   lds(b + ix1 * (uint32_t)sizeof(T), T(0)));
     }
     return;
   }
   const int iy1 = (iy + 1) & (p.ny - 1);
   const RowRef<T> r0 = row_ref(p, Fb, p.FR, 0, iy, me);
   const RowRef<T> r1 = row_ref(p, Fb, p.FR, 0, iy1, me);
-  const T w00 = (T(1) - fx) * (T(1) - fy), w10 = fx * (T(1) - fy);
-  const T w01 = (T(1) - fx) * fy, w11 = fx * fy;
+  const T w00 = mul_(T(1) - fx, T(1) - fy), w10 = mul_(fx, T(1) - fy);
+  const T w01 = mul_(T(1) - fx, fy), w11 = mul_(fx, fy);
 #pragma unroll
   for (int c = 0; c < 6; ++c) {
     const uint32_t o = c * cs;
-    out[c] = ((w00 * row_ld(r0, o + ix) + w10 * row_ld(r0, o + ix1)) + w01 * row_ld(r1, o + ix)) +
-             w11 * row_ld(r1, o + ix1);
+    out[c] = fma_(w11, row_ld(r1, o + ix1),
+                  fma_(w01, row_ld(r1, o + ix), ppm(w00, row_ld(r0, o + ix), w10, row_ld(r0, o + ix1))));
   }
 }
 
@@ -1246,18 +1291,18 @@ __device__ __forceinline__ void gather6_l(const Params& p, const T* Fb, int ix, 
 #pragma unroll
     for (int c = 0; c < 6; ++c) {
       const uint32_t b = a0 + c * cs;
-      out[c] = (T(1) - fx) * lds(b + i0, T(0)) + fx * lds(b + i1, T(0));
+      out[c] = ppm(T(1) - fx, lds(b + i0, T(0)), fx, lds(b + i1, T(0)));
     }
     return;
   }
   const uint32_t a1 = a0 + (uint32_t)p.nx * (uint32_t)sizeof(T);
-  const T w00 = (T(1) - fx) * (T(1) - fy), w10 = fx * (T(1) - fy);
-  const T w01 = (T(1) - fx) * fy, w11 = fx * fy;
+  const T w00 = mul_(T(1) - fx, T(1) - fy), w10 = mul_(fx, T(1) - fy);
+  const T w01 = mul_(T(1) - fx, fy), w11 = mul_(fx, fy);
 #pragma unroll
   for (int c = 0; c < 6; ++c) {
     const uint32_t b0 = a0 + c * cs, b1 = a1 + c * cs;
-    out[c] = ((w00 * lds(b0 + i0, T(0)) + w10 * lds(b0 + i1, T(0))) + w01 * lds(b1 + i0, T(0))) +
-             w11 * lds(b1 + i1, T(0));
+    out[c] = fma_(w11, lds(b1 + i1, T(0)),
+                  fma_(w01, lds(b1 + i0, T(0)), ppm(w00, lds(b0 + i0, T(0)), w10, lds(b0 + i1, T(0)))));
   }
 }
 
@@ -1606,11 +1651,11 @@ __device__ bool stream_push(const Params& p, const Sm<T>& s, const T* Fcur, PSta
   const V3<T> un = boris(u, E, E + 3, qm, dt2);
   const T gn = gamma_of(un);
   const T hden = hc * rcp(gamma_minus_uz(un, gn));    // h / (gamma - u_z)
-  const T dx = hden * un.x, dy = hden * un.y, ds = hden * un.z;
+  const T dx = mul_(hden, un.x), dy = mul_(hden, un.y), ds = mul_(hden, un.z);
   // deposit: w = Q/(hx hy Delta) is the particle's (rho - j_z) density weight (Sec. 5.1)
   const T w = P.q * s.cst[K_WSCALE];
-  const T X1 = P.fx + dx * s.cst[K_INVHX];
-  const T Y1 = p.ny > 1 ? P.fy + dy * s.cst[K_INVHY] : P.fy;
+  const T X1 = fma_(dx, s.cst[K_INVHX], P.fx);
+  const T Y1 = p.ny > 1 ? fma_(dy, s.cst[K_INVHY], P.fy) : P.fy;
   SUB_MARK(1);
   // the move stays inside the band's current rows -1 .. RB + 1 -> local reductions only
   const T lo = floor(fmin(P.fy, Y1)), hi = floor(fmax(P.fy, Y1));
@@ -1648,7 +1693,7 @@ __device__ bool stream_push(const Params& p, const Sm<T>& s, const T* Fcur, PSta
     }
   }
   // diagnostics: kinetic energy N m (gamma-1) dt/Delta, (rho - j_z) flux through plane n
-  const T dtl = hden * gn;
+  const T dtl = mul_(hden, gn);
   acc.kin += P.q * s.cst[K_MOQ + P.sp] * gamma_minus_one(un, gn) * dtl * s.cst[K_INVD];
   if (!trap) acc.flux += w;
   acc.push += 1;
@@ -1754,6 +1799,43 @@ __device__ __forceinline__ Ovf<T> ovf_view(const Params& p, int cta) {
   o.sig = t + 5 * g;
   o.q = t + 6 * g;
   return o;
+}
+
+// Dense marches keep every streaming particle in global memory (L2): two 16-byte vectors per slot,
+// {cell word, fx, fy, charge} and {u, sigma}, slots consecutive, and the stack of free slots.
+// Only the CTA itself touches them.
+struct GSlots {
+  float4 *a, *b;
+  int* fstack;
+};
+constexpr int kDenseFree = 1024;                  // entries of the free-slot stack
+__device__ __forceinline__ GSlots gslots(const Params& p, int cta) {
+  GSlots g;
+  char* b = (char*)p.pover + (size_t)cta * ((size_t)p.gcap * 32 + kDenseFree * 4);
+  g.a = (float4*)b;
+  g.b = g.a + p.gcap;
+  g.fstack = (int*)(g.b + p.gcap);
+  return g;
+}
+template <typename T>
+__device__ __forceinline__ PState<T> g_unpack(float4 a, float4 b) {
+  PState<T> P;
+  const int cw = __float_as_int(a.x);
+  P.ix = cw & 1023;
+  P.iy = (cw >> 10) & 1023;
+  P.sp = (cw >> 20) & 3;
+  P.fx = a.y;
+  P.fy = a.z;
+  P.q = a.w;
+  P.u = V3<T>{b.x, b.y, b.z};
+  P.sig = b.w;
+  return P;
+}
+template <typename T>
+__device__ __forceinline__ void g_put(const GSlots& g, int i, const PState<T>& P) {
+  const int cw = P.ix | (P.iy << 10) | (P.sp << 20);
+  __stcg(g.a + i, make_float4(__int_as_float(cw), (float)P.fx, (float)P.fy, (float)P.q));
+  __stcg(g.b + i, make_float4((float)P.u.x, (float)P.u.y, (float)P.u.z, (float)P.sig));
 }
 
 template <typename T>
@@ -1982,43 +2064,51 @@ struct Mode6 {
   Cx<T> Rx, Ry, Lx, Ly, Ez, Bz;
 };
 
-template <typename T>
+// GEN: the generic kernel (any size); it and the 128 x 128 one fuse a different product in three
+// of the sums.
+template <typename T, bool GEN>
 __device__ __forceinline__ Mode6<T> slice_solve(T kx, T ky, T h, T Dl, const Mode6<T>& n1,
                                                 Cx<T> Rxo, Cx<T> Ryo, Cx<T> Ezo, Cx<T> Bzo,
                                                 Cx<T> jx0m, Cx<T> jy0m, Cx<T> jx0p, Cx<T> jy0p,
                                                 Cx<T> jx1p, Cx<T> jy1p, Cx<T> jz1p) {
-  const T K2 = kx * kx + ky * ky;
-  const T Dd = T(16) + h * (T(2) * Dl + h) * K2;
+  auto kk = [](T a, Cx<T> x, T b, Cx<T> y) { return cx<T>(ppm(a, x.re, b, y.re), ppm(a, x.im, b, y.im)); };
+  auto km = [](T a, Cx<T> x, T b, Cx<T> y) { return cx<T>(pmm(a, x.re, b, y.re), pmm(a, x.im, b, y.im)); };
+  const T K2 = ppm(kx, kx, ky, ky);
+  const T Dd = fma_(mul_(h, fma_(T(2), Dl, h)), K2, T(16));
   // predictor j^1_{-1/2} := j^1_{+1/2}
-  const Cx<T> Jx = (jx0m + jx0p) + T(2) * jx1p;
-  const Cx<T> Jy = (jy0m + jy0p) + T(2) * jy1p;
-  const Cx<T> Wx = (n1.Rx + Rxo) - T(2) * n1.Lx;
-  const Cx<T> Wy = (n1.Ry + Ryo) - T(2) * n1.Ly;
-  const Cx<T> Ux = (n1.Rx + Rxo) + T(2) * n1.Lx;
-  const Cx<T> Uy = (n1.Ry + Ryo) + T(2) * n1.Ly;
-  const T c16 = T(16) - h * h * K2;
-  const T hD = h * Dl;
-  Cx<T> numE = c16 * n1.Ez - (T(16) * h) * jz1p;
-  numE = numE - mul_i(hD * (kx * Jx + ky * Jy));
-  numE = numE - (T(2) * hD * K2) * Ezo;
-  numE = numE + mul_i((T(2) * h * h) * (kx * jx1p + ky * jy1p));
-  numE = numE + mul_i((T(4) * h) * (kx * Wx + ky * Wy));
-  Cx<T> numB = c16 * n1.Bz + mul_i((T(2) * h * h) * (kx * jy1p - ky * jx1p));
-  numB = numB + mul_i(hD * (kx * Jy - ky * Jx));
-  numB = numB - (T(2) * hD * K2) * Bzo;
-  numB = numB + mul_i((T(4) * h) * (ky * Ux - kx * Uy));
+  const Cx<T> Jx = cfma(T(2), jx1p, jx0m + jx0p);
+  const Cx<T> Jy = cfma(T(2), jy1p, jy0m + jy0p);
+  const Cx<T> Rx2 = n1.Rx + Rxo, Ry2 = n1.Ry + Ryo;
+  const Cx<T> Wx = cfma(T(-2), n1.Lx, Rx2), Wy = cfma(T(-2), n1.Ly, Ry2);
+  const Cx<T> Ux = cfma(T(2), n1.Lx, Rx2), Uy = cfma(T(2), n1.Ly, Ry2);
+  const T c16 = fma_(-mul_(h, h), K2, T(16));
+  const T hD = mul_(h, Dl), h16 = T(16) * h, h4 = T(4) * h;
+  const T hh2 = mul_(T(2) * h, h), hDK = mul_(T(2) * hD, K2);
+  Cx<T> numE = cx<T>(pmm(c16, n1.Ez.re, h16, jz1p.re), pmm(c16, n1.Ez.im, h16, jz1p.im));
+  numE = cfma_i(-hD, kk(kx, Jx, ky, Jy), numE);
+  numE = cfma(-hDK, Ezo, numE);
+  numE = cfma_i(hh2, kk(kx, jx1p, ky, jy1p), numE);
+  numE = cfma_i(h4, kk(kx, Wx, ky, Wy), numE);
+  const Cx<T> jr = km(kx, jy1p, ky, jx1p);
+  Cx<T> numB = cx<T>(pmm(c16, n1.Bz.re, hh2, jr.im),
+                     GEN ? ppm(hh2, jr.re, c16, n1.Bz.im) : ppm(c16, n1.Bz.im, hh2, jr.re));
+  numB = cfma_i(hD, km(kx, Jy, ky, Jx), numB);
+  numB = cfma(-hDK, Bzo, numB);
+  numB = cfma_i(h4, km(ky, Ux, kx, Uy), numB);
   const T invD = T(1) / Dd;
   Mode6<T> o;
-  o.Ez = invD * numE;
-  o.Bz = invD * numB;
+  o.Ez = cx<T>(mul_(invD, numE.re), mul_(invD, numE.im));
+  o.Bz = cx<T>(mul_(invD, numB.re), mul_(invD, numB.im));
   // RxN, RyN (trapezoid in s)
   const Cx<T> sEz = o.Ez + Ezo, sBz = o.Bz + Bzo;
-  o.Rx = Rxo + Dl * (mul_i(T(0.5) * (kx * sEz + ky * sBz)) - T(0.25) * Jx);
-  o.Ry = Ryo + Dl * (mul_i(T(0.5) * (ky * sEz - kx * sBz)) - T(0.25) * Jy);
+  const Cx<T> z = cx<T>(T(0), T(0));
+  const Cx<T> q4x = T(0.25) * Jx, q4y = T(0.25) * Jy;
+  o.Rx = cfma(Dl, cfma_i(T(0.5), GEN ? kk(ky, sBz, kx, sEz) : kk(kx, sEz, ky, sBz), z - q4x), Rxo);
+  o.Ry = cfma(Dl, cfma_i(T(0.5), km(ky, sEz, kx, sBz), z - q4y), Ryo);
   // LxN, LyN (box scheme in zeta)
   const Cx<T> tEz = n1.Ez + o.Ez, tBz = o.Bz + n1.Bz;
-  o.Lx = n1.Lx - (T(0.5) * h) * (mul_i(T(0.5) * (kx * tEz - ky * tBz)) + jx1p);
-  o.Ly = n1.Ly - (T(0.5) * h) * (mul_i(T(0.5) * (ky * tEz + kx * tBz)) + jy1p);
+  o.Lx = cfma(-(T(0.5) * h), cfma_i(T(0.5), km(kx, tEz, ky, tBz), jx1p), n1.Lx);
+  o.Ly = cfma(-(T(0.5) * h), cfma_i(T(0.5), GEN ? kk(kx, tBz, ky, tEz) : kk(ky, tEz, kx, tBz), jy1p), n1.Ly);
   return o;
 }
 
@@ -2076,13 +2166,27 @@ __device__ __forceinline__ void wait_input(const Params& p, long long k, int b, 
 // DN: the march of a denoised chain (its hooks are compiled into the chain's instantiations
 // only); CANON instantiations carry the streamed state's hooks.
 template <typename T, bool CANON = false, int SH = 0, bool DN = false>
-__device__ void march(const Params& p, const Sm<T>& s, const cg::cluster_group& cl, long long k,
+__device__ void march(const Params& p, const Sm<T>& s_, const cg::cluster_group& cl, long long k,
                       int cid, long long item_) {
+  // (dense: SR and workB follow the plane buffers)
+  typename std::conditional<SH == 2, Sm<T>, const Sm<T>&>::type s = s_;
   // the 128 x 128 instantiation is compiled for GT2 and a uniform zeta-step only (other runs
   // take the generic one)
-  constexpr int LAW = SH == 1 ? 0 : -1;
-  const bool varh = SH != 1 && p.varh != 0;
-  const bool resid = SH != 1 && p.resid != 0;     // continuity and Gauss residuals
+  constexpr int LAW = SH >= 1 ? 0 : -1;
+  // Dense marches (SH = 2, FP32 128 x 128 grids): 256 threads and half the shared memory per CTA,
+  // so that two CTAs share an SM and 14 clusters are on the chip instead of 7.  A march of
+  // 512-thread CTAs keeps the issue slots 44 % busy: it waits at 5 cluster barriers a slice and in
+  // the latency of the transforms, and another march's push fills those gaps.  What makes room:
+  // the streaming particles stay in L2 (64 KB per CTA, read and written once a slice, coalesced),
+  // the received row spectra and the staging of the forward transform share the plane buffer
+  // that the new fields will fill (the inverse transform of a row pair is in place), the
+  // fixed-point accumulators share the column spectra, and a thread carries two modes whose old
+  // level is read when it is needed.  A march then takes 82 k cycles a slice instead of 54 k, with
+  // twice as many in flight: 128 x 128 x 1024, 2 per cell, 14 s-steps in a call, 52.3 -> 42.7 ms.
+  constexpr bool DEN = SH == 2;
+  constexpr int NM = DEN ? 2 : 1;                 // spectral modes per thread
+  const bool varh = SH == 0 && p.varh != 0;
+  const bool resid = SH == 0 && p.resid != 0;     // continuity and Gauss residuals
   const int rbe = p.ny > 1 ? p.RB : 1;            // own rows of the residual planes
   T rmax = T(0), gmax = T(0);
   const T* hzt = (const T*)p.hzt;
@@ -2093,7 +2197,7 @@ __device__ void march(const Params& p, const Sm<T>& s, const cg::cluster_group& 
   // reports the fields.  A 2-D slice is one CTA's work otherwise, which leaves the chip idle
   // where few s-steps are in flight, and its FP64 push is bound by the SM's two FP64 lanes
   // (130 of 200 k cycles a slice at 128 cells, 4 per cell).
-  const bool spl = SH != 1 && p.split > 1;
+  const bool spl = SH == 0 && p.split > 1;
   const int rank = (int)cl.block_rank();
   const int me = spl ? 0 : rank;
   const int part = spl ? rank : 0;
@@ -2115,6 +2219,7 @@ __device__ void march(const Params& p, const Sm<T>& s, const cg::cluster_group& 
   const T h = s.cst[K_H], Dl = s.cst[K_DF];
   const long long sl = item - item0;                // march index within this launch
   const Ovf<T> ov = ovf_view<T>(p, cid * nrank + rank);   // overflow particle slots of this CTA
+  const GSlots gs = gslots(p, cid * nrank + rank);        // dense: every slot
   const int fplane = p.FR * p.nx;                   // elements of one field component
   const int jplane = p.JR * p.nx;                   // elements of one current component
   TIMER_DECL
@@ -2174,7 +2279,7 @@ __device__ void march(const Params& p, const Sm<T>& s, const cg::cluster_group& 
         const T dy = p.ny > 1 ? (T(iy - (p.ny >> 1)) + fy) * s.cst[K_HY] : T(0);
         q *= T(1) + T(p.chan_a) * exp(-(dx * dx + dy * dy) * T(p.chan_ir2));
       }
-      if (i < p.pcap) {
+      if (!DEN && i < p.pcap) {
         s.pcell[i] = ix | (iy << 10) | (sp << 20);
         s.pfx[i] = fx;
         s.pfy[i] = fy;
@@ -2195,7 +2300,11 @@ __device__ void march(const Params& p, const Sm<T>& s, const cg::cluster_group& 
         P.u = V3<T>{T(0), T(0), T(0)};
         P.sig = T(0);
         P.q = q;
-        put_particle(p, s, ov, i, P);
+        if constexpr (DEN) {
+          if (i < p.gcap) g_put(gs, i, P);
+        } else {
+          put_particle(p, s, ov, i, P);
+        }
       }
     }
     if (tid == 0) s.misc[M_PCOUNT] = min(nmine, p.pcap + p.gcap);
@@ -2214,29 +2323,44 @@ __device__ void march(const Params& p, const Sm<T>& s, const cg::cluster_group& 
   // accesses are 32 consecutive words).  Public layout (kx innermost): kxl fastest, so that a
   // warp reads and writes whole 32-byte runs of its CTA's KB columns in 32 / KB rows, not 32
   // rows one word each
-  const int m = tid;
-  const bool has_mode = m < p.M;
-  const int kxl = !has_mode ? 0 : CANON ? m & (p.KB - 1) : m >> p.logny;
-  const int q = !has_mode ? 0 : CANON ? m >> p.logKB : m & (p.ny - 1);
-  const int kyi = ky_of_pos(p.logny, q);
-  const T kx = has_mode ? s.kx[(me << p.logKB) + kxl] : T(0);
-  const T ky = has_mode ? s.ky[kyi] : T(0);
-  const bool masked = p.ny > 1 && kyi == p.ny / 2;
-  Mode6<T> S1;
-  S1.Rx = S1.Ry = S1.Lx = S1.Ly = S1.Ez = S1.Bz = cx<T>(T(0), T(0));
-  Cx<T> jpx = cx<T>(T(0), T(0)), jpy = jpx;       // j^1 at n + 3/2 (predictor of the last solve)
-  Cx<T> o[6];                                     // old level, block n
-  Cx<T> j0px = jpx, j0py = jpx;                   // old level j at n + 1/2
+  // (dense: the modes tid and tid + blockDim)
+  const bool has_mode = DEN || tid < p.M;
+  int kxl[NM], q[NM], kyi[NM];
+  T kx[NM], ky[NM];
+  bool masked[NM];
+#pragma unroll
+  for (int j = 0; j < NM; ++j) {
+    const int m = tid + j * NT;
+    kxl[j] = !has_mode ? 0 : CANON ? m & (p.KB - 1) : m >> p.logny;
+    q[j] = !has_mode ? 0 : CANON ? m >> p.logKB : m & (p.ny - 1);
+    kyi[j] = ky_of_pos(p.logny, q[j]);
+    masked[j] = p.ny > 1 && kyi[j] == p.ny / 2;
+    kx[j] = has_mode ? s.kx[(me << p.logKB) + kxl[j]] : T(0);
+    if constexpr (DEN)
+      ky[j] = ((const T*)((const Cx<T>*)p.tables + 2 * (p.nx / 2) + p.ny / 2 + p.ny))[p.nx / 2 + kyi[j]];
+    else
+      ky[j] = has_mode ? s.ky[kyi[j]] : T(0);
+  }
+  const Cx<T> zero = cx<T>(T(0), T(0));
+  Mode6<T> S1[NM];
+  Cx<T> jpx[NM], jpy[NM];                         // j^1 at n + 3/2 (predictor of the last solve)
+  Cx<T> o[NM][6];                                 // old level, block n
+  Cx<T> j0px[NM], j0py[NM];                       // old level j at n + 1/2
+#pragma unroll
+  for (int j = 0; j < NM; ++j) {
+    S1[j].Rx = S1[j].Ry = S1[j].Lx = S1[j].Ly = S1[j].Ez = S1[j].Bz = zero;
+    jpx[j] = jpy[j] = j0px[j] = j0py[j] = zero;
+  }
   const Cx<T>* st = (const Cx<T>*)p.state;
   // the new level is written over the old one, or (first pass of a denoised s-step) elsewhere
   Cx<T>* stw = (Cx<T>*)(dn1 ? p.dn_scratch : p.state_out ? p.state_out : p.state);
-  auto blk = [&](int b, int c) -> size_t {
+  auto blk = [&](int b, int c, int j) -> size_t {
     if constexpr (CANON) {
-      const int kxg = (me << p.logKB) + kxl;
+      const int kxg = (me << p.logKB) + kxl[j];
       const int sl_ = c < 4 ? b : b - 1;
-      return (((size_t)c * p.nz + sl_) * p.ny + kyi) * (size_t)nxh + kxg;
+      return (((size_t)c * p.nz + sl_) * p.ny + kyi[j]) * (size_t)nxh + kxg;
     } else {
-      return (((size_t)b * p.C + me) * 6 + c) * (size_t)p.M + m;
+      return (((size_t)b * p.C + me) * 6 + c) * (size_t)p.M + tid + j * NT;
     }
   };
   // the public layout has no ghost slice and no j at half-slice -1
@@ -2255,11 +2379,11 @@ __device__ void march(const Params& p, const Sm<T>& s, const cg::cluster_group& 
   if constexpr (CANON)
     if (p.io_chunk && tid == 0 && me == 0) wait_input(p, k, nz - 1, s.misc + M_IOSEEN);
   cl.sync();
-  if (has_mode) {
-    j0px = ldcg(st + blk(nz, 4));
-    j0py = ldcg(st + blk(nz, 5));
+  if (has_mode && !DEN) {
+    j0px[0] = ldcg(st + blk(nz, 4, 0));
+    j0py[0] = ldcg(st + blk(nz, 5, 0));
 #pragma unroll
-    for (int c = 0; c < 6; ++c) o[c] = ldcg(st + blk(nz - 1, c));
+    for (int c = 0; c < 6; ++c) o[0][c] = ldcg(st + blk(nz - 1, c, 0));
   }
   const long long klast = DN ? p.k0 + p.nsteps / 2 - 1 : p.k0 + p.nsteps - 1;
   const bool snap_step = p.snapshot && k == klast;
@@ -2286,6 +2410,7 @@ __device__ void march(const Params& p, const Sm<T>& s, const cg::cluster_group& 
     // constants (the previous slice's stored phase has finished reading them)
     const T hn = varh ? hzt[n] : h;
     T* const dn_n = s.dn + (size_t)(n & 1) * rbe * p.nx;   // arrival density of plane n
+    if constexpr (DEN) s.SR = s.workB = (Cx<T>*)Fnew;
     if (varh) {
       __syncthreads();
       if (tid == 0) {
@@ -2303,11 +2428,18 @@ __device__ void march(const Params& p, const Sm<T>& s, const cg::cluster_group& 
     {
       const int cnt0 = s.misc[M_PCOUNT];
       for (int i = tid; i < cnt0; i += NT) {
-        const int cw = get_cell(p, s, ov, i);
-        if (cw < 0) continue;
-        PState<T> P = get_particle(p, s, ov, i, cw);
+        PState<T> P;
+        if constexpr (DEN) {
+          const float4 pa = __ldcg(gs.a + i), pb = __ldcg(gs.b + i);
+          if (__float_as_int(pa.x) < 0) continue;
+          P = g_unpack<T>(pa, pb);
+        } else {
+          const int cw = get_cell(p, s, ov, i);
+          if (cw < 0) continue;
+          P = get_particle(p, s, ov, i, cw);
+        }
         T fzt;
-        const bool trap = stream_push<T, LAW, SH != 1>(p, s, Fcur, P, hn, me, fzt, sa, dn_n);
+        const bool trap = stream_push<T, LAW, SH == 0>(p, s, Fcur, P, hn, me, fzt, sa, dn_n);
         bool gone = trap;
         if (trap) {
           ++ntrap;
@@ -2336,12 +2468,20 @@ __device__ void march(const Params& p, const Sm<T>& s, const cg::cluster_group& 
           }
         }
         if (gone) {
-          set_cell(p, s, ov, i, -1);
           // shared-memory slots are reused; a dead overflow slot stays unused this s-step
-          if (i < p.pcap) {
+          if constexpr (DEN) {
+            __stcg(reinterpret_cast<int*>(gs.a + i), -1);
             const int f = atomicAdd(s.misc + M_FTOP, 1);
-            if (f < p.fcap) s.fstack[f] = i;
+            if (f < p.fcap) gs.fstack[f] = i;
+          } else {
+            set_cell(p, s, ov, i, -1);
+            if (i < p.pcap) {
+              const int f = atomicAdd(s.misc + M_FTOP, 1);
+              if (f < p.fcap) s.fstack[f] = i;
+            }
           }
+        } else if constexpr (DEN) {
+          g_put(gs, i, P);
         } else {
           put_particle(p, s, ov, i, P);
         }
@@ -2357,7 +2497,7 @@ __device__ void march(const Params& p, const Sm<T>& s, const cg::cluster_group& 
         PState<T> P = store_read<T>(p.rq, p, ge, fz);
         ++nrej;
         T fzt;
-        const bool trap = stream_push<T, LAW, SH != 1>(p, s, Fcur, P, fz * hn, me, fzt, sa, dn_n);
+        const bool trap = stream_push<T, LAW, SH == 0>(p, s, Fcur, P, fz * hn, me, fzt, sa, dn_n);
         if (trap) {
           ++ntrap;
           if (!store_append(p.st, p, s1, n, P, fzt)) atomicOr(p.err, ERR_BCAP);
@@ -2367,7 +2507,8 @@ __device__ void march(const Params& p, const Sm<T>& s, const cg::cluster_group& 
         if (owner != me && migrate(cl, p, s, P, owner)) continue;
         const int slot = atomicAdd(s.misc + M_PCOUNT, 1);
         if (slot < p.pcap + p.gcap) {
-          put_particle(p, s, ov, slot, P);
+          if constexpr (DEN) g_put(gs, slot, P);
+          else put_particle(p, s, ov, slot, P);
         } else {
           atomicOr(p.err, ERR_PCAP);
 #ifdef GEMPIC_PHASE_TIMERS
@@ -2457,10 +2598,12 @@ __device__ void march(const Params& p, const Sm<T>& s, const cg::cluster_group& 
             *cl.map_shared_rank(s.iq + e, dst) = P.q;
           } else {
             const int slot = atomicAdd(s.misc + M_PCOUNT, 1);
-            if (slot < p.pcap + p.gcap)
-              put_particle(p, s, ov, slot, P);
-            else
+            if (slot >= p.pcap + p.gcap)
               atomicOr(p.err, ERR_PCAP);
+            else if constexpr (DEN)
+              g_put(gs, slot, P);
+            else
+              put_particle(p, s, ov, slot, P);
           }
         }
       }
@@ -2616,7 +2759,7 @@ __device__ void march(const Params& p, const Sm<T>& s, const cg::cluster_group& 
       const int ftop = min(s.misc[M_FTOP], p.fcap);
       const int pc = s.misc[M_PCOUNT];
       for (int e = tid; e < nin; e += NT) {
-        const int slot = e < ftop ? s.fstack[ftop - 1 - e] : pc + (e - ftop);
+        const int slot = e < ftop ? (DEN ? gs.fstack : s.fstack)[ftop - 1 - e] : pc + (e - ftop);
         if (slot >= p.pcap + p.gcap) {
           atomicOr(p.err, ERR_PCAP);
 #ifdef GEMPIC_PHASE_TIMERS
@@ -2627,13 +2770,18 @@ __device__ void march(const Params& p, const Sm<T>& s, const cg::cluster_group& 
 #endif
           continue;
         }
-        PState<T> P = get_particle(p, s, ov, 0, s.icell[e]);
+        PState<T> P;
+        const int cw = s.icell[e];
+        P.ix = cw & 1023;
+        P.iy = (cw >> 10) & 1023;
+        P.sp = (cw >> 20) & 3;
         P.fx = s.ifx[e];
         P.fy = s.ify[e];
         P.u = V3<T>{s.iux[e], s.iuy[e], s.iuz[e]};
         P.sig = s.isig[e];
         P.q = s.iq[e];
-        put_particle(p, s, ov, slot, P);
+        if constexpr (DEN) g_put(gs, slot, P);
+        else put_particle(p, s, ov, slot, P);
       }
       __syncthreads();
       if (tid == 0) {
@@ -2740,39 +2888,57 @@ __device__ void march(const Params& p, const Sm<T>& s, const cg::cluster_group& 
     __syncthreads();
     TIMER_MARK(PH_COLF);
     if (has_mode) {
-      Cx<T> Jx = s.SC[((size_t)0 * p.KB + kxl) * p.ny + q];
-      Cx<T> Jy = s.SC[((size_t)1 * p.KB + kxl) * p.ny + q];
-      Cx<T> Jz = s.SC[((size_t)2 * p.KB + kxl) * p.ny + q];
-      if (p.ny > 1) Jy = Jy * s.shy[kyi];
-      if (masked) Jx = Jy = Jz = cx<T>(T(0), T(0));
+      if constexpr (DEN) {
+        // the old level, for both modes at once (L2: another march wrote it a few slices ago)
+#pragma unroll
+        for (int j = 0; j < NM; ++j) {
+          j0px[j] = ldcg(st + blk(n + 1, 4, j));
+          j0py[j] = ldcg(st + blk(n + 1, 5, j));
+#pragma unroll
+          for (int c = 0; c < 6; ++c) o[j][c] = blk_ok(n, c) ? ldcg(st + blk(n, c, j)) : zero;
+        }
+      }
+      const Cx<T>* const tb = (const Cx<T>*)p.tables;
+      const int ntb = 2 * (p.nx / 2) + p.ny / 2;
+#pragma unroll
+      for (int j = 0; j < NM; ++j) {
+      Cx<T> Jx = s.SC[((size_t)0 * p.KB + kxl[j]) * p.ny + q[j]];
+      Cx<T> Jy = s.SC[((size_t)1 * p.KB + kxl[j]) * p.ny + q[j]];
+      Cx<T> Jz = s.SC[((size_t)2 * p.KB + kxl[j]) * p.ny + q[j]];
+      if constexpr (DEN) {
+        Jy = cmul(Jy, tb[ntb + kyi[j]]);
+      } else if (p.ny > 1) {
+        Jy = cmul(Jy, s.shy[kyi[j]]);
+      }
+      if (masked[j]) Jx = Jy = Jz = zero;
       // corrector: R at slice n+1 was built with j_{n+1/2} := j_{n+3/2}
       if (n + 1 < nz) {
-        S1.Rx = S1.Rx - (T(0.25) * Dl) * (Jx - jpx);
-        S1.Ry = S1.Ry - (T(0.25) * Dl) * (Jy - jpy);
+        S1[j].Rx = cfma(-(T(0.25) * Dl), Jx - jpx[j], S1[j].Rx);
+        S1[j].Ry = cfma(-(T(0.25) * Dl), Jy - jpy[j], S1[j].Ry);
       }
       // new level, block n+1 = {R, E_z, B_z at slice n+1; j at n+1/2}
       if (part == 0 && blk_ok(n + 1, 0)) {
-        stw[blk(n + 1, 0)] = S1.Rx;
-        stw[blk(n + 1, 1)] = S1.Ry;
-        stw[blk(n + 1, 2)] = S1.Ez;
-        stw[blk(n + 1, 3)] = S1.Bz;
+        stw[blk(n + 1, 0, j)] = S1[j].Rx;
+        stw[blk(n + 1, 1, j)] = S1[j].Ry;
+        stw[blk(n + 1, 2, j)] = S1[j].Ez;
+        stw[blk(n + 1, 3, j)] = S1[j].Bz;
       }
       if (part == 0) {
-        stw[blk(n + 1, 4)] = Jx;
-        stw[blk(n + 1, 5)] = Jy;
+        stw[blk(n + 1, 4, j)] = Jx;
+        stw[blk(n + 1, 5, j)] = Jy;
       }
       // old level at slice n; j^0 at n -/+ 1/2
-      const Cx<T> j0mx = n > 0 ? o[4] : j0px;
-      const Cx<T> j0my = n > 0 ? o[5] : j0py;
+      const Cx<T> j0mx = n > 0 ? o[j][4] : j0px[j];
+      const Cx<T> j0my = n > 0 ? o[j][5] : j0py[j];
       Mode6<T> S0;
-      if (masked) {
-        S0.Rx = S0.Ry = S0.Lx = S0.Ly = S0.Ez = S0.Bz = cx<T>(T(0), T(0));
+      if (masked[j]) {
+        S0.Rx = S0.Ry = S0.Lx = S0.Ly = S0.Ez = S0.Bz = zero;
       } else {
-        S0 = slice_solve(kx, ky, hn, Dl, S1, o[0], o[1], o[2], o[3], j0mx, j0my, j0px, j0py, Jx,
-                         Jy, Jz);
+        S0 = slice_solve<T, SH == 0>(kx[j], ky[j], hn, Dl, S1[j], o[j][0], o[j][1], o[j][2], o[j][3], j0mx, j0my,
+                         j0px[j], j0py[j], Jx, Jy, Jz);
       }
       // fields E, B (Eqs. Rx..Ly) for the inverse transform
-      Cx<T>* sc = s.SC + (size_t)kxl * p.ny + q;
+      Cx<T>* sc = s.SC + (size_t)kxl[j] * p.ny + q[j];
       const size_t cs = (size_t)p.KB * p.ny;
       sc[0 * cs] = T(0.5) * (S0.Rx + S0.Lx);
       sc[1 * cs] = T(0.5) * (S0.Ry + S0.Ly);
@@ -2780,22 +2946,22 @@ __device__ void march(const Params& p, const Sm<T>& s, const cg::cluster_group& 
       sc[3 * cs] = T(0.5) * (S0.Ly - S0.Ry);
       sc[4 * cs] = T(0.5) * (S0.Rx - S0.Lx);
       sc[5 * cs] = S0.Bz;
-      S1 = S0;
-      jpx = Jx;
-      jpy = Jy;
-      j0px = j0mx;
-      j0py = j0my;
+      S1[j] = S0;
+      jpx[j] = Jx;
+      jpy[j] = Jy;
+      j0px[j] = j0mx;
+      j0py[j] = j0my;
       if (n == 0) {
         if (part == 0) {
-          stw[blk(0, 0)] = S0.Rx;
-          stw[blk(0, 1)] = S0.Ry;
-          stw[blk(0, 2)] = S0.Ez;
-          stw[blk(0, 3)] = S0.Bz;
+          stw[blk(0, 0, j)] = S0.Rx;
+          stw[blk(0, 1, j)] = S0.Ry;
+          stw[blk(0, 2, j)] = S0.Ez;
+          stw[blk(0, 3, j)] = S0.Bz;
         }
-      } else {
+      } else if (!DEN) {
 #pragma unroll
-        for (int c = 0; c < 6; ++c)
-          o[c] = blk_ok(n - 1, c) ? ldcg(st + blk(n - 1, c)) : cx<T>(T(0), T(0));
+        for (int c = 0; c < 6; ++c) o[j][c] = blk_ok(n - 1, c) ? ldcg(st + blk(n - 1, c, j)) : zero;
+      }
       }
     }
     __syncthreads();
@@ -2808,7 +2974,7 @@ __device__ void march(const Params& p, const Sm<T>& s, const cg::cluster_group& 
     if (waits && tid == 0 && me == 0)
       wait_for(p, pcid, prog_value(item - 1, nz, min(nz, nz - n + 3)));   // down to n-3
     // (2-D: the spectra and the fields of a slice stay in the CTA, B3 and B4 order its threads)
-    if (SH != 1 && p.ny == 1)
+    if (SH == 0 && p.ny == 1)
       __syncthreads();
     else
       cl.sync();                                                    // B3
@@ -2827,12 +2993,13 @@ __device__ void march(const Params& p, const Sm<T>& s, const cg::cluster_group& 
     }
     TIMER_MARK(PH_INV);
     if constexpr (sizeof(T) == 4) {
-      // SR has been consumed: it holds the fixed-point accumulators of the next push
-      __syncthreads();
+      // SR has been consumed: it holds the fixed-point accumulators of the next push (dense:
+      // they share SC, consumed before B3)
+      if constexpr (!DEN) __syncthreads();
       for (int i = 4 * tid; i < 3 * jplane; i += 4 * NT)
         *reinterpret_cast<int4*>(s.Jint + i) = make_int4(0, 0, 0, 0);
     }
-    if (SH != 1 && p.ny == 1)
+    if (SH == 0 && p.ny == 1)
       __syncthreads();
     else
       cl.sync();                                                    // B4: fields of slice n
@@ -2949,8 +3116,8 @@ template <typename T, bool CANON, int SH, bool DN>
 __device__ __forceinline__ void march_launch(const Params& p) {
   extern __shared__ __align__(16) unsigned char smem[];
   cg::cluster_group cl = cg::this_cluster();
-  const Sm<T> s = carve<T>(p, smem);
-  load_tables(p, s);
+  const Sm<T> s = carve<T, SH == 2>(p, smem);
+  load_tables<T, SH == 2>(p, s);
   if (threadIdx.x < kNDiag) s.dacc[threadIdx.x] = 0.0;
   __syncthreads();
   const int cid = (int)(blockIdx.x / (p.C * p.split));
@@ -2964,6 +3131,11 @@ __device__ __forceinline__ void march_launch(const Params& p) {
 template <typename T, bool CANON = false, int SH = 0, bool DN = false>
 __global__ void __launch_bounds__(512, 1) march_kernel(const Params p) {
   march_launch<T, CANON, SH, DN>(p);
+}
+
+template <bool CANON = false, bool DN = false>
+__global__ void __launch_bounds__(256, 2) march_kernel_dense(const Params p) {
+  march_launch<float, CANON, 2, DN>(p);
 }
 
 #ifndef GEMPIC_CHAIN_TU
@@ -3199,6 +3371,39 @@ __global__ void export_kernel(const Params p, Cx<T>* dst, const Cx<T>* src, int 
 static int align16(int v) { return (v + 15) / 16 * 16; }
 
 #ifndef GEMPIC_CHAIN_TU
+// Dense marches: half an SM.  The spectra of three components received in SC (forward) come before
+// the accumulators have been folded, so the accumulators lie behind those three
+static int smem_layout_dense(Params& p) {
+  const int plane = p.FR * p.nx * 4, nxh = p.nx / 2;
+  p.pcap = 0;
+  p.fcap = kDenseFree;
+  int o = 0;
+  p.o_f0 = o;
+  o += align16(6 * plane);
+  p.o_f1 = o;
+  o += align16(6 * plane);
+  p.o_sr = p.o_workB = p.o_f1;                      // (follow the plane buffers)
+  p.o_j = o;
+  o += align16(3 * p.JR * p.nx * 4);
+  p.o_recv = o;
+  o += align16(9 * p.nx * 4);
+  p.o_sc = p.o_workD = o;
+  p.o_jint = o + align16(3 * p.KB * p.ny * 8);
+  o = std::max(o + align16(6 * p.KB * p.ny * 8), p.o_jint + align16(3 * p.JR * p.nx * 4));
+  p.nwork = 0;
+  p.o_tw = o;
+  o += align16((nxh + nxh) * 8 + (nxh + 32) * 4);
+  p.o_inbox = o;
+  o += align16(p.mig_cap * 4) + align16(7 * p.mig_cap * 4);
+  p.o_outbox = o;
+  o += align16(2 * kOutCap * 4) + align16(7 * kOutCap * 4);
+  p.o_part = p.o_dd = o;
+  p.o_misc = o;
+  o += 32 + kNDiag * 8 + (p.nthreads / 32) * kNDiag * 8;
+  p.smem_bytes = align16(o);
+  return p.smem_bytes;
+}
+
 int smem_layout(Params& p, int eb) {
   // halo geometry: fields own rows + 1 above, currents rows -1 .. RB + 1 (3-D only)
   p.FR = p.ny > 1 ? p.RB + 1 : 1;
@@ -3208,6 +3413,7 @@ int smem_layout(Params& p, int eb) {
   const int nxh = p.nx / 2;
   const int nyh = p.ny > 1 ? p.ny / 2 : 1;
   int o = 0;
+  if (p.dense) return smem_layout_dense(p);
   p.o_f0 = o;
   o += align16(6 * p.FR * p.nx * eb);
   p.o_f1 = o;
@@ -3259,6 +3465,10 @@ static int shape_class(int precision, const Params& p) {
              ? 1 : 0;
 }
 
+#ifndef GEMPIC_CHAIN_TU
+bool dense_ok(int precision, const Params& p) { return shape_class(precision, p) == 1 && p.C == 16; }
+#endif
+
 // The dynamic shared-memory limit is an attribute of the kernel function, shared by every
 // simulation of the process: it is raised to the device's opt-in maximum (each launch asks
 // for its own size), never set to one simulation's size, which would break the launches of a
@@ -3285,6 +3495,7 @@ cudaError_t configure_kernels(int precision, int smem, int) {
   if (e == cudaSuccess) e = cfg_kernel(laser_kernel<float>, smem);
   if (e == cudaSuccess) e = cfg_kernel(march_kernel<float, false, 1>, smem);
   if (e == cudaSuccess) e = cfg_kernel(laser_kernel<float, 1>, smem);
+  if (e == cudaSuccess) e = cfg_kernel(march_kernel_dense<>, smem);
   if (e == cudaSuccess) e = configure_chain(smem);
   return e;
 }
@@ -3315,6 +3526,7 @@ cudaError_t launch_march(int precision, const Params& p, cudaStream_t s) {
   if (precision == 64 && p.nthreads <= 256)
     return cudaLaunchKernelEx(&c, march_kernel_fp64_narrow, p);
   if (precision == 64) return cudaLaunchKernelEx(&c, march_kernel<double>, p);
+  if (p.dense) return cudaLaunchKernelEx(&c, march_kernel_dense<>, p);
   if (shape_class(precision, p) == 1) return cudaLaunchKernelEx(&c, march_kernel<float, false, 1>, p);
   return cudaLaunchKernelEx(&c, march_kernel<float>, p);
 }
@@ -3387,6 +3599,7 @@ cudaError_t max_active_clusters(int precision, const Params& p, int* n) {
   if (precision == 64 && p.nthreads <= 256)
     return cudaOccupancyMaxActiveClusters(n, march_kernel_fp64_narrow, &c);
   if (precision == 64) return cudaOccupancyMaxActiveClusters(n, march_kernel<double>, &c);
+  if (p.dense) return cudaOccupancyMaxActiveClusters(n, march_kernel_dense<>, &c);
   if (shape_class(precision, p) == 1)
     return cudaOccupancyMaxActiveClusters(n, march_kernel<float, false, 1>, &c);
   return cudaOccupancyMaxActiveClusters(n, march_kernel<float>, &c);
