@@ -61,11 +61,6 @@ __device__ __forceinline__ Cx<T> conjg(Cx<T> a) { return {a.re, -a.im}; }
 template <typename T>
 __device__ __forceinline__ Cx<T> mul_i(Cx<T> a) { return {-a.im, a.re}; }   // i a
 
-template <typename T>
-struct V3 {
-  T x, y, z;
-};
-
 // FP32 arithmetic of a push with its fused operations spelled out: the march is compiled for
 // several launch shapes, and which multiplication of a sum is fused must not depend on the
 // code around it, so that every shape gives the same bits.  FP64 is left to the compiler.
@@ -90,6 +85,11 @@ template <typename T>
 __device__ __forceinline__ Cx<T> cmul(Cx<T> a, Cx<T> b) {
   return {pmm(a.re, b.re, a.im, b.im), ppm(a.im, b.re, a.re, b.im)};
 }
+
+template <typename T>
+struct V3 {
+  T x, y, z;
+};
 
 template <typename T>
 __device__ __forceinline__ T gamma_of(V3<T> u) {   // sqrt(1 + ux^2 + uy^2 + uz^2)
@@ -264,32 +264,64 @@ __device__ __forceinline__ Cx<T> twiddle(const Cx<T>* tw, int N, int m, bool inv
 // Radix-2 transforms of `rows` consecutive rows of N = 2^logN values by the whole CTA (any N; used
 // for N < 32, N > 256 and for the FP64 rows of 2-D grids).  A 2-D slice has only two rows to
 // transform forward and three back, and rows of 8 or 16 values leave most lanes of a warp idle:
-// with one row per warp the two transforms of a 512-point FP32 slice took 35 of 68 k cycles, each
-// stage a chain of eight dependent passes of one warp; here every stage is one pass of all the
-// CTA's threads.  The butterflies and twiddles are those of the one-warp transform.
-// Input in bit-reversed positions (bitrev); every thread of the CTA calls it.
+// with one row per warp the two transforms of a 512-point FP32 slice took 35 of 68 k cycles, with
+// one stage per pass of all threads 18 of 45 k, each pass a barrier and a round trip through
+// shared memory.  Long FP32 rows take three stages per pass in registers; in FP64, whose rate
+// binds, and for rows of 8 or 16, which then occupy too few threads, that was slower (128 x 256
+// FP64 22.3 -> 23.0 ms, 16 x 16 0.56 -> 0.60 ms).  The butterflies and twiddles are those of the one-warp transform.
+// Input in bit-reversed positions (bitrev); every thread of the CTA calls it.  SWZ: position q of
+// a row lies at swz(q), which spreads the strided accesses of the first passes over the banks.
 __device__ __forceinline__ int bitrev(int i, int logN) {
   return logN ? (int)(__brev((unsigned)i) >> (32 - logN)) : 0;
 }
-template <typename T>
-__device__ void block_fft_r2(Cx<T>* d, int rows, int logN, const Cx<T>* tw, bool inverse) {
-  const int total = rows << (logN - 1);
-  __syncthreads();
-  for (int s = 1; s <= logN; ++s) {
-    const int half = 1 << (s - 1);
-    for (int b = threadIdx.x; b < total; b += blockDim.x) {
-      const int j = b & (half - 1);
-      const int i0 = ((b >> (s - 1)) << s) + j;
-      const int i1 = i0 + half;
-      Cx<T> w = tw[j << (logN - s)];
-      if (inverse) w.im = -w.im;
-      const Cx<T> t = w * d[i1];
-      const Cx<T> u = d[i0];
-      d[i0] = u + t;
-      d[i1] = u - t;
+__device__ __forceinline__ int swz(int q) { return q ^ ((q >> 3) & 7); }
+
+// stages s .. s + R - 1: a thread takes the 2^R values j + m 2^(s-1) of a block
+template <typename T, bool SWZ, int R, bool INV>
+__device__ __forceinline__ void fft_pass(Cx<T>* d, int rows, int logN, int s, const Cx<T>* tw) {
+  constexpr int V = 1 << R;
+  const int half = 1 << (s - 1), lw = logN - R;              // log2 of the blocks per row x half
+  for (int b = threadIdx.x; b < rows << lw; b += blockDim.x) {
+    const int row = b >> lw, i = b & ((1 << lw) - 1);
+    const int j = i & (half - 1);
+    const int p0 = ((i >> (s - 1)) << (s - 1 + R)) + j;
+    Cx<T>* w0 = d + (row << logN);
+    Cx<T> a[V];
+#pragma unroll
+    for (int m = 0; m < V; ++m) {
+      const int q = p0 + m * half;
+      a[m] = w0[SWZ ? swz(q) : q];
     }
-    __syncthreads();
+#pragma unroll
+    for (int st = 0; st < R; ++st) {
+      const int h2 = 1 << st;
+#pragma unroll
+      for (int m = 0; m < V; ++m) {
+        if (m & h2) continue;
+        const int jj = j + (m & (h2 - 1)) * half;
+        const Cx<T> w = tw[jj << (logN - s - st)], x = a[m | h2];
+        // w x, or conj(w) x
+        const Cx<T> t = INV ? cx<T>(ppm(w.re, x.re, w.im, x.im), pmm(w.re, x.im, w.im, x.re)) : cmul(w, x);
+        const Cx<T> u = a[m];
+        a[m] = u + t;
+        a[m | h2] = u - t;
+      }
+    }
+#pragma unroll
+    for (int m = 0; m < V; ++m) {
+      const int q = p0 + m * half;
+      w0[SWZ ? swz(q) : q] = a[m];
+    }
   }
+  __syncthreads();
+}
+template <typename T, bool SWZ, bool INV>
+__device__ __forceinline__ void block_fft(Cx<T>* d, int rows, int logN, const Cx<T>* tw) {
+  __syncthreads();
+  int s = 1;
+  if (sizeof(T) == 4 && logN >= 9)
+    for (; s + 2 <= logN; s += 3) fft_pass<T, SWZ, 3, INV>(d, rows, logN, s, tw);
+  for (; s <= logN; ++s) fft_pass<T, SWZ, 1, INV>(d, rows, logN, s, tw);
 }
 
 template <typename T>
@@ -921,15 +953,15 @@ __device__ void forward_rows(const cg::cluster_group& cl, const Params& p, const
     const int yl = task >> 1, pr = task & 1;
     const T* a = J + ((size_t)(pr == 0 ? 0 : 2) * p.JR + yl + p.JOFF) * p.nx;
     const T* b = J + ((size_t)1 * p.JR + yl + p.JOFF) * p.nx;
-    w[(task << p.lognx) + bitrev(x, p.lognx)] = cx<T>(a[x], pr == 0 ? b[x] : T(0));
+    w[(task << p.lognx) + swz(bitrev(x, p.lognx))] = cx<T>(a[x], pr == 0 ? b[x] : T(0));
   }
-  block_fft_r2(w, ntask, p.lognx, s.twx, false);
+  block_fft<T, true, false>(w, ntask, p.lognx, s.twx);
   for (int i = threadIdx.x; i < ntask * nxh; i += blockDim.x) {
     const int task = i >> (p.lognx - 1), k = i & (nxh - 1);
     const int pr = task & 1, y = (me << p.logRB) + (task >> 1);
     const Cx<T>* wr = w + (task << p.lognx);
-    const Cx<T> zk = wr[k];
-    const Cx<T> zm = conjg(wr[(p.nx - k) & (p.nx - 1)]);
+    const Cx<T> zk = wr[swz(k)];
+    const Cx<T> zm = conjg(wr[swz((p.nx - k) & (p.nx - 1))]);
     Cx<T> X = T(0.5) * (zk + zm);                     // spectrum of the real part
     const Cx<T> Y = T(0.5) * mul_i(zm - zk);          // spectrum of the imaginary part
     const int rd = k >> p.logKB, kxl = k & (p.KB - 1);
@@ -1013,7 +1045,10 @@ __device__ void column_ffts(const Params& p, const Sm<T>& s, int c0, int c1, boo
           d[i - q + r] = t;
         }
       }
-      block_fft_r2(d, ntask, p.logny, s.twy, inverse);
+      if (inverse)
+        block_fft<T, false, true>(d, ntask, p.logny, s.twy);
+      else
+        block_fft<T, false, false>(d, ntask, p.logny, s.twy);
       return;
     }
     const int warp = threadIdx.x >> 5;
@@ -1189,17 +1224,18 @@ __device__ void inverse_rows(const Params& p, const Sm<T>& s, T* Fdst, T& fe) {
         Cx<T>* wr = w + ((i >> (p.lognx - 1)) << p.lognx);
         if (k == 0) {
           wr[0] = cx<T>(x.re, y.re);                        // real DC of each field
-          wr[bitrev(nxh, p.lognx)] = cx<T>(T(0), T(0));     // Nyquist projected out
+          wr[swz(bitrev(nxh, p.lognx))] = cx<T>(T(0), T(0));     // Nyquist projected out
         } else {
-          wr[bitrev(k, p.lognx)] = cx<T>(x.re - y.im, x.im + y.re);          // X + i Y
-          wr[bitrev(p.nx - k, p.lognx)] = cx<T>(x.re + y.im, y.re - x.im);   // conj(X) + i conj(Y)
+          wr[swz(bitrev(k, p.lognx))] = cx<T>(x.re - y.im, x.im + y.re);          // X + i Y
+          wr[swz(bitrev(p.nx - k, p.lognx))] = cx<T>(x.re + y.im, y.re - x.im);   // conj(X) + i conj(Y)
         }
       }
-      block_fft_r2(w, nt, p.lognx, s.twx, true);
+      block_fft<T, true, true>(w, nt, p.lognx, s.twx);
       for (int i = threadIdx.x; i < nt << p.lognx; i += blockDim.x) {
         const int task = t0 + (i >> p.lognx), x = i & (p.nx - 1);
         const int yl = task / 3, pr = task - 3 * yl;
-        const T va = w[i].re * scale, vb = w[i].im * scale;
+        const Cx<T> v = w[i - x + swz(x)];
+        const T va = v.re * scale, vb = v.im * scale;
         Fdst[((size_t)(2 * pr) * p.FR + yl) * p.nx + x] = va;
         Fdst[((size_t)(2 * pr + 1) * p.FR + yl) * p.nx + x] = vb;
         if (yl < p.RB) fe += va * va + vb * vb;
@@ -2064,9 +2100,7 @@ struct Mode6 {
   Cx<T> Rx, Ry, Lx, Ly, Ez, Bz;
 };
 
-// GEN: the generic kernel (any size); it and the 128 x 128 one fuse a different product in three
-// of the sums.
-template <typename T, bool GEN>
+template <typename T>
 __device__ __forceinline__ Mode6<T> slice_solve(T kx, T ky, T h, T Dl, const Mode6<T>& n1,
                                                 Cx<T> Rxo, Cx<T> Ryo, Cx<T> Ezo, Cx<T> Bzo,
                                                 Cx<T> jx0m, Cx<T> jy0m, Cx<T> jx0p, Cx<T> jy0p,
@@ -2090,8 +2124,7 @@ __device__ __forceinline__ Mode6<T> slice_solve(T kx, T ky, T h, T Dl, const Mod
   numE = cfma_i(hh2, kk(kx, jx1p, ky, jy1p), numE);
   numE = cfma_i(h4, kk(kx, Wx, ky, Wy), numE);
   const Cx<T> jr = km(kx, jy1p, ky, jx1p);
-  Cx<T> numB = cx<T>(pmm(c16, n1.Bz.re, hh2, jr.im),
-                     GEN ? ppm(hh2, jr.re, c16, n1.Bz.im) : ppm(c16, n1.Bz.im, hh2, jr.re));
+  Cx<T> numB = cx<T>(pmm(c16, n1.Bz.re, hh2, jr.im), ppm(c16, n1.Bz.im, hh2, jr.re));
   numB = cfma_i(hD, km(kx, Jy, ky, Jx), numB);
   numB = cfma(-hDK, Bzo, numB);
   numB = cfma_i(h4, km(ky, Ux, kx, Uy), numB);
@@ -2103,12 +2136,12 @@ __device__ __forceinline__ Mode6<T> slice_solve(T kx, T ky, T h, T Dl, const Mod
   const Cx<T> sEz = o.Ez + Ezo, sBz = o.Bz + Bzo;
   const Cx<T> z = cx<T>(T(0), T(0));
   const Cx<T> q4x = T(0.25) * Jx, q4y = T(0.25) * Jy;
-  o.Rx = cfma(Dl, cfma_i(T(0.5), GEN ? kk(ky, sBz, kx, sEz) : kk(kx, sEz, ky, sBz), z - q4x), Rxo);
+  o.Rx = cfma(Dl, cfma_i(T(0.5), kk(kx, sEz, ky, sBz), z - q4x), Rxo);
   o.Ry = cfma(Dl, cfma_i(T(0.5), km(ky, sEz, kx, sBz), z - q4y), Ryo);
   // LxN, LyN (box scheme in zeta)
   const Cx<T> tEz = n1.Ez + o.Ez, tBz = o.Bz + n1.Bz;
   o.Lx = cfma(-(T(0.5) * h), cfma_i(T(0.5), km(kx, tEz, ky, tBz), jx1p), n1.Lx);
-  o.Ly = cfma(-(T(0.5) * h), cfma_i(T(0.5), GEN ? kk(kx, tBz, ky, tEz) : kk(ky, tEz, kx, tBz), jy1p), n1.Ly);
+  o.Ly = cfma(-(T(0.5) * h), cfma_i(T(0.5), kk(ky, tEz, kx, tBz), jy1p), n1.Ly);
   return o;
 }
 
@@ -2934,7 +2967,7 @@ __device__ void march(const Params& p, const Sm<T>& s_, const cg::cluster_group&
       if (masked[j]) {
         S0.Rx = S0.Ry = S0.Lx = S0.Ly = S0.Ez = S0.Bz = zero;
       } else {
-        S0 = slice_solve<T, SH == 0>(kx[j], ky[j], hn, Dl, S1[j], o[j][0], o[j][1], o[j][2], o[j][3], j0mx, j0my,
+        S0 = slice_solve(kx[j], ky[j], hn, Dl, S1[j], o[j][0], o[j][1], o[j][2], o[j][3], j0mx, j0my,
                          j0px[j], j0py[j], Jx, Jy, Jz);
       }
       // fields E, B (Eqs. Rx..Ly) for the inverse transform
