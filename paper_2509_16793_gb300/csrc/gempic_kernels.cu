@@ -2510,10 +2510,15 @@ __device__ void march(const Params& p, const Sm<T>& s_, const cg::cluster_group&
     // ---------------- A: streaming push from plane n+1 to plane n -----------------------
     {
       const int cnt0 = s.misc[M_PCOUNT];
+      float4 na = make_float4(__int_as_float(-1), 0.f, 0.f, 0.f);
+      if (DEN && tid < cnt0) na = __ldcg(gs.a + tid);
       for (int i = tid; i < cnt0; i += NT) {
         PState<T> P;
         if constexpr (DEN) {
-          const float4 pa = __ldcg(gs.a + i), pb = __ldcg(gs.b + i);
+          // the next particle's position is under way while this one is pushed; the momentum
+          // arrives during the gather
+          const float4 pa = na, pb = __ldcg(gs.b + i);
+          if (i + NT < cnt0) na = __ldcg(gs.a + i + NT);
           if (__float_as_int(pa.x) < 0) continue;
           P = g_unpack<T>(pa, pb);
         } else {
