@@ -205,6 +205,7 @@ gempic_status ensure_initialized(gempic_sim* s) {
   if (s->initialized) return GEMPIC_OK;
   const int prec = s->cfg.precision;
   cudaError_t e = cudaSuccess;
+  s->p.bunch = (s->has_beam && s->beam.n_macro > 0) || !s->px.empty() ? 1 : 0;
   if (s->has_laser) {
     e = gempic::launch_laser_init(prec, s->p, s->laser.a0, s->laser.waist, s->laser.duration,
                                   s->laser.zeta_center, s->laser.pol, s->stream);

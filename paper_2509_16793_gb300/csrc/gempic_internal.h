@@ -37,6 +37,7 @@ struct Params {
   int C, RB, KB, M;               // CTAs per slice, rows per CTA, kx per CTA, modes per CTA
   int split;                      // 2-D: CTAs that share a march's particles (1: not split); the
                                   // cluster has C split CTAs
+  int bunch;                      // 1: particles were placed in the box (a bunch)
   int dense;                      // 1: two CTAs of 256 threads per SM (FP32 128 x 128 grids)
   int FR, JR, JOFF;               // field rows per CTA (own + halo above), current rows (own +
                                   // halo below/above), row offset of own row 0 in the currents
@@ -185,6 +186,8 @@ cudaError_t launch_tables(int precision, const Params& p, void* dst, cudaStream_
 // the denoised chain's march (FP32, p.dn_pipe = 1; compiled in gempic_chain.cu)
 cudaError_t configure_chain(int smem_bytes);
 cudaError_t launch_march_chain(const Params& p, cudaStream_t s);
+// the 128 x 128 FP32 march of simulations with a bunch (compiled in gempic_chain.cu)
+cudaError_t launch_march_bunch(const Params& p, cudaStream_t s);
 // the learned current denoiser on output half-slices [z0, z1) (gempic_denoise.cu); status codes
 // of gempic_status
 int denoise_range(struct gempic_denoiser* d, const float* j_in, float* j_out, int nx, int ny,

@@ -602,7 +602,8 @@ enum CstSlot {
   K_H = 0, K_INVH, K_HX, K_HY, K_D, K_DF, K_WSCALE, K_CX, K_CY, K_INVHX, K_INVHY, K_FLUX,
   K_BEAM, K_JREF, K_JSCALE, K_JINV, K_QM = 16, K_MOQ = 20, K_QF = 24, K_INVD = 28, K_N = 29
 };
-enum MiscSlot { M_PCOUNT = 0, M_FTOP, M_INBOX, M_RQN, M_JFLAG, M_STN, M_OUTN, M_IOSEEN };
+enum MiscSlot { M_PCOUNT = 0, M_FTOP, M_INBOX, M_RQN, M_JFLAG, M_STN, M_OUTN, M_IOSEEN, M_WINX, M_WINY,
+                M_N = 12 };
 // particles leaving the band during a push wait in a local outbox of this many entries
 constexpr int kOutCap = 64;
 
@@ -635,7 +636,7 @@ struct Sm {
   int* pcell;       // [pcap] ix | iy << 10 | sp << 20, -1 = empty
   T *pfx, *pfy, *pux, *puy, *puz, *psig, *pq;
   int* fstack;      // [fcap] free particle slots
-  int* misc;        // MiscSlot
+  int* misc;        // MiscSlot [M_N]
   double* dacc;     // [kNDiag]; dacc[0], dacc[1]: the march's continuity and Gauss residual
                     // maxima (verification mode)
   T* dd;            // [RBe][nx] continuity residual: w CIC(start) - w CIC(end) of the slab's
@@ -710,7 +711,7 @@ __device__ Sm<T> carve(const Params& p, unsigned char* base) {
   s.pq = pt + 6 * p.pcap;
   s.fstack = (int*)(pt + 7 * p.pcap);
   s.misc = (int*)(base + p.o_misc);
-  s.dacc = (double*)(base + p.o_misc + 32);
+  s.dacc = (double*)(base + p.o_misc + M_N * 4);
   s.dwarp = s.dacc + kNDiag;
   s.dd = (T*)(base + p.o_dd);
   s.dn = s.dd + (size_t)(p.ny > 1 ? p.RB : 1) * p.nx;
@@ -953,7 +954,8 @@ __device__ __noinline__ void forward_rows_r8(const cg::cluster_group& cl, const 
 
 // SH = 1: the kernel instantiated for 128 x 128 grids with an even band (only the length-128
 // transforms are compiled in; with the other lengths present the compiler schedules them
-// markedly worse).  SH = 2: the same for two CTAs per SM (march(), "dense")
+// markedly worse).  SH = 2: the same for two CTAs per SM (march(), "dense"); SH = 3: SH = 1 for
+// simulations with a bunch (stored_phase)
 // J: the slice's currents (s.J, or the sum over the CTAs of a split march)
 template <typename T, int SH>
 __device__ void forward_rows(const cg::cluster_group& cl, const Params& p, const Sm<T>& s,
@@ -1798,12 +1800,22 @@ __device__ bool stream_push(const Params& p, const Sm<T>& s, const T* Fcur, PSta
   return trap;
 }
 
-// write a particle into a stored store (ring slot, bucket); false on overflow
-template <typename T>
+// write a particle into a stored store (ring slot, bucket); false on overflow.  GROUP: the lanes
+// that append to one bucket together reserve their entries with one atomic (a bunch's 2^20
+// particles stay in their slab for most s-steps, and one address takes one atomic at a time)
+template <typename T, bool GROUP = false>
 __device__ bool store_append(const PartStore& S, const Params& p, int slot, int bucket,
                              const PState<T>& P, T fz) {
   int* cnt = S.cnt + (size_t)slot * p.nz + bucket;
-  const int i = atomicAdd(cnt, 1);
+  int i = 0;
+  if constexpr (GROUP) {
+    const unsigned grp = __match_any_sync(__activemask(), (unsigned long long)cnt);
+    const int leader = __ffs(grp) - 1;
+    if ((int)(threadIdx.x & 31) == leader) i = atomicAdd(cnt, __popc(grp));
+    i = __shfl_sync(grp, i, leader) + __popc(grp & ((1u << (threadIdx.x & 31)) - 1u));
+  } else {
+    i = atomicAdd(cnt, 1);
+  }
   if (i >= p.bcap) return false;
   const size_t e = ((size_t)slot * p.nz + bucket) * p.bcap + i;
   S.cell[e] = P.ix | (P.iy << 10) | (P.sp << 20);
@@ -1992,6 +2004,28 @@ __device__ __forceinline__ void put_particle(const Params& p, const Sm<T>& s, co
 // Stored particle along s (Sec. 5.1: trapped / beam particles are integrated along s):
 // bucket n of level k+1, fields of slices n (Fn) and n+1 (Fn1) of that level.
 // ------------------------------------------------------------------------------------------
+// Adds v0, v1 to the neighbouring nodes gx, gx + 1 (mod nx) of a row in global memory: one 8- or
+// 16-byte reduction where the pair lies in one (PAIR), else two.
+template <bool PAIR>
+__device__ __forceinline__ void red_pair(float* row, int gx, int gx1, float v0, float v1) {
+  float* a = row + gx;
+  if (PAIR && (gx & 1) == 0) {
+    asm volatile("red.global.add.v2.f32 [%0], {%1, %2};" ::"l"(a), "f"(v0), "f"(v1) : "memory");
+  } else if (PAIR && (gx & 3) == 1) {
+    asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(a - 1), "f"(0.0f), "f"(v0),
+                 "f"(v1), "f"(0.0f)
+                 : "memory");
+  } else {
+    atomicAdd(a, v0);
+    atomicAdd(row + gx1, v1);
+  }
+}
+template <bool PAIR>
+__device__ __forceinline__ void red_pair(double* row, int gx, int gx1, double v0, double v1) {
+  atomicAdd(row + gx, v0);
+  atomicAdd(row + gx1, v1);
+}
+
 // Adds the warp's sum of v into the warp's row of FP64 diagnostics.  The sum runs in the
 // type of v (FP32 sums in FP32: FP64 arithmetic is a small fraction of the FP32 rate), and lane
 // 0 adds it in FP64.  Every lane of the warp calls it.
@@ -2002,7 +2036,17 @@ __device__ __forceinline__ void warp_diag_add(double* dwarp, int slot, V v) {
   if ((threadIdx.x & 31) == 0) dwarp[(threadIdx.x >> 5) * kNDiag + slot] += (double)v;
 }
 
-template <typename T>
+//
+// Large buckets (a bunch) of a cluster: each CTA first copies the fields around the bunch (a window
+// of the cells around the mean of a sample, both planes, as much as the free column spectra's
+// shared memory holds) and gathers from the copy.  Without it the particles of a narrow bunch, dealt
+// out over the CTAs, read the two or three CTAs on the axis through distributed shared memory,
+// 48 scattered values each: 31 k cycles of a slice on average with 2^20 macroparticles on
+// 128 x 128 x 768, 80 k where the bunch is, and as much in waits for the slowest CTA.  (Giving each
+// particle to the CTA of its row was slower: the two CTAs on the axis then do every reduction.)
+// pwfa 128 x 128 x 768, 7 s-steps: 47.7 -> 32.7 ms.  WIN: compiled in (the registers of the window
+// cost the 128 x 128 march without a bunch 1.5 %, so that one has an instantiation of its own).
+template <typename T, bool DEN, bool WIN>
 __device__ void stored_phase(const Params& p, const Sm<T>& s, const T* Fn, const T* Fn1,
                              int s1, int s2, int n, int me, int rank, int nrank, int cnt_raw,
                              bool varh) {
@@ -2012,7 +2056,42 @@ __device__ void stored_phase(const Params& p, const Sm<T>& s, const T* Fn, const
   const int cnt = min(cnt_raw, p.bcap);
   const T D = s.cst[K_D], h = s.cst[K_H], invh = s.cst[K_INVH];
   const int mx = p.nx - 1, my = p.ny - 1;
-  for (int e0 = rank * blockDim.x + threadIdx.x; e0 < cnt; e0 += nrank * blockDim.x) {
+  constexpr int WX = DEN ? 16 : 24;               // window: WX columns, WY rows of 2 x 6 planes
+  const int WY = (DEN ? 3 : 6) * p.KB * p.ny * 2 / (12 * WX);
+  const bool window = WIN && p.C > 1 && p.nx >= 32 && WY >= 4 && cnt > (int)blockDim.x;
+  T* const win = reinterpret_cast<T*>(s.SC);
+  int x0 = 0, y0 = 0;
+  if (window) {
+    if (threadIdx.x < 32) {
+      const int c = ldcg(p.st.cell + ((size_t)s1 * p.nz + n) * p.bcap +
+                         (size_t)threadIdx.x * (size_t)cnt / 32);
+      int sx = c & 1023, sy = (c >> 10) & 1023;
+#pragma unroll
+      for (int off = 16; off > 0; off >>= 1) {
+        sx += __shfl_xor_sync(0xffffffffu, sx, off);
+        sy += __shfl_xor_sync(0xffffffffu, sy, off);
+      }
+      if (threadIdx.x == 0) {
+        s.misc[M_WINX] = (sx / 32 - WX / 2) & mx;
+        s.misc[M_WINY] = (sy / 32 - WY / 2) & my;
+      }
+    }
+    __syncthreads();
+    x0 = s.misc[M_WINX];
+    y0 = s.misc[M_WINY];
+    for (int i = threadIdx.x; i < 12 * WY * WX; i += blockDim.x) {
+      const int rx = i % WX, t = i / WX;
+      const int ry = t % WY, pc = t / WY;           // plane and component
+      const T* F = pc < 6 ? Fn : Fn1;
+      const int c = pc < 6 ? pc : pc - 6;
+      const RowRef<T> rr = row_ref(p, F, p.FR, 0, (y0 + ry) & my, me);
+      win[i] = row_ld(rr, (uint32_t)(c * p.FR * p.nx + ((x0 + rx) & mx)));
+    }
+    __syncthreads();
+  }
+  // (equal shares: the slowest CTA holds up the next slice's first barrier)
+  const int share = (cnt + nrank - 1) / nrank;
+  for (int e0 = rank * share + threadIdx.x; e0 < min(cnt, (rank + 1) * share); e0 += blockDim.x) {
     T fz;
     PState<T> P = store_read<T>(p.st, p, ((size_t)s1 * p.nz + n) * p.bcap + e0, fz);
     const T g = gamma_of(P.u);
@@ -2029,8 +2108,21 @@ __device__ void stored_phase(const Params& p, const Sm<T>& s, const T* Fn, const
       continue;
     }
     T lo[6], hi[6], E[6];
-    gather6_g(p, Fn, P.ix, P.fx, P.iy, P.fy, me, lo);
-    gather6_g(p, Fn1, P.ix, P.fx, P.iy, P.fy, me, hi);
+    const int wx = (P.ix - x0) & mx, wy = (P.iy - y0) & my;
+    if (window && wx < WX - 1 && wy < WY - 1) {
+      const T w00 = mul_(T(1) - P.fx, T(1) - P.fy), w10 = mul_(P.fx, T(1) - P.fy);
+      const T w01 = mul_(T(1) - P.fx, P.fy), w11 = mul_(P.fx, P.fy);
+      const T* f = win + wy * WX + wx;
+#pragma unroll
+      for (int c = 0; c < 12; ++c) {
+        const T* g = f + c * WY * WX;
+        (c < 6 ? lo[c] : hi[c - 6]) =
+            fma_(w11, g[WX + 1], fma_(w01, g[WX], ppm(w00, g[0], w10, g[1])));
+      }
+    } else {
+      gather6_g(p, Fn, P.ix, P.fx, P.iy, P.fy, me, lo);
+      gather6_g(p, Fn1, P.ix, P.fx, P.iy, P.fy, me, hi);
+    }
 #pragma unroll
     for (int c = 0; c < 6; ++c) E[c] = (T(1) - fz) * lo[c] + fz * hi[c];
     // GT2: the s-step is the distance Delta along z (dt = Delta/v_z); GT1: the lab time Delta
@@ -2120,16 +2212,16 @@ __device__ void stored_phase(const Params& p, const Sm<T>& s, const T* Fn, const
           } else {
             const T j0f = floor(Y), fy = Y - j0f;
             const int gy = (P.iy + (int)j0f) & my, gy1 = (gy + 1) & my;
-            atomicAdd(pl + (size_t)gy * p.nx + gx, ((T(1) - fx) * (T(1) - fy)) * vals[c]);
-            atomicAdd(pl + (size_t)gy * p.nx + gx1, (fx * (T(1) - fy)) * vals[c]);
-            atomicAdd(pl + (size_t)gy1 * p.nx + gx, ((T(1) - fx) * fy) * vals[c]);
-            atomicAdd(pl + (size_t)gy1 * p.nx + gx1, (fx * fy) * vals[c]);
+            red_pair<WIN>(pl + (size_t)gy * p.nx, gx, gx1, ((T(1) - fx) * (T(1) - fy)) * vals[c],
+                          (fx * (T(1) - fy)) * vals[c]);
+            red_pair<WIN>(pl + (size_t)gy1 * p.nx, gx, gx1, ((T(1) - fx) * fy) * vals[c],
+                          (fx * fy) * vals[c]);
           }
         }
-        atomicExch(p.jflag + (size_t)s2 * p.nz + iz, 1);
+        __stcg(p.jflag + (size_t)s2 * p.nz + iz, 1);
       }
     }
-    if (!store_append(p.st, p, s2, m, P, fz)) atomicOr(p.err, ERR_BCAP);
+    if (!store_append<T, WIN>(p.st, p, s2, m, P, fz)) atomicOr(p.err, ERR_BCAP);
   }
   if (p.diag) {
     if (__any_sync(0xffffffffu, (dsto | dlost) != 0)) {
@@ -3145,7 +3237,7 @@ __device__ void march(const Params& p, const Sm<T>& s_, const cg::cluster_group&
     // ---------------- E: stored particles of cell (zeta_n, zeta_{n+1}] along s -------------
     // (most cells hold no stored particle: the call is skipped, uniformly over the CTA)
     if (s.misc[M_STN] > 0 && !p.skip_stored && !dn1)
-      stored_phase(p, s, Fnew, Fcur, s1, s2, n, me, rank, nrank, s.misc[M_STN], varh);
+      stored_phase<T, DEN, (SH >= 2)>(p, s, Fnew, Fcur, s1, s2, n, me, rank, nrank, s.misc[M_STN], varh);
     TIMER_MARK(PH_E);
     T* t = Fcur;
     Fcur = Fnew;
@@ -3487,7 +3579,7 @@ static int smem_layout_dense(Params& p) {
   o += align16(2 * kOutCap * 4) + align16(7 * kOutCap * 4);
   p.o_part = p.o_dd = o;
   p.o_misc = o;
-  o += 32 + kNDiag * 8 + (p.nthreads / 32) * kNDiag * 8;
+  o += M_N * 4 + kNDiag * 8 + (p.nthreads / 32) * kNDiag * 8;
   p.smem_bytes = align16(o);
   return p.smem_bytes;
 }
@@ -3538,7 +3630,7 @@ int smem_layout(Params& p, int eb) {
   p.o_dd = o;
   if (p.resid) o += align16(3 * (p.ny > 1 ? p.RB : 1) * p.nx * eb);
   p.o_misc = o;
-  o += 32 + kNDiag * 8 + (p.nthreads / 32) * kNDiag * 8;
+  o += M_N * 4 + kNDiag * 8 + (p.nthreads / 32) * kNDiag * 8;
   p.smem_bytes = align16(o);
   return p.smem_bytes;
 }
@@ -3615,6 +3707,7 @@ cudaError_t launch_march(int precision, const Params& p, cudaStream_t s) {
     return cudaLaunchKernelEx(&c, march_kernel_fp64_narrow, p);
   if (precision == 64) return cudaLaunchKernelEx(&c, march_kernel<double>, p);
   if (p.dense) return cudaLaunchKernelEx(&c, march_kernel_dense<>, p);
+  if (shape_class(precision, p) == 1 && p.bunch) return launch_march_bunch(p, s);
   if (shape_class(precision, p) == 1) return cudaLaunchKernelEx(&c, march_kernel<float, false, 1>, p);
   return cudaLaunchKernelEx(&c, march_kernel<float>, p);
 }
@@ -3697,8 +3790,15 @@ cudaError_t max_active_clusters(int precision, const Params& p, int* n) {
 
 // the denoised chain's instantiations of the march (FP32; the 128 x 128 one where it applies)
 cudaError_t configure_chain(int smem) {
-  cudaError_t e = cfg_kernel(march_kernel<float, false, 0, true>, smem);
+  cudaError_t e = cfg_kernel(march_kernel<float, false, 3>, smem);
+  if (e == cudaSuccess) e = cfg_kernel(march_kernel<float, false, 0, true>, smem);
   return e == cudaSuccess ? cfg_kernel(march_kernel<float, false, 1, true>, smem) : e;
+}
+
+cudaError_t launch_march_bunch(const Params& p, cudaStream_t s) {
+  cudaLaunchAttribute attr[1];
+  cudaLaunchConfig_t c = make_cfg(p, p.P, s, attr);
+  return cudaLaunchKernelEx(&c, march_kernel<float, false, 3>, p);
 }
 
 cudaError_t launch_march_chain(const Params& p, cudaStream_t s) {
