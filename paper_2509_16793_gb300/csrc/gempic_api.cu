@@ -620,8 +620,11 @@ gempic_status create_sim(const gempic_config* cfg, gempic_sim** out, bool one_ct
   }
   // marches in flight: a march trails the one before it by about four slices, so up to a quarter
   // of the window's slices march at once.  2-D marches take one CTA each, and 16 of them (the
-  // limit of the clustered 3-D marches) left 136 of 152 SMs idle
-  const int deepest = s->shapes.empty() ? 16 : std::min(64, std::max(16, g.nzeta / 4));
+  // limit of the clustered 3-D marches) left 136 of 152 SMs idle.  Beyond the depth that was always
+  // taken, the rings of s-levels (stored particles, rejoin queues, beam current) may take 16 GiB.
+  const double level_bytes = (double)g.nzeta * (2.0 * p.bcap * (4 + 7 * s->eb) + 3.0 * g.nx * g.ny * s->eb);
+  const int levels = (int)std::min(128.0, 17179869184.0 / level_bytes) - 2;
+  const int deepest = s->shapes.empty() ? 16 : std::max(16, std::min(std::min(64, g.nzeta / 4), levels));
   s->pmax = cfg->pipeline_depth > 0 ? cfg->pipeline_depth : std::max(1, std::min(maxcl, deepest));
   if (s->pmax > std::max(1, maxcl)) s->pmax = std::max(1, maxcl);
   for (gempic_sim::Shape& sh : s->shapes) sh.maxcl = std::min(sh.maxcl, s->pmax);
@@ -644,7 +647,7 @@ gempic_status create_sim(const gempic_config* cfg, gempic_sim** out, bool one_ct
         return GEMPIC_ECUDA;
       }
       if (cfg->pipeline_depth > 0) two.maxcl = std::min(two.maxcl, cfg->pipeline_depth);
-      two.maxcl = std::min(two.maxcl, 16);
+      two.maxcl = std::min(two.maxcl, std::min(16, levels));
       if (two.maxcl > s->pmax) {
         s->shapes.push_back(one);
         s->shapes.push_back(two);

@@ -1055,9 +1055,11 @@ size_t conv_smem() { return (size_t)kTaps * kTapBytesB + 2u * kRound * kTapBytes
 
 // buffers for nx x ny x nz voxels (activations in their layout's size)
 cudaError_t grow(gempic_denoiser* d, int nx, int ny, int nz) {
-  const long long V = (long long)nx * ny * nz;
-  const size_t bytes = nx == kRowVox ? (size_t)ny * nz * kRowBytes : (size_t)V * kCh * sizeof(__nv_bfloat16);
+  long long V = (long long)nx * ny * nz;
+  size_t bytes = nx == kRowVox ? (size_t)ny * nz * kRowBytes : (size_t)V * kCh * sizeof(__nv_bfloat16);
   if (bytes <= d->act_bytes && V <= d->cap) return cudaSuccess;
+  bytes = std::max(bytes, d->act_bytes);           // neither shrinks: calls may alternate layouts
+  V = std::max(V, d->cap);
   for (auto*& a : d->act) {
     if (a) cudaFree(a);
     a = nullptr;
