@@ -313,7 +313,8 @@ gempic_status gempic_get_onaxis_ez(struct gempic_sim* sim, double* dst, int32_t 
 /* Device kernels this library launched since create (for launch accounting). */
 int64_t gempic_launch_count(const struct gempic_sim* sim);
 
-/* Launch shape chosen at create: CTAs per cluster, threads per CTA, dynamic shared bytes,
+/* Launch shape of one s-step chosen at create (a call of several s-steps may spread a march over
+ * other CTAs): CTAs per cluster, threads per CTA, dynamic shared bytes,
  * s-steps marched concurrently. */
 gempic_status gempic_launch_shape(const struct gempic_sim* sim, int32_t* cluster_ctas,
                                   int32_t* threads, int32_t* smem_bytes, int32_t* pipeline);
@@ -456,7 +457,7 @@ void gempic_denoiser_destroy(gempic_denoiser* d);
  * s-step saw the first pass's fields: the net needs the current of half-slices on both sides
  * of each one, which the march produces only one at a time.  The n s-steps of a call run as
  * one chain of 2n marches in one launch, each following the one before it slice by slice; up
- * to min(7, pipeline_depth) in flight, or, with pipeline_depth 0, as many as leave a third of
+ * to min(7, pipeline_depth) in flight, or, with pipeline_depth 0, as many as leave a quarter of
  * the SMs to the net.  The calling thread runs the net on groups of half-slices as soon as the
  * first pass has written them and the three half-slices beyond, on a stream of its own, and
  * releases each group to the second pass, which waits for it (bounded).  The call waits for

@@ -344,14 +344,14 @@ int pick_threads(int precision, int M, int fresh) {
   return std::min(512, std::max(std::max(M, 128), (std::min(most, fresh) + 31) / 32 * 32));
 }
 
-// cycles of one slice of a 2-D march on S CTAs, from the phase timers: the push (FP64 bound by
-// the SM's two lanes, FP32 by issue) divides, transforms and solve do not, and the summation
-// over the CTAs adds two cluster barriers and S reads per current
+// cycles of one slice of a 2-D march on S CTAs, fitted to lone marches of 64 to 1024 cells: the
+// push (FP64 bound by the SM's two lanes, FP32 by issue) divides, transforms and solve do not,
+// and each further CTA adds to the cluster barriers and to the sum over the CTAs.  FP64, 128
+// cells, 4 per cell on 1, 2, 4, 8 CTAs: 140, 90, 72, 71 k; FP32, 512 cells: 39, 31, 27, 30 k.
 double slice_cycles_2d(const Params& p, int eb, int S) {
   const double np = (double)p.nx * p.ppc_sum / S;
-  const double push = eb == 8 ? 260.0 * np + 4000.0 : 8.0 * np + 3000.0;
-  const double fixed = eb == 8 ? 10000.0 + 160.0 * p.nx : 12000.0 + 16.0 * p.nx;
-  return push + fixed + (S > 1 ? 2500.0 + 2.0 * S * p.nx * 3 / p.nthreads * 8.0 : 0.0);
+  if (eb == 8) return 200.0 * np + 18000.0 + 140.0 * p.nx + 2500.0 * (S - 1);
+  return 10.0 * np + 8500.0 + 28.0 * p.nx + (S > 1 ? 900.0 + 1200.0 * (S - 1) : 0.0);
 }
 
 // the same of a 128 x 128 FP32 march: 54 k cycles with an SM to itself per CTA, 82 k with two

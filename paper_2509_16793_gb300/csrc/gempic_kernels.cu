@@ -2357,7 +2357,7 @@ __device__ void march(const Params& p, const Sm<T>& s_, const cg::cluster_group&
   // that the new fields will fill (the inverse transform of a row pair is in place), the
   // fixed-point accumulators share the column spectra, and a thread carries two modes whose old
   // level is read when it is needed.  A march then takes 82 k cycles a slice instead of 54 k, with
-  // twice as many in flight: 128 x 128 x 1024, 2 per cell, 14 s-steps in a call, 52.3 -> 42.7 ms.
+  // twice as many in flight: 128 x 128 x 1024, 2 per cell, 14 s-steps in a call, 52.3 -> 42.1 ms.
   constexpr bool DEN = SH == 2;
   constexpr int NM = DEN ? 2 : 1;                 // spectral modes per thread
   const bool varh = SH == 0 && p.varh != 0;
@@ -3687,7 +3687,12 @@ static cudaLaunchConfig_t make_cfg(const Params& p, int nclusters, cudaStream_t 
   cudaLaunchConfig_t c = {};
   c.gridDim = dim3((unsigned)(nclusters * p.C * p.split), 1, 1);
   c.blockDim = dim3((unsigned)p.nthreads, 1, 1);
-  c.dynamicSmemBytes = (size_t)p.smem_bytes;
+  // a split march's CTAs are small enough for two on an SM, and a pair that shares one holds up
+  // every march behind its own: 38 marches of 4 CTAs (128 cells, FP64, 256 slices) took 15.4 ms
+  // where 36 took 13.6.  Above half of an SM's shared memory they get an SM each, and the count of
+  // clusters that fit says so.
+  constexpr size_t kOwnSm = 116 * 1024;
+  c.dynamicSmemBytes = p.split > 1 ? std::max((size_t)p.smem_bytes, kOwnSm) : (size_t)p.smem_bytes;
   c.stream = s;
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = (unsigned)(p.C * p.split);
