@@ -59,7 +59,7 @@ struct gempic_sim {
   std::vector<double> px, py, pz, pux, puy, puz, pq;
   std::vector<int> psp;
   // gempic_step_streamed: input and output levels on the device (public layout), the
-  // host-mapped words [ready: pmax][done: pmax], the copy streams (out, in, and the first
+  // host-mapped words [ready: deepest + 1][done: deepest], the copy streams (out, in, and the first
   // s-step's input) and their events
   void* io_a = nullptr;
   void* io_b = nullptr;
@@ -360,10 +360,10 @@ double slice_cycles_128(const Params& p) { return p.dense ? 82000.0 : 54000.0; }
 
 // The launch of n s-steps: parameters with the shape and the number of marches in flight.  2-D
 // grids choose how many CTAs share a march by the modelled time of the wavefront: march c starts
-// when march c - 1 is a few slices ahead (kLag) and march c - P has finished.  Many s-steps fill
+// when march c - 1 is a few slices ahead (`lag`) and march c - P has finished.  Many s-steps fill
 // the chip with marches of one CTA; few s-steps (or one) leave SMs to share a march's particles.
-Params plan_launch(const gempic_sim* s, int n) {
-  constexpr double kLag = 4.0;
+constexpr double kLag = 4.0;
+Params plan_launch(const gempic_sim* s, int n, double lag = kLag) {
   const int depth = s->cfg.pipeline_depth;
   const Params* best = &s->p;
   int bestP = std::min(s->pmax, n);
@@ -373,12 +373,12 @@ Params plan_launch(const gempic_sim* s, int n) {
     if (depth > 0) P = std::min(P, depth);
     if (P < 1) continue;
     std::vector<double> end((size_t)P, 0.0);
-    double start = -kLag;
+    double start = -lag;
     for (int i = 0; i < n; ++i) {
-      start = std::max(start + kLag, end[i % P]);
+      start = std::max(start + lag, end[i % P]);
       end[i % P] = start + c.p.nz;
       if (i >= 4 * P && i % P == P - 1) {              // steady: the remaining waves alike
-        const double wave = std::max(P * kLag, (double)c.p.nz);
+        const double wave = std::max(P * lag, (double)c.p.nz);
         start += wave * ((n - 1 - i) / P);
         break;
       }
@@ -1175,8 +1175,8 @@ cudaError_t ensure_stream_io(gempic_sim* s) {
   if (!s->io_a) e = dalloc(s, &s->io_a, nb);
   if (e == cudaSuccess && !s->io_b) e = dalloc(s, &s->io_b, nb);
   if (e == cudaSuccess && !s->io_host) {
-    // [ready: pmax + 1][done: pmax]
-    const size_t words = 2 * (size_t)s->pmax + 1;
+    // [ready: deepest + 1][done: deepest]
+    const size_t words = 2 * (size_t)(s->p.ring - 2) + 1;
     void* h = nullptr;
     e = cudaHostAlloc(&h, words * sizeof(unsigned long long), cudaHostAllocMapped);
     if (e != cudaSuccess) return e;
@@ -1195,24 +1195,28 @@ cudaError_t ensure_stream_io(gempic_sim* s) {
 
 // Copy group j of the public layout [6][nz][ny][nx/2] between the host buffer and a device
 // level: blocks [lo, hi) are R_x, R_y, E_z, B_z at slices lo .. hi-1 (below nz) and j_x, j_y at
-// half-slices lo-1 .. hi-2 (from 0); one contiguous copy per component (measured faster than
-// strided two-dimensional copies of the same bytes).
+// half-slices lo-1 .. hi-2 (from 0).  One strided copy for the fields and one for the currents
+// (2.3 us of the calling thread a group; a copy per component took 6.4, 9 of 62 ms of a call of
+// 14 s-steps), in pieces where a component is longer than the largest pitch of such a copy.
 cudaError_t io_copy(gempic_sim* s, int j, int chunk, void* dev, void* host, bool out,
                     cudaStream_t st) {
   const int nz = s->p.nz;
   const size_t sb = (size_t)s->p.ny * (s->p.nx / 2) * 2 * s->eb;    // one slice of one component
   const size_t cb = (size_t)nz * sb;                                 // one component
   const int hi = nz + 1 - j * chunk, lo = std::max(0, hi - chunk);
-  char* d = (char*)dev;
-  char* h = (char*)host;
+  char* to = (char*)(out ? host : dev);
+  const char* from = (const char*)(out ? dev : host);
   const cudaMemcpyKind kind = out ? cudaMemcpyDeviceToHost : cudaMemcpyHostToDevice;
+  const int per = cb <= 0x7fffffff ? 6 : 1;                          // components per copy
   cudaError_t e = cudaSuccess;
-  for (int c = 0; c < 6 && e == cudaSuccess; ++c) {
+  for (int c = 0, m = 0; c < 6 && e == cudaSuccess; c += m) {
+    m = std::min(per, c < 4 ? 4 - c : 6 - c);
     const int s0 = c < 4 ? lo : std::max(lo, 1) - 1;                // fields / currents
     const int s1 = c < 4 ? std::min(hi, nz) : hi - 1;
     if (s1 <= s0) continue;
     const size_t off = (size_t)c * cb + (size_t)s0 * sb, w = (size_t)(s1 - s0) * sb;
-    e = out ? cudaMemcpyAsync(h + off, d + off, w, kind, st) : cudaMemcpyAsync(d + off, h + off, w, kind, st);
+    e = m > 1 ? cudaMemcpy2DAsync(to + off, cb, from + off, cb, w, (size_t)m, kind, st)
+              : cudaMemcpyAsync(to + off, from + off, w, kind, st);
   }
   return e;
 }
@@ -1237,21 +1241,32 @@ gempic_status gempic_step_streamed(gempic_sim* s, int32_t n, void* host, size_t 
   const size_t by_bytes = std::max<size_t>(1, ((size_t)8 << 20) / block_bytes);
   const int chunk = (int)std::max<size_t>(2, std::min<size_t>(by_bytes, (size_t)(nz + 8) / 8));
   const int nch = (nz + 1 + chunk - 1) / chunk;
+  // a copy from pageable memory may read it when it is issued, not in its stream's order
+  cudaPointerAttributes at{};
+  e = cudaPointerGetAttributes(&at, host);
+  if (e != cudaSuccess) return cuda_fail(s, e);
+  const bool pinned = at.type == cudaMemoryTypeHost;
+  // an s-step trails the one before it by a group (its copies out and in take less than a
+  // group's slices), which decides between the shapes: 14 s-steps of 128 x 128 x 1024 take 60 ms
+  // with 7 in flight and 57 with 14 (two CTAs per SM), 28 take 115 and 101; groups of 4 MiB
+  // 59, of 2 MiB 64, of 12 MiB 61.  2-D grids march in the simulation's own shape.
+  const int deepest = s->p.ring - 2;
   Params q = s->p;
+  if (s->p.ny > 1) q = plan_launch(s, n, chunk + kLag);
+  else q.P = std::min(s->pmax, n);
   q.k0 = s->k;
   q.nsteps = n;
-  q.P = std::min(s->pmax, n);
   q.inject = q.nspecies > 0 ? 1 : 0;
   q.delta_field = s->p.delta;
   q.state = s->io_a;
   q.state_out = s->io_b;
   q.io_ready = s->io_dev;
-  q.io_done = s->io_dev + s->pmax + 1;
+  q.io_done = s->io_dev + deepest + 1;
   q.io_chunk = chunk;
   q.io_nchunk = nch;
-  q.io_ring = s->pmax + 1;
+  q.io_ring = deepest + 1;
   unsigned long long* ready = s->io_host;
-  const unsigned long long* done = s->io_host + s->pmax + 1;
+  const unsigned long long* done = s->io_host + deepest + 1;
   const long long k0 = s->k;
   auto slot = [&](int i) { return i % q.P; };
   // the first s-step's input goes in before the launch's marches reach it, on a stream of
@@ -1272,9 +1287,10 @@ gempic_status gempic_step_streamed(gempic_sim* s, int32_t n, void* host, size_t 
     return cuda_fail(s, e);
   }
   // Drive the copies: a group of s-step i's result goes out once its march has written it,
-  // back in as s-step i+1's input once it is out, and is released to that march once it is
-  // in.  Each link waits for the one before it, so the host buffer and both device levels are
-  // only rewritten after their last reader is done.
+  // back in as s-step i+1's input once it is out (the second stream waits for the first's
+  // event), and is released to that march once it is in.  Each link waits for the one before
+  // it, so the host buffer and both device levels are only rewritten after their last reader
+  // is done.
   std::vector<int> next_out(n, 0), blocked;
   int first = 0, outs_done = 0;
   gempic_status result = GEMPIC_OK;
@@ -1297,6 +1313,15 @@ gempic_status gempic_step_streamed(gempic_sim* s, int32_t n, void* host, size_t 
         if (e == cudaSuccess) e = io_copy(s, j, chunk, s->io_b, host, true, s->io_out);
         if (e == cudaSuccess) e = cudaEventRecord(pd.ev, s->io_out);
         if (e == cudaSuccess) outq.push_back(pd);
+        if (e == cudaSuccess && i + 1 < n) {
+          IoPending nx{i + 1, j, nullptr};
+          e = io_event(s, &nx.ev);
+          if (e == cudaSuccess)
+            e = pinned ? cudaStreamWaitEvent(s->io_in, pd.ev, 0) : cudaEventSynchronize(pd.ev);
+          if (e == cudaSuccess) e = io_copy(s, j, chunk, s->io_a, host, false, s->io_in);
+          if (e == cudaSuccess) e = cudaEventRecord(nx.ev, s->io_in);
+          if (e == cudaSuccess) inq.push_back(nx);
+        }
         ++next_out[i];
         moved = true;
       }
@@ -1308,18 +1333,10 @@ gempic_status gempic_step_streamed(gempic_sim* s, int32_t n, void* host, size_t 
         e = qe;
         break;
       }
-      IoPending pd = outq.front();
+      s->io_events.push_back(outq.front().ev);
       outq.pop_front();
       ++outs_done;
       moved = true;
-      if (pd.step + 1 < n) {
-        IoPending nx{pd.step + 1, pd.group, pd.ev};
-        e = io_copy(s, pd.group, chunk, s->io_a, host, false, s->io_in);
-        if (e == cudaSuccess) e = cudaEventRecord(nx.ev, s->io_in);
-        if (e == cudaSuccess) inq.push_back(nx);
-      } else {
-        s->io_events.push_back(pd.ev);
-      }
     }
     // an s-step's groups are released in order (one word per s-step); the first s-step's
     // copies run on their own stream, so the next s-step's may finish before them

@@ -3760,6 +3760,7 @@ cudaError_t launch_import_state(int precision, const Params& p, const void* src,
 cudaError_t configure_march_canon(int precision, int smem) {
   if (precision == 64) return cfg_kernel(march_kernel<double, true>, smem);
   cudaError_t e = cfg_kernel(march_kernel<float, true>, smem);
+  if (e == cudaSuccess) e = cfg_kernel(march_kernel_dense<true>, smem);
   return e == cudaSuccess ? cfg_kernel(march_kernel<float, true, 1>, smem) : e;
 }
 
@@ -3767,6 +3768,7 @@ cudaError_t launch_march_canon(int precision, const Params& p, cudaStream_t s) {
   cudaLaunchAttribute attr[1];
   cudaLaunchConfig_t c = make_cfg(p, p.P, s, attr);
   if (precision == 64) return cudaLaunchKernelEx(&c, march_kernel<double, true>, p);
+  if (p.dense) return cudaLaunchKernelEx(&c, march_kernel_dense<true>, p);
   if (shape_class(precision, p) == 1) return cudaLaunchKernelEx(&c, march_kernel<float, true, 1>, p);
   return cudaLaunchKernelEx(&c, march_kernel<float, true>, p);
 }

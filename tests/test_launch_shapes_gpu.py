@@ -107,3 +107,25 @@ def test_128_two_ctas_per_sm_with_a_beam(G):
         da, db = a.diagnostics(), b.diagnostics()
         assert da["n_stored"] == db["n_stored"] > 0 and da["pushes"] == db["pushes"]
         assert abs(da["field_energy"] - db["field_energy"]) <= 1e-3 * db["field_energy"]
+
+
+@pytest.mark.parametrize("nz,n", [(640, 14), (637, 9), (640, 7)])
+def test_128_streamed_equal_single_steps(G, nz, n):
+    """Streamed calls that march with two CTAs per SM (and 7 s-steps, which do not, from pageable
+    memory); a ragged last group of slices."""
+    import torch
+    w = W.lwfa_3d_128x128x1024()
+    w = w.with_(nzeta=nz, laser=W.Laser(**{**w.laser.__dict__, "zeta_center": 0.5 * nz * w.h}))
+    with G.Sim(w) as a, G.Sim(w) as b:
+        host = a.state()
+        if n != 7:
+            pinned = torch.empty(host.shape, dtype=torch.complex64, pin_memory=True).numpy()
+            pinned[...] = host
+            host = pinned
+        diags = a.step_streamed(n, host)
+        for i in range(n):
+            b.step(1)
+            assert diags[i]["pushes"] == b.diagnostics()["pushes"]
+        assert np.array_equal(host, b.state())
+        assert np.array_equal(a.state(), host)
+        assert np.array_equal(a.onaxis_ez(), b.onaxis_ez())
