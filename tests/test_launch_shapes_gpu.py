@@ -73,7 +73,8 @@ def test_2d_shapes_equal_one_cta(G, option, precision, nx, ppc):
                 assert np.abs(a.current() - c.current()).max() <= tol * np.abs(a.current()).max()
 
 
-@pytest.mark.parametrize("nz,ppc,a0,n", [(120, 2, 1.0, 16), (96, 1, 1.5, 17), (90, 5, 1.0, 14)])
+@pytest.mark.parametrize("nz,ppc,a0,n", [(120, 2, 1.0, 16), (96, 1, 1.5, 17), (90, 5, 1.0, 14),
+                                           (300, 1, 1.0, 19)])
 def test_128_two_ctas_per_sm_equal_single_steps(G, nz, ppc, a0, n):
     """More s-steps than one CTA per SM keeps in flight: marches with two CTAs per SM."""
     w = W.lwfa_3d_128x128x1024()
