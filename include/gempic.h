@@ -215,7 +215,8 @@ gempic_status gempic_add_particles(struct gempic_sim* sim, int64_t n, const doub
                                    const double* uy, const double* uz, const double* weight,
                                    const int32_t* species);
 
-/* Advance n s-steps (one persistent device launch), then wait and check the device status. */
+/* Advance n s-steps (persistent device launches: one, or a few where the last wave of s-steps in
+ * flight would be nearly empty), then wait and check the device status. */
 gempic_status gempic_step(struct gempic_sim* sim, int32_t n);
 
 /* Same, without waiting: launches on the simulation's stream and returns. */

@@ -6,7 +6,8 @@
 //   * real-space rows y in [r RB, (r+1) RB) of every slice plane (fields for the gather,
 //     current accumulators for the deposit), and the fresh particles injected into them;
 //   * spectral columns kx in [r KB, (r+1) KB) for all ky (per-mode slice solve, App. B),
-//     with one mode per thread whose carried state lives in registers.
+//     with one mode per thread (two in the march with two CTAs per SM) whose carried state lives
+//     in registers.  In 2-D several CTAs may share a march's particles and repeat the rest.
 // Per slice n = nz-1 .. 0 (zeta_n = n h):
 //   A  gather E,B of slice n+1 at every streaming particle, push it to plane n along the GT2
 //      characteristics (two-pass Boris, budget rule of Eq. trap2), deposit the transverse
