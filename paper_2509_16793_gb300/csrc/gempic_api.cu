@@ -15,6 +15,7 @@
 
 #include "../../include/gempic.h"
 #include "gempic_internal.h"
+#include "gempic_plan.h"
 #include "gempic_setup.h"
 
 using gempic::Params;
@@ -366,18 +367,8 @@ constexpr double kLag = 4.0;
 
 // modelled cycles of n s-steps in shape c, P of them in flight
 double wavefront_cycles(const gempic_sim* s, const gempic_sim::Shape& c, int n, int P, double lag) {
-  std::vector<double> end((size_t)P, 0.0);
-  double start = -lag;
-  for (int i = 0; i < n; ++i) {
-    start = std::max(start + lag, end[i % P]);
-    end[i % P] = start + c.p.nz;
-    if (i >= 4 * P && i % P == P - 1) {                  // steady: the remaining waves alike
-      const double wave = std::max(P * lag, (double)c.p.nz);
-      start += wave * ((n - 1 - i) / P);
-      break;
-    }
-  }
-  return (start + c.p.nz) * (c.p.ny > 1 ? slice_cycles_128(c.p) : slice_cycles_2d(c.p, s->eb, c.p.split));
+  return gempic::wavefront_slices(n, P, c.p.nz, lag) *
+         (c.p.ny > 1 ? slice_cycles_128(c.p) : slice_cycles_2d(c.p, s->eb, c.p.split));
 }
 
 // With `count`, the launch may take only the first *count of the n s-steps, whole waves of its
