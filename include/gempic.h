@@ -314,11 +314,20 @@ gempic_status gempic_get_onaxis_ez(struct gempic_sim* sim, double* dst, int32_t 
 /* Device kernels this library launched since create (for launch accounting). */
 int64_t gempic_launch_count(const struct gempic_sim* sim);
 
-/* Launch shape of one s-step chosen at create (a call of several s-steps may spread a march over
- * other CTAs): CTAs per cluster, threads per CTA, dynamic shared bytes,
- * s-steps marched concurrently. */
+/* Launch shape that gempic_create chose for the simulation's own march (its initialisation, the
+ * denoised s-steps, the streamed s-steps of 2-D grids): CTAs per cluster, threads per CTA,
+ * dynamic shared bytes, s-steps marched concurrently.  A gempic_step call chooses among several
+ * shapes by its number of s-steps and may march another one, a single s-step included (2-D: 1 to 8
+ * CTAs share a march; 128 x 128 in FP32: up to twice as many s-steps in flight, two CTAs per SM);
+ * gempic_last_launch says which. */
 gempic_status gempic_launch_shape(const struct gempic_sim* sim, int32_t* cluster_ctas,
                                   int32_t* threads, int32_t* smem_bytes, int32_t* pipeline);
+
+/* Shape of the simulation's last launch: CTAs that share a march, threads per CTA, s-steps (or
+ * passes of denoised s-steps) in flight.  Any pointer may be NULL.  GEMPIC_ESTATE before the
+ * simulation has been initialised. */
+gempic_status gempic_last_launch(const struct gempic_sim* sim, int32_t* march_ctas,
+                                 int32_t* threads, int32_t* in_flight);
 
 /* ---- Batched parameter scan ------------------------------------------------------------
  * Independent simulations stepped together (the paper has no counterpart: a scan over grids,

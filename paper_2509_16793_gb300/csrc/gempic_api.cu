@@ -39,7 +39,8 @@ struct gempic_sim {
   // 2-D: the particles of a march on 1, 2, 4, 8 CTAs; FP32 128 x 128: one or two CTAs per SM
   struct Shape { Params p; int maxcl; };
   std::vector<Shape> shapes;
-  int nrank_last = 1;              // CTAs per march of the last launch (diagnostic partials)
+  // the last launch: CTAs per march (diagnostic partials), threads per CTA, marches in flight
+  int nrank_last = 1, threads_last = 0, inflight_last = 1;
   cudaStream_t stream = nullptr;
   long long k = 0;                 // s-steps completed
   bool initialized = false;
@@ -125,6 +126,12 @@ gempic_status check_device_error(gempic_sim* s) {
                          : GEMPIC_ESTATE;
   s->failed = st;
   return st;
+}
+
+void note_launch(gempic_sim* s, const Params& q) {
+  s->nrank_last = q.C * q.split;
+  s->threads_last = q.nthreads;
+  s->inflight_last = q.P;
 }
 
 cudaError_t ensure_diag_cap(gempic_sim* s, int n) {
@@ -252,7 +259,7 @@ gempic_status ensure_initialized(gempic_sim* s) {
   q.snapshot = 0;
   e = gempic::launch_march(prec, q, s->stream);
   s->launches++;
-  s->nrank_last = s->p.C;
+  note_launch(s, q);
   if (e != cudaSuccess) return cuda_fail(s, e);
   st = check_device_error(s);
   if (st != GEMPIC_OK) return st;
@@ -308,7 +315,9 @@ void batch_advance(gempic_sim* s, int n) {
   s->k += n;
   s->launches++;
   s->denoised_last = false;
-  s->nrank_last = s->p.C;
+  Params q = s->p;
+  q.P = n;
+  note_launch(s, q);
 }
 
 int batch_precision(const gempic_sim* s) { return s->cfg.precision; }
@@ -1011,7 +1020,7 @@ static gempic_status denoised_chain(gempic_sim* s, int n) {
   if (e != cudaSuccess) return cuda_fail(s, e);
   s->last_launch_k0 = k0;
   s->last_launch_n = 2 * n;
-  s->nrank_last = s->p.C;
+  note_launch(s, q);
   s->denoised_last = true;
   s->jcap_last = s->dn_jcap[(k0 + n - 1) & 3];
   s->k += n;
@@ -1042,7 +1051,7 @@ gempic_status gempic_step_async(gempic_sim* s, int32_t n) {
     q.inject = q.nspecies > 0 ? 1 : 0;
     q.delta_field = s->p.delta;
     e = gempic::launch_march(s->cfg.precision, q, s->stream);
-    s->nrank_last = q.C * q.split;
+    note_launch(s, q);
     s->launches++;
     if (e != cudaSuccess) return cuda_fail(s, e);
     s->last_launch_k0 = s->k;
@@ -1417,7 +1426,7 @@ gempic_status gempic_step_streamed(gempic_sim* s, int32_t n, void* host, size_t 
   if (e != cudaSuccess) return cuda_fail(s, e);
   s->last_launch_k0 = s->k;
   s->last_launch_n = n;
-  s->nrank_last = s->p.C;
+  note_launch(s, q);
   s->denoised_last = false;
   s->k += n;
   if (result != GEMPIC_OK) {
@@ -1609,6 +1618,16 @@ gempic_status gempic_launch_shape(const gempic_sim* s, int32_t* cluster_ctas, in
   if (threads) *threads = s->p.nthreads;
   if (smem_bytes) *smem_bytes = s->p.smem_bytes;
   if (pipeline) *pipeline = s->pmax;
+  return GEMPIC_OK;
+}
+
+gempic_status gempic_last_launch(const gempic_sim* s, int32_t* march_ctas, int32_t* threads,
+                                 int32_t* in_flight) {
+  if (!s) return GEMPIC_EINVAL;
+  if (!s->initialized) return GEMPIC_ESTATE;
+  if (march_ctas) *march_ctas = s->nrank_last;
+  if (threads) *threads = s->threads_last;
+  if (in_flight) *in_flight = s->inflight_last;
   return GEMPIC_OK;
 }
 

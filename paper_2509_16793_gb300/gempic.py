@@ -104,6 +104,7 @@ SIGNATURES = {
     "gempic_get_onaxis_ez": (c_int32, [c_void_p, c_void_p, c_int32]),
     "gempic_launch_count": (c_int64, [c_void_p]),
     "gempic_launch_shape": (c_int32, [c_void_p] + [POINTER(c_int32)] * 4),
+    "gempic_last_launch": (c_int32, [c_void_p] + [POINTER(c_int32)] * 3),
     "gempic_step_noalloc": (c_int32, [POINTER(gempic_config), c_int64, c_void_p, c_size_t,
                                        POINTER(gempic_diag), c_void_p]),
     "gempic_batch_create": (c_int32, [POINTER(gempic_config), c_int32, POINTER(c_void_p)]),
@@ -431,6 +432,11 @@ class Sim:
         _check(self.lib.gempic_launch_shape(self.h, *[byref(x) for x in v]), "gempic_launch_shape")
         return dict(cluster_ctas=v[0].value, threads=v[1].value, smem_bytes=v[2].value,
                     pipeline=v[3].value)
+
+    def last_launch(self) -> dict:
+        v = [c_int32() for _ in range(3)]
+        _check(self.lib.gempic_last_launch(self.h, *[byref(x) for x in v]), "gempic_last_launch")
+        return dict(march_ctas=v[0].value, threads=v[1].value, in_flight=v[2].value)
 
     def close(self):
         if getattr(self, "h", None) is not None and self.h.value:

@@ -1,0 +1,185 @@
+"""Which launch a call of s-steps takes, and that the taken ones agree: every case states the shape
+it is there for (Sim.last_launch) next to its results."""
+import numpy as np
+import pytest
+
+from paper_2509_16793_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def G():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.fail("GPU tests need a CUDA device")
+    from paper_2509_16793_gb300 import build, gempic
+    build.build()
+    return gempic
+
+
+def _lwfa(nz, ppc=2, a0=1.0, **kw):
+    w = W.lwfa_3d_128x128x1024()
+    return w.with_(nzeta=nz, species=[W.Species(-1.0, 1.0, w.species[0].density, ppc)],
+                   laser=W.Laser(**{**w.laser.__dict__, "a0": a0, "zeta_center": 0.5 * nz * w.h}), **kw)
+
+
+def _two_ctas_per_sm(sim):
+    """128 x 128 marches are 16 CTAs of 512 threads, or (two CTAs per SM) of 256."""
+    t = sim.last_launch()
+    assert t["march_ctas"] == 16 and t["threads"] in (256, 512)
+    return t["threads"] == 256
+
+
+# the diagnostics are FP32 sums over each thread's particles, added in FP64: other threads, other
+# groups of at most 16 slices' particles a thread, so the last bits differ
+DIAG_RTOL = 1e-5
+
+
+def _same_bits(a, b):
+    assert np.array_equal(a.state(), b.state())
+    assert np.array_equal(a.onaxis_ez(), b.onaxis_ez())
+    da, db = a.diagnostics(), b.diagnostics()
+    for k in ("n_trapped", "n_stored", "n_rejoined", "pushes", "step"):
+        assert da[k] == db[k], k
+    for k in ("field_energy", "kinetic_energy"):
+        assert abs(da[k] - db[k]) <= DIAG_RTOL * abs(db[k]), k
+
+
+def test_before_any_launch(G):
+    with G.Sim(W.small_2d(nzeta=16)) as s:
+        with pytest.raises(G.GempicError):
+            s.last_launch()
+        s.step(1)
+        assert s.last_launch()["in_flight"] == 1
+
+
+# particles beyond the free-slot stack (ppc 5: 5120 fresh slots a CTA), a strong laser, a density
+# channel; the plain runs of this grid never store a particle, so the bits are equal
+@pytest.mark.parametrize("nz,ppc,a0,n,channel", [(240, 5, 1.0, 14, None), (240, 1, 1.5, 14, None),
+                                                 (200, 2, 1.0, 10, (0.25, 20.0)),
+                                                 (220, 8, 0.5, 9, None)])
+def test_dense_march_equals_single_steps(G, nz, ppc, a0, n, channel):
+    w = _lwfa(nz, ppc, a0)
+    if channel:
+        w = w.with_(channel=W.Channel(*channel))
+    with G.Sim(w) as a, G.Sim(w) as b:
+        a.step(n)
+        assert _two_ctas_per_sm(a) and a.last_launch()["in_flight"] == n
+        for _ in range(n):
+            b.step(1)
+            assert not _two_ctas_per_sm(b)
+        _same_bits(a, b)
+
+
+@pytest.mark.parametrize("n", [14, 17])
+def test_dense_march_keeps_snapshot_and_current(G, n):
+    """Fields and currents of the last s-step: in the dense launch itself (14), and where the call
+    goes on in a second launch (17)."""
+    w = _lwfa(260, 2, 1.0, snapshot=True, capture_current=True)
+    with G.Sim(w) as a, G.Sim(w) as b:
+        launches = a.launch_count()
+        a.step(0)
+        init = a.launch_count() - launches
+        a.step(n)
+        assert a.launch_count() - launches - init == (1 if n == 14 else 2)
+        assert _two_ctas_per_sm(a) == (n == 14)
+        for _ in range(n):
+            b.step(1)
+        _same_bits(a, b)
+        for f in ("Ex", "Ez", "Bz", "jx", "jy", "jz"):
+            assert np.array_equal(a.fields(f), b.fields(f)), f
+        assert np.array_equal(a.current(), b.current())
+
+
+def test_dense_march_with_a_bunch(G):
+    """A bunch of more particles per slab than threads (the window of the fields), pushed, appended
+    and deposited by dense marches.  Stored particles deposit by FP32 reductions in global memory,
+    in any order: one rounding (2^-24) for each of the up to 10^3 contributions that a node takes."""
+    w = W.pwfa_3d_128x128x768(n_macro=1 << 15)
+    w = w.with_(nzeta=240, beam=W.Beam(**{**w.beam.__dict__, "n_peak": 0.05, "zeta_center": 120 * w.h,
+                                          "sigma_z": 0.4}))
+    with G.Sim(w) as a, G.Sim(w) as b:
+        a.step(14)
+        assert _two_ctas_per_sm(a)
+        for _ in range(14):
+            b.step(1)
+        assert not _two_ctas_per_sm(b)
+        sa, sb = a.state(), b.state()
+        assert np.abs(sa - sb).max() <= 1e-3 * np.abs(sb).max()
+        da, db = a.diagnostics(), b.diagnostics()
+        assert da["n_stored"] == db["n_stored"] > 20000 and da["pushes"] == db["pushes"]
+        assert abs(da["field_energy"] - db["field_energy"]) <= 1e-3 * db["field_energy"]
+
+
+def test_dense_march_with_rejoining_particles(G):
+    """A slow bunch: its particles (v_z = 0.75, budgets used up after some 17 slices) rejoin the
+    streaming ones in every s-step, in the dense march's slots.  A budget that ends within rounding
+    of a slice may end in its neighbour: 1 % of the counts."""
+    w = W.pwfa_3d_128x128x768(n_macro=1 << 12)
+    w = w.with_(nzeta=240, delta=1.0,
+                beam=W.Beam(**{**w.beam.__dict__, "n_peak": 0.01, "zeta_center": 220 * w.h,
+                               "sigma_z": 0.1, "gamma": 1.5, "rel_spread": 0.1}))
+    with G.Sim(w) as a, G.Sim(w) as b:
+        a.step(9)
+        assert _two_ctas_per_sm(a) and a.last_launch()["in_flight"] == 9
+        for _ in range(9):
+            b.step(1)
+        da, db = a.diagnostics(), b.diagnostics()
+        for k in ("n_trapped", "n_stored", "n_rejoined"):
+            assert db[k] > 1000 and abs(da[k] - db[k]) <= 2 + db[k] // 100, k
+        sa, sb = a.state(), b.state()
+        assert np.abs(sa - sb).max() <= 1e-3 * np.abs(sb).max()
+
+
+@pytest.mark.parametrize("nz,n", [(800, 14), (901, 10)])
+def test_dense_streamed_equals_single_steps(G, nz, n):
+    import torch
+    w = _lwfa(nz)
+    with G.Sim(w) as a, G.Sim(w) as b:
+        host = torch.empty(a.state_shape(), dtype=torch.complex64, pin_memory=True).numpy()
+        host[...] = a.state()
+        a.step_streamed(n, host)
+        assert _two_ctas_per_sm(a)
+        for _ in range(n):
+            b.step(1)
+        assert np.array_equal(host, b.state())
+        _same_bits(a, b)
+
+
+def test_streamed_2d_with_many_marches(G):
+    """More than 16 streamed 2-D s-steps in flight."""
+    import torch
+    w = W.small_2d(nx=64, nzeta=300, ppc=2, precision=32, a0=0.5, delta=5.0)
+    with G.Sim(w) as a, G.Sim(w) as b:
+        host = torch.empty(a.state_shape(), dtype=torch.complex64, pin_memory=True).numpy()
+        host[...] = a.state()
+        a.step_streamed(40, host)
+        assert a.last_launch()["in_flight"] > 16 and a.last_launch()["march_ctas"] == 1
+        for _ in range(40):
+            b.step(1)
+        assert np.array_equal(host, b.state())
+
+
+@pytest.mark.parametrize("option", ["trapping", "gt1", "beam"])
+def test_split_fp32_marches_with_stored_particles(G, option):
+    """FP32 marches whose particles several CTAs share, with stored particles, against the FP64
+    march of one CTA: as far from it as the FP32 march of one CTA is, to a factor of 10 (both are
+    FP32 runs of the same scheme, with the reductions of the stored particles in another order)."""
+    kw = {"trapping": dict(delta=3.0), "gt1": dict(particle_law="GT1", delta=8.0),
+          "beam": dict(beam=W.Beam(n_peak=0.002, sigma_r=3.0, sigma_z=1.5, zeta_center=8.0,
+                                   gamma=200.0, n_macro=500))}[option]
+    states = []
+    for prec, ctas in ((64, 1), (32, 1), (32, 0)):
+        w = W.small_2d(nx=128, nzeta=50, ppc=4, precision=prec, a0=2.0, delta=20.0).with_(**kw)
+        with G.Sim(w, cluster_ctas=ctas, bucket_capacity=4096) as s:
+            s.step(1)
+            assert (s.last_launch()["march_ctas"] > 1) == (ctas == 0)
+            s.step(1)
+            d = s.diagnostics()
+            assert d["n_stored"] + d["n_trapped"] > 0
+            states.append(s.state().astype(np.complex128))
+    ref, one, split = states
+    for part in (slice(0, 4), slice(4, 6)):
+        own = np.abs(one[part] - ref[part]).max()
+        assert np.abs(split[part] - ref[part]).max() <= 10.0 * own
