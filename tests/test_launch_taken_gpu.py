@@ -92,21 +92,32 @@ def test_dense_march_keeps_snapshot_and_current(G, n):
         assert np.array_equal(a.current(), b.current())
 
 
+def _runs_apart(sims, n):
+    """(state of the first, largest difference among the others) of simulations of one workload: the
+    first does n s-steps in one call, the others one at a time.  Stored particles deposit by FP32
+    reductions in global memory in whatever order they come, which the plasma then amplifies: two
+    runs of the same launches differ, and the spread of three says by how much."""
+    sims[0].step(n)
+    for s in sims[1:]:
+        for _ in range(n):
+            s.step(1)
+        assert not _two_ctas_per_sm(s)
+    st = [s.state() for s in sims[1:]]
+    return st[0], max(np.abs(x - y).max() for i, x in enumerate(st) for y in st[:i])
+
+
 def test_dense_march_with_a_bunch(G):
     """A bunch of more particles per slab than threads (the window of the fields), pushed, appended
-    and deposited by dense marches.  Stored particles deposit by FP32 reductions in global memory,
-    in any order: one rounding (2^-24) for each of the up to 10^3 contributions that a node takes."""
+    and deposited by dense marches, is no further from single steps than 4 times as far as those
+    are from each other."""
     w = W.pwfa_3d_128x128x768(n_macro=1 << 15)
     w = w.with_(nzeta=240, beam=W.Beam(**{**w.beam.__dict__, "n_peak": 0.05, "zeta_center": 120 * w.h,
                                           "sigma_z": 0.4}))
-    with G.Sim(w) as a, G.Sim(w) as b:
-        a.step(14)
+    with G.Sim(w) as a, G.Sim(w) as b, G.Sim(w) as c, G.Sim(w) as d:
+        ref, apart = _runs_apart((a, b, c, d), 14)
         assert _two_ctas_per_sm(a)
-        for _ in range(14):
-            b.step(1)
-        assert not _two_ctas_per_sm(b)
-        sa, sb = a.state(), b.state()
-        assert np.abs(sa - sb).max() <= 1e-3 * np.abs(sb).max()
+        assert 0 < apart <= 1e-2 * np.abs(ref).max()
+        assert np.abs(a.state() - ref).max() <= 4 * apart
         da, db = a.diagnostics(), b.diagnostics()
         assert da["n_stored"] == db["n_stored"] > 20000 and da["pushes"] == db["pushes"]
         assert abs(da["field_energy"] - db["field_energy"]) <= 1e-3 * db["field_energy"]
@@ -120,16 +131,13 @@ def test_dense_march_with_rejoining_particles(G):
     w = w.with_(nzeta=240, delta=1.0,
                 beam=W.Beam(**{**w.beam.__dict__, "n_peak": 0.01, "zeta_center": 220 * w.h,
                                "sigma_z": 0.1, "gamma": 1.5, "rel_spread": 0.1}))
-    with G.Sim(w) as a, G.Sim(w) as b:
-        a.step(9)
+    with G.Sim(w) as a, G.Sim(w) as b, G.Sim(w) as c, G.Sim(w) as d:
+        ref, apart = _runs_apart((a, b, c, d), 9)
         assert _two_ctas_per_sm(a) and a.last_launch()["in_flight"] == 9
-        for _ in range(9):
-            b.step(1)
         da, db = a.diagnostics(), b.diagnostics()
         for k in ("n_trapped", "n_stored", "n_rejoined"):
             assert db[k] > 1000 and abs(da[k] - db[k]) <= 2 + db[k] // 100, k
-        sa, sb = a.state(), b.state()
-        assert np.abs(sa - sb).max() <= 1e-3 * np.abs(sb).max()
+        assert np.abs(a.state() - ref).max() <= 4 * apart + 1e-6 * np.abs(ref).max()
 
 
 @pytest.mark.parametrize("nz,n", [(800, 14), (901, 10)])
