@@ -36,7 +36,8 @@ struct gempic_sim {
   int eb = 8;                      // bytes per real
   int pmax = 1;                    // concurrent marches of p's launch shape
   // launch shapes that a call of several s-steps chooses from (plan_launch); empty: only p's.
-  // 2-D: the particles of a march on 1, 2, 4, 8 CTAs; FP32 128 x 128: one or two CTAs per SM
+  // 2-D: the particles of a march on 1, 2, 4, 8 CTAs; FP32 128 x 128: one or two CTAs per SM;
+  // other 3-D grids: the cluster sizes up to p's
   struct Shape { Params p; int maxcl; };
   std::vector<Shape> shapes;
   // the last launch: CTAs per march (diagnostic partials), threads per CTA, marches in flight
@@ -137,7 +138,8 @@ void note_launch(gempic_sim* s, const Params& q) {
 cudaError_t ensure_diag_cap(gempic_sim* s, int n) {
   if (n <= s->diag_cap) return cudaSuccess;
   double *d = nullptr, *o = nullptr, *r = nullptr, *gr = nullptr;
-  cudaError_t e = dalloc(s, &d, (size_t)n * gempic::kNDiag * std::max(s->p.C, s->p.ny == 1 ? kMaxSplit : 1) * sizeof(double));
+  cudaError_t e = dalloc(s, &d, (size_t)n * gempic::kNDiag * std::max(s->p.C, s->p.ny == 1 ? kMaxSplit : 1) *
+                                    sizeof(double));
   if (e != cudaSuccess) return e;
   e = dalloc(s, &o, (size_t)n * s->p.nz * sizeof(double));
   if (e != cudaSuccess) return e;
@@ -354,84 +356,40 @@ int pick_threads(int precision, int M, int fresh) {
   return std::min(512, std::max(std::max(M, 128), (std::min(most, fresh) + 31) / 32 * 32));
 }
 
-// cycles of one slice of a 2-D march on S CTAs, fitted to lone marches of 64 to 1024 cells: the
-// push (FP64 bound by the SM's two lanes, FP32 by issue) divides, transforms and solve do not,
-// and each further CTA adds to the cluster barriers and to the sum over the CTAs.  FP64, 128
-// cells, 4 per cell on 1, 2, 4, 8 CTAs: 140, 90, 72, 71 k; FP32, 512 cells: 39, 31, 27, 30 k.
-double slice_cycles_2d(const Params& p, int eb, int S) {
-  const double np = (double)p.nx * p.ppc_sum / S;
-  if (eb == 8) return 200.0 * np + 18000.0 + 140.0 * p.nx + 2500.0 * (S - 1);
-  return 10.0 * np + 8500.0 + 28.0 * p.nx + (S > 1 ? 900.0 + 1200.0 * (S - 1) : 0.0);
-}
-
-// the same of a 128 x 128 FP32 march: 54 k cycles with an SM to itself per CTA, 82 k with two
-// CTAs per SM and 14 marches in flight
-double slice_cycles_128(const Params& p) { return p.dense ? 82000.0 : 54000.0; }
-
-// The launch of n s-steps: parameters with the shape and the number of marches in flight.  2-D
-// grids choose how many CTAs share a march by the modelled time of the wavefront: march c starts
-// when march c - 1 is a few slices ahead (`lag`) and march c - P has finished.  Many s-steps fill
-// the chip with marches of one CTA; few s-steps (or one) leave SMs to share a march's particles.
+// The launch of n s-steps: parameters with the shape and the number of marches in flight, by the
+// modelled time of the wavefront (gempic_plan.h): march c starts when march c - 1 is a few slices
+// ahead (`lag`) and march c - P has finished.  Many s-steps fill the chip with marches of few CTAs;
+// few s-steps (or one) leave SMs to spread a march over.
 constexpr double kLag = 4.0;
 
-// modelled cycles of n s-steps in shape c, P of them in flight
-double wavefront_cycles(const gempic_sim* s, const gempic_sim::Shape& c, int n, int P, double lag) {
-  return gempic::wavefront_slices(n, P, c.p.nz, lag) *
-         (c.p.ny > 1 ? slice_cycles_128(c.p) : slice_cycles_2d(c.p, s->eb, c.p.split));
+// q with the launch shape of b: decomposition, threads and shared-memory layout
+void take_shape(Params& q, const Params& b, int eb) {
+  q.C = b.C;
+  q.RB = b.RB;
+  q.KB = b.KB;
+  q.logRB = b.logRB;
+  q.logKB = b.logKB;
+  q.M = b.M;
+  q.split = b.split;
+  q.dense = b.dense;
+  q.nthreads = b.nthreads;
+  q.pcap = b.pcap;
+  q.gcap = b.gcap;
+  gempic::smem_layout(q, eb);
 }
 
-// With `count`, the launch may take only the first *count of the n s-steps, whole waves of its
-// shape, and leave a last wave that would be nearly empty to a launch of another shape.
+// With `count`, the launch may take only the first *count of the n s-steps (pick_shape).
 Params plan_launch(const gempic_sim* s, int n, double lag = kLag, int* count = nullptr) {
-  const int depth = s->cfg.pipeline_depth;
-  const auto in_flight = [&](const gempic_sim::Shape& c, int m) {
-    const int P = std::min(m, c.maxcl);
-    return depth > 0 ? std::min(P, depth) : P;
-  };
-  const auto shortest = [&](int m, const gempic_sim::Shape** which) {
-    double t0 = -1.0;
-    for (const gempic_sim::Shape& c : s->shapes) {
-      const int P = in_flight(c, m);
-      if (P < 1) continue;
-      const double t = wavefront_cycles(s, c, m, P, lag);
-      if (t0 < 0 || t < t0) {
-        t0 = t;
-        *which = &c;
-      }
-    }
-    return t0;
-  };
-  const gempic_sim::Shape *shape = nullptr, *other = nullptr;
-  double t = shortest(n, &shape);
-  int m = n;
-  if (count) {
-    for (const gempic_sim::Shape& c : s->shapes) {
-      const int P = in_flight(c, n);
-      if (P < 1 || P == n || n % P == 0) continue;
-      const int whole = n - n % P;
-      const double tc = wavefront_cycles(s, c, whole, P, lag) + shortest(n - whole, &other);
-      if (tc < 0.98 * t) {
-        t = tc;
-        shape = &c;
-        m = whole;
-      }
-    }
-    *count = m;
-  }
-  const Params* best = shape ? &shape->p : &s->p;
-  const int bestP = shape ? in_flight(*shape, m) : std::min(s->pmax, n);
+  std::vector<gempic::ShapeTime> t;
+  for (const gempic_sim::Shape& c : s->shapes)
+    t.push_back({gempic::slice_cycles({c.p.nx, c.p.ny, c.p.ppc_sum, s->eb, c.p.C, c.p.split, c.p.dense,
+                                       c.p.smem_bytes}),
+                 c.maxcl});
+  const gempic::Pick k = gempic::pick_shape(t, n, s->p.nz, lag, s->cfg.pipeline_depth, count != nullptr);
   Params q = s->p;
-  if (best != &s->p) {
-    // the shape: split, threads and shared-memory layout; everything else is the simulation's
-    const Params& b = *best;
-    q.split = b.split;
-    q.dense = b.dense;
-    q.nthreads = b.nthreads;
-    q.pcap = b.pcap;
-    q.gcap = b.gcap;
-    gempic::smem_layout(q, s->eb);
-  }
-  q.P = bestP;
+  if (k.shape >= 0) take_shape(q, s->shapes[k.shape].p, s->eb);
+  q.P = k.shape >= 0 ? k.in_flight : std::min(s->pmax, n);
+  if (count) *count = k.shape >= 0 ? k.count : n;
   return q;
 }
 
@@ -546,6 +504,7 @@ gempic_status create_sim(const gempic_config* cfg, gempic_sim** out, bool one_ct
   const int nxh = g.nx / 2;
   const int C = cfg->cluster_ctas;
   bool chosen = false;
+  std::vector<Params> sizes;                       // the cluster sizes that hold a slice
   for (int cand = (C > 0 ? C : 1); cand <= (C > 0 ? C : 16); cand *= 2) {
     if (g.ny % cand || nxh % cand) continue;
     if (g.ny == 1 && cand != 1) continue;
@@ -558,8 +517,9 @@ gempic_status create_sim(const gempic_config* cfg, gempic_sim** out, bool one_ct
     // by the CTAs, the barriers do not grow.  ms per s-step of one march, 96 slices, 2 per cell,
     // C = 1, 2, 4, 8, 16: 16 x 16 FP32 1.31 1.11 1.10 1.05 -; 32 x 32 FP32 3.19 1.69 1.24 1.07 1.09;
     // 64 x 64 FP32 - - 2.98 1.65 1.27; 32 x 32 FP64 - 21.1 11.4 6.9 5.1.  Clusters of 16 leave room
-    // for 7 to 14 marches where those of 8 leave 15 or more (64 x 64 FP32 with 48 s-steps in a call:
-    // 0.133 ms per s-step with 8, 0.174 with 16), so they want more work per CTA
+    // for 7 marches where those of 8 leave 15: the simulation's own shape is the largest that still
+    // has work for its CTAs, and a call of many s-steps takes a smaller one (plan_launch).  ms for
+    // 48 s-steps of 200 slices on 8 and 16: 64 x 64 13.0, 17.3; 128 x 64 with 8 per cell 47.2, 58.9.
     if (chosen && fresh < (cand <= 8 ? 64 : cfg->precision == 64 ? 128 : 512)) break;
     Params t = p;
     t.C = cand;
@@ -591,6 +551,7 @@ gempic_status create_sim(const gempic_config* cfg, gempic_sim** out, bool one_ct
     }
     if (!fits) continue;
     p = t;
+    sizes.push_back(t);
     chosen = true;
     if (one_cta) break;
   }
@@ -654,7 +615,7 @@ gempic_status create_sim(const gempic_config* cfg, gempic_sim** out, bool one_ct
   // taken, the rings of s-levels (stored particles, rejoin queues, beam current) may take 16 GiB.
   const double level_bytes = (double)g.nzeta * (2.0 * p.bcap * (4 + 7 * s->eb) + 3.0 * g.nx * g.ny * s->eb);
   const int levels = (int)std::min(128.0, 17179869184.0 / level_bytes) - 2;
-  const int deepest = s->shapes.empty() ? 16 : std::max(16, std::min(std::min(64, g.nzeta / 4), levels));
+  const int deepest = g.ny > 1 || s->shapes.empty() ? 16 : std::max(16, std::min(std::min(64, g.nzeta / 4), levels));
   s->pmax = cfg->pipeline_depth > 0 ? cfg->pipeline_depth : std::max(1, std::min(maxcl, deepest));
   if (s->pmax > std::max(1, maxcl)) s->pmax = std::max(1, maxcl);
   for (gempic_sim::Shape& sh : s->shapes) sh.maxcl = std::min(sh.maxcl, s->pmax);
@@ -662,6 +623,26 @@ gempic_status create_sim(const gempic_config* cfg, gempic_sim** out, bool one_ct
   // beyond their shared-memory capacity into these
   p.gcap = std::max(1024, g.nx * (g.ny / p.C) * std::max(ppc_sum, 1) * 2);
   for (gempic_sim::Shape& sh : s->shapes) sh.p.gcap = p.gcap;
+  if (g.ny > 1 && C == 0 && !one_cta && sizes.size() > 1) {
+    // 3-D: the cluster sizes a launch chooses from (plan_launch).  A CTA of any of them holds as
+    // many particles as one of the smallest, whose band holds the bands of the others: no shape
+    // overflows where another does not.
+    const int hold = sizes[0].pcap + std::max(1024, g.nx * sizes[0].RB * std::max(ppc_sum, 1) * 2);
+    p.gcap = std::max(p.gcap, hold - p.pcap);
+    for (const Params& t : sizes) {
+      gempic_sim::Shape sh{p, 0};
+      take_shape(sh.p, t, s->eb);
+      sh.p.gcap = t.C == p.C ? p.gcap : hold - t.pcap;
+      e = gempic::max_active_clusters(cfg->precision, sh.p, &sh.maxcl);
+      if (e != cudaSuccess) {
+        delete s;
+        return GEMPIC_ECUDA;
+      }
+      sh.maxcl = std::min(sh.maxcl, 16);
+      if (cfg->pipeline_depth > 0) sh.maxcl = std::min(sh.maxcl, cfg->pipeline_depth);
+      s->shapes.push_back(sh);
+    }
+  }
   if (C == 0 && !one_cta && gempic::dense_ok(cfg->precision, p) && cfg->particle_headroom <= 0) {
     // 128 x 128 FP32: two CTAs per SM where more s-steps are in flight than one per SM allows;
     // as many particle slots per CTA as p's in shared memory and overflow together

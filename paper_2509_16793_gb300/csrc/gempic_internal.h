@@ -81,7 +81,8 @@ struct Params {
   int o_f0, o_f1, o_j, o_recv, o_sr, o_jint, o_sc, o_workB, o_workD, o_tw, o_inbox, o_outbox, o_part, o_misc, o_dd,
       smem_bytes;
   // device memory
-  void* state;                    // blocks [nz+1][C][6][M] complex
+  void* state;                    // blocks [nz+1][6][C][M] complex (C M = (nx/2) ny: the same for
+                                  // every cluster size, so launches of other sizes may follow)
   unsigned long long* progress;   // [P] completed-iteration counters
   int* err;
   const void* tables;             // twx[nx/2], twy[ny/2], shx[nx/2], shy[ny], kx[nx/2], ky[ny]

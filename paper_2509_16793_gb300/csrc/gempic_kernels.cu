@@ -2336,7 +2336,7 @@ __device__ __forceinline__ void wait_input(const Params& p, long long k, int b, 
 // ------------------------------------------------------------------------------------------
 // the march of one s-step k (computes level k+1)
 // ------------------------------------------------------------------------------------------
-// CANON = false: the library's block layout [nz+1][C][6][M].  CANON = true: the public layout
+// CANON = false: the library's block layout [nz+1][6][C][M].  CANON = true: the public layout
 // of gempic_get_state ([6][nz][ny][nx/2]; j at half-slice index n <-> block n+1), used by the
 // allocation-free entry point on a caller's buffer.
 // DN: the march of a denoised chain (its hooks are compiled into the chain's instantiations
@@ -2536,7 +2536,9 @@ __device__ void march(const Params& p, const Sm<T>& s_, const cg::cluster_group&
       const int sl_ = c < 4 ? b : b - 1;
       return (((size_t)c * p.nz + sl_) * p.ny + kyi[j]) * (size_t)nxh + kxg;
     } else {
-      return (((size_t)b * p.C + me) * 6 + c) * (size_t)p.M + tid + j * NT;
+      // (SH >= 1: 64 x 128 modes, 512 per CTA)
+      const int modes = SH >= 1 ? 64 * 128 : nxh * p.ny, m0 = me * (SH >= 1 ? 512 : p.M);
+      return (size_t)(b * 6 + c) * (size_t)modes + (size_t)(m0 + tid + j * NT);
     }
   };
   // the public layout has no ghost slice and no j at half-slice -1
@@ -3449,7 +3451,7 @@ __global__ void __launch_bounds__(512, 1)
       if (p.ny > 1 && ky_of_pos(p.logny, q) == p.ny / 2) v = cx<T>(T(0), T(0));
       const Cx<T> z = cx<T>(T(0), T(0));
       for (int c = 0; c < 6; ++c)
-        stw[(((size_t)n * p.C + me) * 6 + c) * p.M + m] = (c == pol) ? v : z;
+        stw[(((size_t)n * 6 + c) * p.C + me) * p.M + m] = (c == pol) ? v : z;
     }
     cl.sync();
   }
@@ -3521,7 +3523,7 @@ __global__ void beam_kernel(const Params p, BeamArgs b) {
 }
 
 // ------------------------------------------------------------------------------------------
-// layout conversion of the spectral state: blocks [nz+1][C][6][M] <-> [6][nz][ny][nx/2]
+// layout conversion of the spectral state: blocks [nz+1][6][C][M] <-> [6][nz][ny][nx/2]
 // ------------------------------------------------------------------------------------------
 template <typename T>
 __global__ void export_kernel(const Params p, Cx<T>* dst, const Cx<T>* src, int dir) {
@@ -3535,7 +3537,7 @@ __global__ void export_kernel(const Params p, Cx<T>* dst, const Cx<T>* src, int 
     const int c = (int)(i / (nxh * p.ny * p.nz));
     const int b = c >= 4 ? n + 1 : n;
     const int r = kx / p.KB, kxl = kx % p.KB;
-    const size_t e = (((size_t)b * p.C + r) * 6 + c) * p.M + (size_t)kxl * p.ny +
+    const size_t e = (((size_t)b * 6 + c) * p.C + r) * p.M + (size_t)kxl * p.ny +
                      pos_of_ky(p.logny, ky);
     if (dir == 0)
       dst[i] = src[e];

@@ -191,3 +191,39 @@ def test_split_fp32_marches_with_stored_particles(G, option):
     for part in (slice(0, 4), slice(4, 6)):
         own = np.abs(one[part] - ref[part]).max()
         assert np.abs(split[part] - ref[part]).max() <= 10.0 * own
+
+
+@pytest.mark.parametrize("nx,ny,ppc,precision", [(64, 64, 2, 32), (128, 64, 1, 32), (64, 128, 3, 32),
+                                                 (64, 64, 2, 64)])
+def test_3d_cluster_sizes_agree(G, nx, ny, ppc, precision):
+    """Calls of many s-steps march on smaller clusters than single ones, streamed ones as well; the
+    state and the stored set pass from one to the other.  The sums of a halo row's fixed-point
+    currents are converted to FP32 band by band: one rounding more or less for a node and slice
+    (6e-8), of which a state value takes up some hundred."""
+    import torch
+    w = W.small_3d(nx=nx, ny=ny, nzeta=120, ppc=ppc, precision=precision, a0=1.0)
+    tol = 1e-5 if precision == 32 else 1e-11
+    with G.Sim(w) as a, G.Sim(w) as b:
+        for _ in range(2):                           # 15 together, one alone: there and back
+            a.step(15)
+            many = a.last_launch()
+            a.step(1)
+            assert many["march_ctas"] < a.last_launch()["march_ctas"] == a.launch_shape()["cluster_ctas"]
+            for _ in range(16):
+                b.step(1)
+            ra, rb = a.state(), b.state()
+            for part in (slice(0, 4), slice(4, 6)):
+                assert np.abs(ra[part] - rb[part]).max() <= tol * np.abs(rb[part]).max()
+            da, db = a.diagnostics(), b.diagnostics()
+            for k in ("n_trapped", "n_stored", "n_rejoined", "pushes", "step"):
+                assert da[k] == db[k], k
+        host = torch.empty(a.state_shape(), pin_memory=True,
+                           dtype=torch.complex128 if precision == 64 else torch.complex64).numpy()
+        host[...] = a.state()
+        d = a.step_streamed(12, host)
+        for i in range(12):
+            b.step(1)
+            assert d[i]["pushes"] == b.diagnostics()["pushes"]
+        rb = b.state()
+        for part in (slice(0, 4), slice(4, 6)):
+            assert np.abs(host[part] - rb[part]).max() <= 2 * tol * np.abs(rb[part]).max()
