@@ -468,7 +468,8 @@ void gempic_denoiser_destroy(gempic_denoiser* d);
  * of each one, which the march produces only one at a time.  The n s-steps of a call run as
  * one chain of 2n marches in one launch, each following the one before it slice by slice; up
  * to min(7, pipeline_depth) in flight, or, with pipeline_depth 0, as many as leave a quarter of
- * the SMs to the net.  The calling thread runs the net on groups of half-slices as soon as the
+ * the SMs to the net (slices of 4096 nodes and more in rows of other than 128: a third, and
+ * the marches take clusters that leave it half where there is a choice).  The calling thread runs the net on groups of half-slices as soon as the
  * first pass has written them and the three half-slices beyond, on a stream of its own, and
  * releases each group to the second pass, which waits for it (bounded).  The call waits for
  * its stream.  The diagnostics combine both passes: the field energy, on-axis E_z and stored

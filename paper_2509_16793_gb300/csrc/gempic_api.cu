@@ -881,25 +881,39 @@ static gempic_status denoised_chain(gempic_sim* s, int n) {
   const int lead = 3 % chunk;
   // at most 7 marches in flight: the first pass of s-step i+4 reuses the current buffers of
   // s-step i only after it starts, i.e. after march 2i+8-P, the second pass of s-step i or later,
-  // has finished with them.  The net runs on the SMs the marches leave free: unless the
-  // configuration sets the depth, the marches take at most three quarters of them (on GB300 at
-  // 128 x 128 x 512, 1 ppc, 7 s-steps, the chain's time per s-step against its depth is 7.5, 6.7,
-  // 5.3, 5.2 and 4.1 ms for 3 to 7 clusters of 16 CTAs; with the net twice as slow 7 of them
-  // starved it, 7.3 ms against 5.3 with 6).
+  // has finished with them.  The net runs on the SMs the marches leave free.  Rows of 128 voxels
+  // (the net's row kernel): at most three quarters of the SMs to the marches unless the
+  // configuration sets the depth (on GB300 at 128 x 128 x 512, 1 ppc, 7 s-steps, the chain's time
+  // per s-step against its depth is 7.5, 6.7, 5.3, 5.2 and 4.1 ms for 3 to 7 clusters of 16 CTAs).
+  // Other rows take the net's gather kernel, several times slower a voxel, which on slices of 4096
+  // nodes and more 7 clusters of 16 starve: there the marches take the largest clusters that fit
+  // half of the SMs, and two thirds where there is only one size (64 x 128 x 256, 7 s-steps: 7
+  // clusters of 16 27.5 ms, 6 23.1, 7 of 8 18.1; 1 s-step, two marches: clusters of 16 4.9, of 8
+  // 7.0; 32 x 32, 7 s-steps: 7 clusters of 16 8.0, 6 9.8).
   int dev = 0, nsm = 0;
   e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return cuda_fail(s, e);
+  const bool gathers = s->p.nx != 128 && s->p.ny > 1 && s->p.nx * s->p.ny >= 4096;
+  Params q = s->p;
+  int most = s->pmax;
+  if (gathers) {
+    for (const gempic_sim::Shape& c : s->shapes) {           // (in ascending order of size)
+      const int P = std::min(std::min(2 * n, 7), c.maxcl);
+      if (&c != &s->shapes[0] && 2 * P * c.p.C > nsm) break;
+      take_shape(q, c.p, s->eb);
+      most = c.maxcl;
+    }
+  }
   const int want = s->cfg.pipeline_depth > 0 ? s->cfg.pipeline_depth
-                                             : std::max(1, 3 * nsm / (4 * s->p.C));
-  const int P = std::min(std::min(std::min(s->pmax, 2 * n), 7), want);
+                                             : std::max(1, gathers ? 2 * nsm / (3 * q.C) : 3 * nsm / (4 * q.C));
+  const int P = std::min(std::min(std::min(most, 2 * n), 7), want);
   const long long k0 = s->k;
   unsigned long long* done = s->dn_host;
   unsigned long long* ready = s->dn_host + 8;
   std::memset(s->dn_host, 0, 16 * sizeof(unsigned long long));
   // progress words carry march indices here: start from zero
-  e = cudaMemsetAsync(s->p.progress, 0, (size_t)s->pmax * sizeof(unsigned long long), s->stream);
-  Params q = s->p;
+  e = cudaMemsetAsync(s->p.progress, 0, (size_t)P * sizeof(unsigned long long), s->stream);
   q.k0 = k0;
   q.nsteps = 2 * n;
   q.P = P;
@@ -996,7 +1010,7 @@ static gempic_status denoised_chain(gempic_sim* s, int n) {
   if (e == cudaSuccess) e = e2 != cudaSuccess ? e2 : e3;
   // leave the progress words as a plain launch expects them (below any s-step's value)
   if (e == cudaSuccess)
-    e = cudaMemsetAsync(s->p.progress, 0, (size_t)s->pmax * sizeof(unsigned long long), s->stream);
+    e = cudaMemsetAsync(s->p.progress, 0, (size_t)P * sizeof(unsigned long long), s->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
   if (e != cudaSuccess) return cuda_fail(s, e);
   s->last_launch_k0 = k0;
