@@ -28,9 +28,13 @@ inline double slice_cycles_2d(const SliceWork& w) {
   return 10.0 * np + 8500.0 + 28.0 * w.nx + (S > 1 ? 900.0 + 1200.0 * (S - 1) : 0.0);
 }
 
-// 128 x 128 FP32: 54 k cycles with an SM to itself per CTA, 82 k with two CTAs per SM and 14 marches
-// in flight
-inline double slice_cycles_128(const SliceWork& w) { return w.dense ? 82000.0 : 54000.0; }
+// 128 x 128 FP32, fitted to 7 marches in flight with an SM to each CTA and to 8 to 14 with two CTAs
+// per SM (whose slices take the shared pace as soon as some SMs hold two), 512 slices: 40, 48, 65, 100,
+// 169 k cycles with 1, 2, 4, 8, 16 per cell, and 56, 71, 100, 161, 299 k (one species or two; a bunch
+// adds the same share to both)
+inline double slice_cycles_128(const SliceWork& w) {
+  return w.dense ? 42500.0 + 14700.0 * w.ppc : 30600.0 + 8600.0 * w.ppc;
+}
 
 // other 3-D grids, fitted (to 15 %) to lone marches of 16 x 16 to 512 x 8 on 1 to 16 CTAs with 1 to
 // 16 particles per cell: cells and particles of a CTA; in FP32 what spilled registers cost where a

@@ -77,3 +77,58 @@ def test_3d_cluster_sizes_follow_the_number_of_s_steps(host, grid):
     for n, line in zip(ns, host(body)):
         taken = list(sizes.values())[int(line)][2][n]
         assert taken <= 1.06 * min(v[2][n] for v in sizes.values()), n
+
+
+# measured, 128 x 128 x 512 FP32: particles per cell -> ms of n s-steps in one launch, 7 marches in
+# flight with an SM to each CTA and 14 with two CTAs per SM
+MEASURED_128 = {
+    1: ({7: 10.29, 8: 19.29, 14: 19.44, 21: 28.58, 28: 37.44},
+        {7: 12.57, 8: 15.00, 14: 15.40, 21: 26.13, 28: 29.28}),
+    2: ({7: 12.36, 8: 23.32, 14: 23.43, 21: 34.53, 28: 45.39},
+        {7: 15.72, 8: 18.79, 14: 19.42, 21: 32.42, 28: 36.86}),
+    4: ({7: 16.88, 8: 32.09, 14: 32.31, 21: 47.51, 28: 62.20},
+        {7: 21.62, 8: 26.15, 14: 27.13, 21: 45.00, 28: 51.53}),
+    8: ({7: 25.83, 8: 49.19, 14: 49.74, 21: 73.43, 28: 96.54},
+        {7: 33.33, 8: 40.77, 14: 43.86, 21: 72.20, 28: 84.21}),
+    16: ({7: 43.75, 8: 83.26, 14: 84.45, 21: 124.59, 28: 164.17},
+         {7: 59.47, 8: 72.85, 14: 81.54, 21: 134.30, 28: 157.04}),
+}
+
+
+@pytest.mark.parametrize("ppc", list(MEASURED_128))
+def test_two_ctas_per_sm_where_they_are_faster(host, ppc):
+    """A call, whole waves and the rest apart, takes no longer than the faster shape in one launch."""
+    shapes = "std::vector<ShapeTime> t;\n"
+    for dense, maxcl in ((0, 7), (1, 14)):
+        shapes += f"t.push_back({{slice_cycles({{128, 128, {ppc}, 4, 16, 1, {dense}, 0}}), {maxcl}}});\n"
+    for n in MEASURED_128[ppc][0]:
+        ms = 0.0
+        for line in host(shapes + f"for (int n = {n}; n > 0;) {{\n"
+                         "Pick k = pick_shape(t, n, 512, 4.0, 0, true);\n"
+                         'printf("%d %d\\n", k.shape, k.count);\nn -= k.count;\n}'):
+            shape, count = map(int, line.split())
+            ms += MEASURED_128[ppc][shape][count]
+        assert ms <= 1.02 * min(v[n] for v in MEASURED_128[ppc]), n
+
+
+# measured, 128 x 128 FP32 on short windows: (particles per cell, nz) -> ms of 8, 10 and 14 s-steps
+SHORT_128 = {
+    (1, 100): ({8: 3.741, 10: 3.790, 14: 4.000}, {8: 3.249, 10: 3.408, 14: 3.819}),
+    (2, 100): ({8: 4.527, 10: 4.625, 14: 4.860}, {8: 4.089, 10: 4.282, 14: 4.796}),
+    (8, 100): ({8: 9.504, 10: 9.713, 14: 10.390}, {8: 8.964, 10: 9.467, 14: 10.795}),
+    (16, 100): ({8: 16.090, 10: 16.484, 14: 17.726}, {8: 15.835, 10: 17.201, 14: 19.830}),
+    (16, 150): ({8: 24.290, 10: 24.646, 14: 25.615}, {8: 22.679, 10: 24.386, 14: 27.166}),
+    (16, 250): ({8: 40.356, 10: 41.061, 14: 41.838}, {8: 36.271, 10: 38.679, 14: 42.082}),
+}
+
+
+@pytest.mark.parametrize("ppc,nz", list(SHORT_128))
+def test_two_ctas_per_sm_on_short_windows(host, ppc, nz):
+    body = "std::vector<ShapeTime> t;\n"
+    for dense, maxcl in ((0, 7), (1, 14)):
+        body += f"t.push_back({{slice_cycles({{128, 128, {ppc}, 4, 16, 1, {dense}, 0}}), {maxcl}}});\n"
+    for n in (8, 10, 14):
+        body += f'printf("%d\\n", pick_shape(t, {n}, {nz}, 4.0, 0, false).shape);\n'
+    for n, line in zip((8, 10, 14), host(body)):
+        both = [v[n] for v in SHORT_128[ppc, nz]]
+        assert both[int(line)] <= 1.05 * min(both), n
