@@ -381,10 +381,11 @@ void take_shape(Params& q, const Params& b, int eb) {
 // With `count`, the launch may take only the first *count of the n s-steps (pick_shape).
 Params plan_launch(const gempic_sim* s, int n, double lag = kLag, int* count = nullptr) {
   std::vector<gempic::ShapeTime> t;
-  for (const gempic_sim::Shape& c : s->shapes)
-    t.push_back({gempic::slice_cycles({c.p.nx, c.p.ny, c.p.ppc_sum, s->eb, c.p.C, c.p.split, c.p.dense,
-                                       c.p.smem_bytes}),
-                 c.maxcl});
+  for (const gempic_sim::Shape& c : s->shapes) {
+    const gempic::SliceWork w{c.p.nx, c.p.ny, c.p.ppc_sum, s->eb, c.p.C, c.p.split, c.p.dense, c.p.smem_bytes};
+    // (two CTAs per SM: s->pmax marches have an SM to each CTA)
+    t.push_back({gempic::slice_cycles(w), c.maxcl, gempic::slice_cycles(w, false), c.p.dense ? s->pmax : c.maxcl});
+  }
   const gempic::Pick k = gempic::pick_shape(t, n, s->p.nz, lag, s->cfg.pipeline_depth, count != nullptr);
   Params q = s->p;
   if (k.shape >= 0) take_shape(q, s->shapes[k.shape].p, s->eb);
@@ -1275,13 +1276,14 @@ gempic_status gempic_step_streamed(gempic_sim* s, int32_t n, void* host, size_t 
   e = cudaPointerGetAttributes(&at, host);
   if (e != cudaSuccess) return cuda_fail(s, e);
   const bool pinned = at.type == cudaMemoryTypeHost;
-  // an s-step trails the one before it by a group (its copies out and in take less than a
-  // group's slices), which decides between the shapes: 14 s-steps of 128 x 128 x 1024 take 60 ms
-  // with 7 in flight and 57 with 14 (two CTAs per SM), 28 take 115 and 101; groups of 4 MiB
-  // 59, of 2 MiB 64, of 12 MiB 61.  2-D grids march in the simulation's own shape.
+  // an s-step trails the one before it by a group of slices and its copies out and in, 16 slices
+  // more on 128 x 128, which decides between the shapes: with 7 in flight and with 14 (two CTAs per
+  // SM), 14 s-steps of 512 slices take 29.8 and 31.7 ms, of 700 39.4 and 40.8, of 1024 59 and 56, 28 of
+  // 1024 115 and 101; 9 of 700 35.9 and 33.6.  Groups of 4 MiB instead of 8: 14 of 1024 59 ms, of 2 MiB
+  // 64, of 12 MiB 61.  2-D grids march in the simulation's own shape.
   const int deepest = s->p.ring - 2;
   Params q = s->p;
-  if (s->p.ny > 1) q = plan_launch(s, n, chunk + kLag);
+  if (s->p.ny > 1) q = plan_launch(s, n, chunk + 16.0);
   else q.P = std::min(s->pmax, n);
   q.k0 = s->k;
   q.nsteps = n;

@@ -28,12 +28,13 @@ inline double slice_cycles_2d(const SliceWork& w) {
   return 10.0 * np + 8500.0 + 28.0 * w.nx + (S > 1 ? 900.0 + 1200.0 * (S - 1) : 0.0);
 }
 
-// 128 x 128 FP32, fitted to 7 marches in flight with an SM to each CTA and to 8 to 14 with two CTAs
-// per SM (whose slices take the shared pace as soon as some SMs hold two), 512 slices: 40, 48, 65, 100,
-// 169 k cycles with 1, 2, 4, 8, 16 per cell, and 56, 71, 100, 161, 299 k (one species or two; a bunch
-// adds the same share to both)
-inline double slice_cycles_128(const SliceWork& w) {
-  return w.dense ? 42500.0 + 14700.0 * w.ppc : 30600.0 + 8600.0 * w.ppc;
+// 128 x 128 FP32, k cycles of a slice with 1, 2, 4, 8, 16 per cell (one species or two; a bunch adds
+// the same share to all): 40, 48, 65, 100, 169 with 512 threads and an SM to each CTA; 256 threads
+// with two CTAs on some SM 57, 72, 101, 165, 307, with an SM each 49, 61, 83, 129, 230
+inline double slice_cycles_128(const SliceWork& w, bool shared) {
+  if (!w.dense) return 30600.0 + 8600.0 * w.ppc;
+  // (quadratic: the particles of the marches in flight outgrow the L2)
+  return shared ? 43400.0 + (13800.0 + 167.0 * w.ppc) * w.ppc : 36500.0 + 12000.0 * w.ppc;
 }
 
 // other 3-D grids, fitted (to 15 %) to lone marches of 16 x 16 to 512 x 8 on 1 to 16 CTAs with 1 to
@@ -48,9 +49,10 @@ inline double slice_cycles_3d(const SliceWork& w) {
   return 19800.0 + 11.9 * c + 10.0 * np + l1 + (w.nx >= 256 ? 700.0 * w.C : 0.0);
 }
 
-inline double slice_cycles(const SliceWork& w) {
+// shared: while more marches are in flight than have an SM to each CTA
+inline double slice_cycles(const SliceWork& w, bool shared = true) {
   if (w.ny == 1) return slice_cycles_2d(w);
-  return w.eb == 4 && w.nx == 128 && w.ny == 128 ? slice_cycles_128(w) : slice_cycles_3d(w);
+  return w.eb == 4 && w.nx == 128 && w.ny == 128 ? slice_cycles_128(w, shared) : slice_cycles_3d(w);
 }
 
 // Slice times that n marches over nz slices take, P of them in flight: march i starts `lag` slices
@@ -65,7 +67,20 @@ inline double wavefront_slices(int n, int P, int nz, double lag) {
 struct ShapeTime {
   double cycles;                   // of one slice
   int maxcl;                       // marches in flight at most
+  double alone;                    // of one slice with an SM to each CTA,
+  int alone_cl;                    // which at most so many marches in flight have
 };
+
+// Modelled cycles of n marches over nz slices, P in flight.  Marches that share SMs hold up those
+// behind them, so all go at the shared pace while more than alone_cl are in flight: not in the
+// first alone_cl lags, the last ones, or a last wave of few.
+inline double march_cycles(const ShapeTime& t, int n, int P, int nz, double lag) {
+  const double total = wavefront_slices(n, P, nz, lag);
+  if (P <= t.alone_cl) return total * t.alone;
+  const bool few_last = n > P && (n - 1) % P + 1 <= t.alone_cl;
+  const double alone = std::min(total, 2.0 * t.alone_cl * lag + (few_last ? nz : 0));
+  return total * t.cycles - alone * (t.cycles - t.alone);
+}
 struct Pick {
   int shape;                       // index, -1: none can march
   int in_flight, count;            // marches in flight; s-steps of this launch
@@ -81,7 +96,7 @@ inline Pick pick_shape(const std::vector<ShapeTime>& shapes, int n, int nz, doub
   };
   const auto time = [&](int i, int m) {
     const int P = in_flight(i, m);
-    return P < 1 ? -1.0 : wavefront_slices(m, P, nz, lag) * shapes[i].cycles;
+    return P < 1 ? -1.0 : march_cycles(shapes[i], m, P, nz, lag);
   };
   const auto shortest = [&](int m, int* which) {
     double t0 = -1.0;

@@ -71,7 +71,7 @@ def test_3d_cluster_sizes_follow_the_number_of_s_steps(host, grid):
     ns = list(next(iter(sizes.values()))[2])
     body = "std::vector<ShapeTime> t;\n"
     for C, (smem, maxcl, _) in sizes.items():
-        body += f"t.push_back({{slice_cycles({{{nx}, {ny}, {ppc}, {eb}, {C}, 1, 0, {smem}}}), {maxcl}}});\n"
+        body += f"t.push_back({{slice_cycles({{{nx}, {ny}, {ppc}, {eb}, {C}, 1, 0, {smem}}}), {maxcl}, 0, 0}});\n"
     for n in ns:
         body += f'printf("%d\\n", pick_shape(t, {n}, 200, 4.0, 0, false).shape);\n'
     for n, line in zip(ns, host(body)):
@@ -100,7 +100,8 @@ def test_two_ctas_per_sm_where_they_are_faster(host, ppc):
     """A call, whole waves and the rest apart, takes no longer than the faster shape in one launch."""
     shapes = "std::vector<ShapeTime> t;\n"
     for dense, maxcl in ((0, 7), (1, 14)):
-        shapes += f"t.push_back({{slice_cycles({{128, 128, {ppc}, 4, 16, 1, {dense}, 0}}), {maxcl}}});\n"
+        shapes += (f"SliceWork w{dense}{{128, 128, {ppc}, 4, 16, 1, {dense}, 0}};\n"
+                   f"t.push_back({{slice_cycles(w{dense}), {maxcl}, slice_cycles(w{dense}, false), 7}});\n")
     for n in MEASURED_128[ppc][0]:
         ms = 0.0
         for line in host(shapes + f"for (int n = {n}; n > 0;) {{\n"
@@ -126,7 +127,8 @@ SHORT_128 = {
 def test_two_ctas_per_sm_on_short_windows(host, ppc, nz):
     body = "std::vector<ShapeTime> t;\n"
     for dense, maxcl in ((0, 7), (1, 14)):
-        body += f"t.push_back({{slice_cycles({{128, 128, {ppc}, 4, 16, 1, {dense}, 0}}), {maxcl}}});\n"
+        body += (f"SliceWork w{dense}{{128, 128, {ppc}, 4, 16, 1, {dense}, 0}};\n"
+                 f"t.push_back({{slice_cycles(w{dense}), {maxcl}, slice_cycles(w{dense}, false), 7}});\n")
     for n in (8, 10, 14):
         body += f'printf("%d\\n", pick_shape(t, {n}, {nz}, 4.0, 0, false).shape);\n'
     for n, line in zip((8, 10, 14), host(body)):

@@ -72,11 +72,11 @@ def test_dense_march_equals_single_steps(G, nz, ppc, a0, n, channel):
         _same_bits(a, b)
 
 
-@pytest.mark.parametrize("n", [14, 17])
-def test_dense_march_keeps_snapshot_and_current(G, n):
+@pytest.mark.parametrize("nz,n", [(260, 14), (520, 17)])
+def test_dense_march_keeps_snapshot_and_current(G, nz, n):
     """Fields and currents of the last s-step: in the dense launch itself (14), and where the call
     goes on in a second launch (17)."""
-    w = _lwfa(260, 2, 1.0, snapshot=True, capture_current=True)
+    w = _lwfa(nz, 2, 1.0, snapshot=True, capture_current=True)
     with G.Sim(w) as a, G.Sim(w) as b:
         launches = a.launch_count()
         a.step(0)
