@@ -155,7 +155,14 @@ typedef struct {
   const gempic_laser* laser;     /* NULL: no driver */
   int32_t stored_bucket_capacity;/* stored particles per zeta-cell and s-level; 0 = auto */
   int32_t particle_headroom;     /* extra streaming slots per CTA for rejoining particles; 0 = auto */
-  int32_t pipeline_depth;        /* s-steps marched concurrently (wavefront); 0 = auto, 1 = none */
+  /* s-steps marched concurrently (wavefront); 0 = auto, 1 = none.  The simulation holds as many
+   * s-levels as the deepest wavefront it may march and two more, each of nzeta (2 bucket capacity
+   * (4 + 7 reals) + 3 nx ny reals) bytes, from gempic_create on, whatever calls follow (128 x 128 x
+   * 1024 in FP32 with 2 per cell: 0.74 GB a level, 7 in flight 6.6 GB, 14 11.8 GB; 2-D grids up to
+   * 64 in flight).  Auto takes more than 7 (128 x 128 FP32) or 16 (elsewhere) only where the levels
+   * fit 16 GiB and a sixteenth of the free device memory; for many simulations on one device set
+   * the depth.  Results do not depend on it but for rounding. */
+  int32_t pipeline_depth;
   int32_t reserved;
   void* cuda_stream;             /* cudaStream_t; NULL = legacy default stream */
   const gempic_channel* channel; /* NULL: uniform density; copied at create */

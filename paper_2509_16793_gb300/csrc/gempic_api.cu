@@ -613,9 +613,16 @@ gempic_status create_sim(const gempic_config* cfg, gempic_sim** out, bool one_ct
   // marches in flight: a march trails the one before it by about four slices, so up to a quarter
   // of the window's slices march at once.  2-D marches take one CTA each, and 16 of them (the
   // limit of the clustered 3-D marches) left 136 of 152 SMs idle.  Beyond the depth that was always
-  // taken, the rings of s-levels (stored particles, rejoin queues, beam current) may take 16 GiB.
+  // taken, the rings of s-levels (stored particles, rejoin queues, beam current) are bounded
+  // (ring_levels): 128 x 128 x 1024 with 2 per cell takes 6.6 GB for 7 in flight, 11.8 for 14.
   const double level_bytes = (double)g.nzeta * (2.0 * p.bcap * (4 + 7 * s->eb) + 3.0 * g.nx * g.ny * s->eb);
-  const int levels = (int)std::min(128.0, 17179869184.0 / level_bytes) - 2;
+  size_t mem_free = 0, mem_total = 0;
+  e = cudaMemGetInfo(&mem_free, &mem_total);
+  if (e != cudaSuccess) {
+    delete s;
+    return GEMPIC_ECUDA;
+  }
+  const int levels = gempic::ring_levels(level_bytes, (double)mem_free) - 2;
   const int deepest = g.ny > 1 || s->shapes.empty() ? 16 : std::max(16, std::min(std::min(64, g.nzeta / 4), levels));
   s->pmax = cfg->pipeline_depth > 0 ? cfg->pipeline_depth : std::max(1, std::min(maxcl, deepest));
   if (s->pmax > std::max(1, maxcl)) s->pmax = std::max(1, maxcl);

@@ -64,6 +64,14 @@ inline double wavefront_slices(int n, int P, int nz, double lag) {
   return (double)((n - 1) / P) * wave + (double)((n - 1) % P) * lag + nz;
 }
 
+// Levels that a ring of s-levels may have for the sake of a deeper wavefront than was always taken
+// (7 marches of 128 x 128, 16 elsewhere): 16 GiB, and a sixteenth of the memory that is free, so that
+// one simulation of many, or on a full device, does not take room that the next one needs.
+inline int ring_levels(double level_bytes, double free_bytes) {
+  const double most = std::min(17179869184.0, free_bytes / 16.0);
+  return (int)std::min(128.0, most / level_bytes);
+}
+
 struct ShapeTime {
   double cycles;                   // of one slice
   int maxcl;                       // marches in flight at most

@@ -134,3 +134,12 @@ def test_two_ctas_per_sm_on_short_windows(host, ppc, nz):
     for n, line in zip((8, 10, 14), host(body)):
         both = [v[n] for v in SHORT_128[ppc, nz]]
         assert both[int(line)] <= 1.05 * min(both), n
+
+
+def test_ring_levels_leave_room(host):
+    """Deeper wavefronts take 16 GiB and a sixteenth of the free memory at most."""
+    gib = float(1 << 30)
+    cases = [(0.74e9, 280e9, 23), (0.74e9, 200e9, 16), (0.74e9, 100e9, 8), (0.74e9, 8e9, 0),
+             (1e6, 280e9, 128), (2 * gib, 1000 * gib, 8), (2 * gib, 16 * gib, 0)]
+    out = host("".join(f'printf("%d\\n", ring_levels({a}, {b}));\n' for a, b, _ in cases))
+    assert [int(v) for v in out] == [c for _, _, c in cases]

@@ -252,3 +252,21 @@ def test_denoised_chain_leaves_the_net_half_of_the_chip(G):
         for k in ("n_trapped", "n_stored", "n_rejoined", "pushes", "step"):
             assert da[k] == db[k], k
         assert abs(da["field_energy"] - db["field_energy"]) <= 4e-4 * db["field_energy"]
+
+
+def test_a_full_device_takes_the_former_depth(G):
+    """With less memory free than sixteen times the rings of 14 s-steps in flight (11.8 GB) a
+    128 x 128 x 1024 simulation takes those of 7, and is not refused."""
+    import torch
+    w = W.lwfa_3d_128x128x1024()
+    free, _ = torch.cuda.mem_get_info()
+    ballast = torch.empty(int(free - 90e9), dtype=torch.uint8, device="cuda")
+    try:
+        before, _ = torch.cuda.mem_get_info()
+        with G.Sim(w) as s:
+            assert before - torch.cuda.mem_get_info()[0] < 10e9
+            s.step(14)
+            assert not _two_ctas_per_sm(s) and s.last_launch()["in_flight"] == 7
+    finally:
+        del ballast
+        torch.cuda.empty_cache()
