@@ -476,11 +476,12 @@ void gempic_denoiser_destroy(gempic_denoiser* d);
  * one chain of 2n marches in one launch, each following the one before it slice by slice; up
  * to min(7, pipeline_depth) in flight, or, with pipeline_depth 0, as many as leave a quarter of
  * the SMs to the net (slices of 4096 nodes and more in rows of other than 128: a third, and
- * the marches take clusters that leave it half where there is a choice).  The calling thread runs the net on groups of half-slices as soon as the
- * first pass has written them and the three half-slices beyond, on a stream of its own, and
- * releases each group to the second pass, which waits for it (bounded).  The call waits for
- * its stream.  The diagnostics combine both passes: the field energy, on-axis E_z and stored
- * set are the second pass's, the streaming particles' energy, flux and counts the first's.
+ * the marches take clusters that leave it half where there is a choice).  The calling thread
+ * runs the net on groups of half-slices as soon as the first pass has written them and the three
+ * half-slices beyond, on a stream of its own, and releases each group to the second pass, which
+ * waits for it (bounded).  The call waits for its stream.  The diagnostics combine both passes:
+ * the field energy, on-axis E_z and stored set are the second pass's, the streaming particles'
+ * energy, flux and counts the first's.
  * d = NULL returns to plain steps.  The denoiser is borrowed: it must outlive its use.
  * GEMPIC_EINVAL for an FP64 simulation. */
 gempic_status gempic_set_denoiser(struct gempic_sim* sim, gempic_denoiser* d);

@@ -138,8 +138,8 @@ void note_launch(gempic_sim* s, const Params& q) {
 cudaError_t ensure_diag_cap(gempic_sim* s, int n) {
   if (n <= s->diag_cap) return cudaSuccess;
   double *d = nullptr, *o = nullptr, *r = nullptr, *gr = nullptr;
-  cudaError_t e = dalloc(s, &d, (size_t)n * gempic::kNDiag * std::max(s->p.C, s->p.ny == 1 ? kMaxSplit : 1) *
-                                    sizeof(double));
+  const int ranks = std::max(s->p.C, s->p.ny == 1 ? kMaxSplit : 1);
+  cudaError_t e = dalloc(s, &d, (size_t)n * gempic::kNDiag * ranks * sizeof(double));
   if (e != cudaSuccess) return e;
   e = dalloc(s, &o, (size_t)n * s->p.nz * sizeof(double));
   if (e != cudaSuccess) return e;
@@ -382,9 +382,11 @@ void take_shape(Params& q, const Params& b, int eb) {
 Params plan_launch(const gempic_sim* s, int n, double lag = kLag, int* count = nullptr) {
   std::vector<gempic::ShapeTime> t;
   for (const gempic_sim::Shape& c : s->shapes) {
-    const gempic::SliceWork w{c.p.nx, c.p.ny, c.p.ppc_sum, s->eb, c.p.C, c.p.split, c.p.dense, c.p.smem_bytes};
+    const Params& b = c.p;
+    const gempic::SliceWork w{b.nx, b.ny, b.ppc_sum, s->eb, b.C, b.split, b.dense, b.smem_bytes};
     // (two CTAs per SM: s->pmax marches have an SM to each CTA)
-    t.push_back({gempic::slice_cycles(w), c.maxcl, gempic::slice_cycles(w, false), c.p.dense ? s->pmax : c.maxcl});
+    const int alone_cl = b.dense ? s->pmax : c.maxcl;
+    t.push_back({gempic::slice_cycles(w), c.maxcl, gempic::slice_cycles(w, false), alone_cl});
   }
   const gempic::Pick k = gempic::pick_shape(t, n, s->p.nz, lag, s->cfg.pipeline_depth, count != nullptr);
   Params q = s->p;
@@ -516,11 +518,12 @@ gempic_status create_sim(const gempic_config* cfg, gempic_sim** out, bool one_ct
     const int fresh = RB * g.nx * ppc_sum;
     // a larger cluster than the slice needs shortens the march: the push and the transforms divide
     // by the CTAs, the barriers do not grow.  ms per s-step of one march, 96 slices, 2 per cell,
-    // C = 1, 2, 4, 8, 16: 16 x 16 FP32 1.31 1.11 1.10 1.05 -; 32 x 32 FP32 3.19 1.69 1.24 1.07 1.09;
-    // 64 x 64 FP32 - - 2.98 1.65 1.27; 32 x 32 FP64 - 21.1 11.4 6.9 5.1.  Clusters of 16 leave room
-    // for 7 marches where those of 8 leave 15: the simulation's own shape is the largest that still
-    // has work for its CTAs, and a call of many s-steps takes a smaller one (plan_launch).  ms for
-    // 48 s-steps of 200 slices on 8 and 16: 64 x 64 13.0, 17.3; 128 x 64 with 8 per cell 47.2, 58.9.
+    // C = 1, 2, 4, 8, 16: 16 x 16 FP32 1.31 1.11 1.10 1.05 -; 32 x 32 FP32 3.19 1.69 1.24 1.07
+    // 1.09; 64 x 64 FP32 - - 2.98 1.65 1.27; 32 x 32 FP64 - 21.1 11.4 6.9 5.1.  Clusters of 16
+    // leave room for 7 marches where those of 8 leave 15: the simulation's own shape is the
+    // largest that still has work for its CTAs, and a call of many s-steps takes a smaller one
+    // (plan_launch).  ms for 48 s-steps of 200 slices on 8 and 16: 64 x 64 13.0, 17.3; 128 x 64
+    // with 8 per cell 47.2, 58.9.
     if (chosen && fresh < (cand <= 8 ? 64 : cfg->precision == 64 ? 128 : 512)) break;
     Params t = p;
     t.C = cand;
@@ -913,8 +916,8 @@ static gempic_status denoised_chain(gempic_sim* s, int n) {
       most = c.maxcl;
     }
   }
-  const int want = s->cfg.pipeline_depth > 0 ? s->cfg.pipeline_depth
-                                             : std::max(1, gathers ? 2 * nsm / (3 * q.C) : 3 * nsm / (4 * q.C));
+  const int leave = std::max(1, gathers ? 2 * nsm / (3 * q.C) : 3 * nsm / (4 * q.C));
+  const int want = s->cfg.pipeline_depth > 0 ? s->cfg.pipeline_depth : leave;
   const int P = std::min(std::min(std::min(most, 2 * n), 7), want);
   const long long k0 = s->k;
   unsigned long long* done = s->dn_host;
@@ -1284,10 +1287,10 @@ gempic_status gempic_step_streamed(gempic_sim* s, int32_t n, void* host, size_t 
   if (e != cudaSuccess) return cuda_fail(s, e);
   const bool pinned = at.type == cudaMemoryTypeHost;
   // an s-step trails the one before it by a group of slices and its copies out and in, 16 slices
-  // more on 128 x 128, which decides between the shapes: with 7 in flight and with 14 (two CTAs per
-  // SM), 14 s-steps of 512 slices take 29.8 and 31.7 ms, of 700 39.4 and 40.8, of 1024 59 and 56, 28 of
-  // 1024 115 and 101; 9 of 700 35.9 and 33.6.  Groups of 4 MiB instead of 8: 14 of 1024 59 ms, of 2 MiB
-  // 64, of 12 MiB 61.  2-D grids march in the simulation's own shape.
+  // more on 128 x 128, which decides between the shapes: with 7 in flight and with 14 (two CTAs
+  // per SM), 14 s-steps of 512 slices take 29.8 and 31.7 ms, of 700 39.4 and 40.8, of 1024 59 and
+  // 56, 28 of 1024 115 and 101; 9 of 700 35.9 and 33.6.  Groups of 4 MiB instead of 8: 14 of 1024
+  // 59 ms, of 2 MiB 64, of 12 MiB 61.  2-D grids march in the simulation's own shape.
   const int deepest = s->p.ring - 2;
   Params q = s->p;
   if (s->p.ny > 1) q = plan_launch(s, n, chunk + 16.0);

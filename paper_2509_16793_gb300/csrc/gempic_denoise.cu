@@ -6,9 +6,10 @@
 //
 // Tensors are channel-last, X[z][y][x][16] in BF16 (z = half-slice, periodic across, zero
 // outside the window along zeta); rows of 128 voxels lie in memory in the tensor core's operand
-// layout and take conv_ws_kernel, described there.  Other widths (conv_kernel): a convolution is an implicit GEMM: a tile of 128 voxels
-// (consecutive in z, y, x order) is the M dimension, the 16 output channels N, and each of the
-// 27 taps adds a K = 16 slice (the 16 input channels of the tap's neighbour).  Per tap the
+// layout and take conv_ws_kernel, described there.  Other widths (conv_kernel): a convolution
+// is an implicit GEMM: a tile of 128 voxels (consecutive in z, y, x order) is the M dimension,
+// the 16 output channels N, and each of the 27 taps adds a K = 16 slice (the 16 input channels
+// of the tap's neighbour).  Per tap the
 // CTA gathers its tile's 128 neighbour voxels into shared memory in the tensor core's K-major
 // layout without swizzle (8-row x 16-byte core matrices: 128 B apart along K, 256 B apart
 // along M), one thread issues the MMA, and the 27 MMAs of a tile accumulate in 16 columns of
@@ -386,10 +387,12 @@ __device__ __forceinline__ uint64_t sdesc_row(uint32_t saddr) {
 // thread waits for its MMAs in flight before the tensor memory is freed, the staging thread for
 // its copies before the CTA ends.
 // Bound: the issuing thread and the tensor pipe, about half each.  An MMA of K = 16 takes 62-68
-// cycles on its CTA whatever N <= 128 is (88 with two CTAs on the SM), 596 of a unit's 1130
-// cycles; waits and commits take the rest.  128 x 128 x 512, 16 -> 16 channels: 346 us with
+// cycles on its CTA whatever N <= 128 is; with two CTAs on the SM, as here, a CTA completes one in
+// 88 and the SM's pipe one in 44.  MMAs are 596 of a unit's 1130 cycles; waits and commits take
+// the rest.  128 x 128 x 512, 16 -> 16 channels: 346 us with
 // asynchronous 16-byte copies by two warps, 325 us with bulk copies, 164 us with the two
-// single-thread roles cut to a few instructions per unit (DRAM floor 75 us); last layer 500 -> 204 us.
+// single-thread roles cut to a few instructions per unit (DRAM floor 75 us); last layer 500 ->
+// 204 us.
 constexpr int kUnits = 6;                            // ring of staged units
 constexpr int kStripW = 14;                          // output rows per strip
 constexpr int kSets = kStripW + 2;                   // accumulator sets (16 columns each)
@@ -430,7 +433,8 @@ __device__ __forceinline__ void tmem_zero16(uint32_t taddr) {
 }
 
 // What the epilogue of voxel x of row (z, y) reads: the current (last layer) or the mask
-// (backward); loaded a row ahead, so that its latency passes meanwhile (the last layer took 0.49 ms at 128 x 128 x 512, 3.0 k cycles a row in these loads)
+// (backward); loaded a row ahead, so that its latency passes meanwhile (the last layer took
+// 0.49 ms at 128 x 128 x 512, 3.0 k cycles a row in these loads)
 struct EpiIn {
   uint4 a, b;
 };
@@ -541,7 +545,8 @@ __global__ void __launch_bounds__(kWsThreads) conv_ws_kernel(ConvArgs a) {
 
   // The two single-thread roles run a few instructions per unit: ring slot and phase are
   // counters (a 64-bit modulo per unit and barrier cost the issuing thread more than its MMAs
-  // take: 190 cycles per MMA against 44 in the tensor pipe), descriptors advance by constants.
+  // take: 190 cycles per MMA where a CTA alone completes one in 62-68), descriptors advance by
+  // constants.
   if (warp == 0) {
     // ---- staging: units (z, r) for r = y0-1 .. y1 of every strip, in order; one thread ----
     if (lane == 0) {
@@ -769,7 +774,8 @@ __global__ void loss_kernel(const float* j, const float* t, const float* r, __nv
 // (in FP64), so gradients are reproducible bit for bit.
 // Bound: L2 and issue latency of the staging (16 KB per row and layer; the products are 1 % of
 // the tensor rate).  A training step at 128 x 128 x 32 voxels took 3.10 ms with FP32 FMA reductions
-// per tap and float atomics (2.7 ms of it here) and takes 0.43 ms.
+// per tap and float atomics (2.7 ms of it here) and 0.43 ms with this kernel; 0.34 with the row
+// convolution as it is now.
 constexpr int kSeg = 128;                            // voxels of a row segment
 constexpr int kGradWarps = 9;
 constexpr int kGradThreads = 32 * kGradWarps;

@@ -300,7 +300,8 @@ __device__ __forceinline__ Cx<T> twiddle(const Cx<T>* tw, int N, int m, bool inv
 // one stage per pass of all threads 18 of 45 k, each pass a barrier and a round trip through
 // shared memory.  Long FP32 rows take three stages per pass in registers; in FP64, whose rate
 // binds, and for rows of 8 or 16, which then occupy too few threads, that was slower (128 x 256
-// FP64 22.3 -> 23.0 ms, 16 x 16 0.56 -> 0.60 ms).  The butterflies and twiddles are those of the one-warp transform.
+// FP64 22.3 -> 23.0 ms, 16 x 16 0.56 -> 0.60 ms).  The butterflies and twiddles are those of a
+// transform by one warp.
 // Input in bit-reversed positions (bitrev); every thread of the CTA calls it.  SWZ: position q of
 // a row lies at swz(q), which spreads the strided accesses of the first passes over the banks.
 __device__ __forceinline__ int bitrev(int i, int logN) {
@@ -2040,8 +2041,8 @@ __device__ __forceinline__ void warp_diag_add(double* dwarp, int slot, V v) {
 //
 // Large buckets (a bunch) of a cluster: each CTA first copies the fields around the bunch (a window
 // of the cells around the mean of a sample, both planes, as much as the free column spectra's
-// shared memory holds) and gathers from the copy.  Without it the particles of a narrow bunch, dealt
-// out over the CTAs, read the two or three CTAs on the axis through distributed shared memory,
+// shared memory holds) and gathers from the copy.  Without it the particles of a narrow bunch,
+// dealt out over the CTAs, read the two or three CTAs on the axis through distributed shared memory,
 // 48 scattered values each: 31 k cycles of a slice on average with 2^20 macroparticles on
 // 128 x 128 x 768, 80 k where the bunch is, and as much in waits for the slowest CTA.  (Giving each
 // particle to the CTA of its row was slower: the two CTAs on the axis then do every reduction.)
@@ -2357,8 +2358,9 @@ __device__ void march(const Params& p, const Sm<T>& s_, const cg::cluster_group&
   // the received row spectra and the staging of the forward transform share the plane buffer
   // that the new fields will fill (the inverse transform of a row pair is in place), the
   // fixed-point accumulators share the column spectra, and a thread carries two modes whose old
-  // level is read when it is needed.  A march then takes 82 k cycles a slice instead of 54 k, with
-  // twice as many in flight: 128 x 128 x 1024, 2 per cell, 14 s-steps in a call, 52.3 -> 42.1 ms.
+  // level is read when it is needed.  A march then takes 78 k cycles a slice instead of 54 k, with
+  // twice as many in flight: 128 x 128 x 1024, 2 per cell, 14 s-steps in a call, 52.3 -> 40.7 ms
+  // (42.0 before the strides of the state's blocks were constants).
   constexpr bool DEN = SH == 2;
   constexpr int NM = DEN ? 2 : 1;                 // spectral modes per thread
   const bool varh = SH == 0 && p.varh != 0;

@@ -1,5 +1,5 @@
-// Modelled times of the launch shapes that a call of s-steps chooses from (host arithmetic, no CUDA).
-// The cycles are those of one GB300 at its clock of 2.07 GHz; only their ratios decide.
+// Modelled times of the launch shapes that a call of s-steps chooses from (host arithmetic, no
+// CUDA).  The cycles are those of one GB300 at its clock of 2.07 GHz; only their ratios decide.
 #pragma once
 
 #include <algorithm>
@@ -28,9 +28,9 @@ inline double slice_cycles_2d(const SliceWork& w) {
   return 10.0 * np + 8500.0 + 28.0 * w.nx + (S > 1 ? 900.0 + 1200.0 * (S - 1) : 0.0);
 }
 
-// 128 x 128 FP32, k cycles of a slice with 1, 2, 4, 8, 16 per cell (one species or two; a bunch adds
-// the same share to all): 40, 48, 65, 100, 169 with 512 threads and an SM to each CTA; 256 threads
-// with two CTAs on some SM 57, 72, 101, 165, 307, with an SM each 49, 61, 83, 129, 230
+// 128 x 128 FP32, k cycles of a slice with 1, 2, 4, 8, 16 per cell (one species or two; a bunch
+// adds the same share to all): 40, 48, 65, 100, 169 with 512 threads and an SM to each CTA; 256
+// threads with two CTAs on some SM 57, 72, 101, 165, 307, with an SM each 49, 61, 83, 129, 230
 inline double slice_cycles_128(const SliceWork& w, bool shared) {
   if (!w.dense) return 30600.0 + 8600.0 * w.ppc;
   // (quadratic: the particles of the marches in flight outgrow the L2)
@@ -46,7 +46,8 @@ inline double slice_cycles_3d(const SliceWork& w) {
   const double c = (double)w.nx * w.ny / w.C, np = c * w.ppc;
   if (w.eb == 8) return 60000.0 + 22.5 * std::log2((double)w.nx * w.ny) * c + 249.0 * np;
   const double l1 = w.smem_bytes > 212000 ? 13600.0 : w.smem_bytes > 200000 ? 10000.0 : 0.0;
-  return 19800.0 + 11.9 * c + 10.0 * np + l1 + (w.nx >= 256 ? 700.0 * w.C : 0.0);
+  const double rows = w.nx >= 256 ? 700.0 * w.C : 0.0;
+  return 19800.0 + 11.9 * c + 10.0 * np + l1 + rows;
 }
 
 // shared: while more marches are in flight than have an SM to each CTA
@@ -65,8 +66,8 @@ inline double wavefront_slices(int n, int P, int nz, double lag) {
 }
 
 // Levels that a ring of s-levels may have for the sake of a deeper wavefront than was always taken
-// (7 marches of 128 x 128, 16 elsewhere): 16 GiB, and a sixteenth of the memory that is free, so that
-// one simulation of many, or on a full device, does not take room that the next one needs.
+// (7 marches of 128 x 128, 16 elsewhere): 16 GiB, and a sixteenth of the memory that is free, so
+// that one simulation of many, or on a full device, does not take room that the next one needs.
 inline int ring_levels(double level_bytes, double free_bytes) {
   const double most = std::min(17179869184.0, free_bytes / 16.0);
   return (int)std::min(128.0, most / level_bytes);
@@ -97,7 +98,8 @@ struct Pick {
 // The shape that n s-steps of nz slices take the least modelled time in.  depth: marches in flight
 // at most, 0: no limit.  whole: the launch may take only the first `count` s-steps, whole waves of
 // its shape, and leave a last wave that would be nearly empty to a launch of another shape.
-inline Pick pick_shape(const std::vector<ShapeTime>& shapes, int n, int nz, double lag, int depth, bool whole) {
+inline Pick pick_shape(const std::vector<ShapeTime>& shapes, int n, int nz, double lag, int depth,
+                       bool whole) {
   const auto in_flight = [&](int i, int m) {
     const int P = std::min(m, shapes[i].maxcl);
     return depth > 0 ? std::min(P, depth) : P;
