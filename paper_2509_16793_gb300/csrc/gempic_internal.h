@@ -35,6 +35,7 @@ struct Params {
   // grid and decomposition
   int nx, ny, nz;                 // transverse nodes, slices
   int C, RB, KB, M;               // CTAs per slice, rows per CTA, kx per CTA, modes per CTA
+  int modes;                      // modes of a slice, C M
   int split;                      // 2-D: CTAs that share a march's particles (1: not split); the
                                   // cluster has C split CTAs
   int bunch;                      // 1: particles were placed in the box (a bunch)

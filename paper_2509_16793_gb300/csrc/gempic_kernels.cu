@@ -2539,8 +2539,8 @@ __device__ void march(const Params& p, const Sm<T>& s_, const cg::cluster_group&
       return (((size_t)c * p.nz + sl_) * p.ny + kyi[j]) * (size_t)nxh + kxg;
     } else {
       // (SH >= 1: 64 x 128 modes, 512 per CTA)
-      const int modes = SH >= 1 ? 64 * 128 : nxh * p.ny, m0 = me * (SH >= 1 ? 512 : p.M);
-      return (size_t)(b * 6 + c) * (size_t)modes + (size_t)(m0 + tid + j * NT);
+      const int m0 = me * (SH >= 1 ? 512 : p.M);
+      return ((size_t)b * 6 + c) * (size_t)(SH >= 1 ? 64 * 128 : p.modes) + m0 + tid + j * NT;
     }
   };
   // the public layout has no ghost slice and no j at half-slice -1
@@ -3590,6 +3590,7 @@ static int smem_layout_dense(Params& p) {
 }
 
 int smem_layout(Params& p, int eb) {
+  p.modes = p.nx / 2 * p.ny;
   // halo geometry: fields own rows + 1 above, currents rows -1 .. RB + 1 (3-D only)
   p.FR = p.ny > 1 ? p.RB + 1 : 1;
   p.JR = p.ny > 1 ? p.RB + 3 : 1;
