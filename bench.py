@@ -357,11 +357,11 @@ def main():
     flops = algorithmic_flops(w) * args.steps
     achieved = flops / (ms / 1e3) / 1e12
     hbm = algorithmic_bytes(w) * args.steps / (ms / 1e3) / 1e9
-    traffic = measured_traffic(w) * args.steps if measured_traffic(w) else None
+    traffic = measured_traffic(w, args.steps) if args.pipeline == 0 else None
     roof = {"bound": "alu", "achieved": achieved, "peak": peak_alu, "unit": "TFLOP/s",
             "frac": achieved / peak_alu, "traffic": traffic,
             "traffic_source": ("profiles/march_kernel_lwfa3d_128x128x1024.md (ncu DRAM bytes per "
-                               "s-step, used while its kernel hash matches the source)"
+                               "wave, used while its kernel hash matches the source)"
                                if traffic else None),
             "peak_source": f"measured: FP32 FMA probe (gempic_probe_fp32_fma, {probe_ms:.0f} ms, "
                            f"SM clock median {pclk.summary().get('sm_mhz')} MHz); spec figure "
@@ -441,17 +441,22 @@ def time_plain(w, steps: int, warmup: int, stream):
     return w.pushes_per_step * steps / (ms / 1e3), ms / steps
 
 
-def measured_traffic(w):
-    """DRAM bytes per s-step of the march kernel from the committed ncu summary, if it was
-    taken on this kernel source and this workload's grid (else None)."""
+def measured_traffic(w, steps: int):
+    """DRAM bytes of a call of `steps` s-steps from the committed ncu summary, if it was taken on
+    this source and this workload's grid (else None).  A wave of s-steps in flight moves the state
+    in and out once: whole waves of 14 (two CTAs per SM), the rest in a wave of its own, of up to
+    7 with one CTA per SM."""
     import re
     f = os.path.join(ROOT, "profiles", "march_kernel_lwfa3d_128x128x1024.md")
     if not os.path.exists(f) or (w.nx, w.ny, w.nzeta) != (128, 128, 1024) or w.precision != 32:
         return None
-    m = re.search(r"traffic_bytes_per_step: (\d+) kernel_hash: (\w+)", open(f).read())
-    if not m or m.group(2) != kernel_hash():
+    m = re.search(r"traffic_bytes_per_wave: (\d+) two CTAs per SM, (\d+) one "
+                  r"kernel_hash: (\w+)", open(f).read())
+    if not m or m.group(3) != kernel_hash():
         return None
-    return int(m.group(1))
+    two, one = int(m.group(1)), int(m.group(2))
+    whole, rest = divmod(steps, 14)
+    return whole * two + (0 if rest == 0 else one if rest <= 7 else two)
 
 
 def run_scan(args):
@@ -528,7 +533,7 @@ def run_scan(args):
 def kernel_hash() -> str:
     import hashlib
     h = hashlib.sha1()
-    for f in ("gempic_kernels.cu", "gempic_internal.h"):
+    for f in ("gempic_kernels.cu", "gempic_internal.h", "gempic_plan.h"):
         h.update(open(os.path.join(ROOT, "paper_2509_16793_gb300", "csrc", f), "rb").read())
     return h.hexdigest()[:12]
 
