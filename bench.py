@@ -316,6 +316,7 @@ def main():
             torch.distributed.barrier()
     sim.sync()
     launches = sim.launch_count() - launches0
+    shape["last_launch"] = sim.last_launch()         # the call's last wave may take another shape
     ms = max_over_ranks(e0.elapsed_time(e1), "cuda")
     ms_step = ms / args.steps
     value = job_rate(w.pushes_per_step * args.steps, world, ms / 1e3)
