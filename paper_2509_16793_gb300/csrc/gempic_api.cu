@@ -468,7 +468,11 @@ gempic_status create_sim(const gempic_config* cfg, gempic_sim** out, bool one_ct
   s->eb = cfg->precision == 64 ? 8 : 4;
 
   Params& p = s->p;
-  p.resid = (cfg->flags & GEMPIC_FLAG_RESIDUAL) ? 1 : 0;   // sizes shared memory
+  // what decides the kernel, before a shape is chosen: the residuals (which also size shared
+  // memory), the particle law, a zeta-step table
+  p.resid = (cfg->flags & GEMPIC_FLAG_RESIDUAL) ? 1 : 0;
+  p.gt1 = (cfg->flags & GEMPIC_FLAG_GT1) ? 1 : 0;
+  p.varh = s->hz.empty() ? 0 : 1;
   p.split = 1;
   p.nx = g.nx;
   p.ny = g.ny;
@@ -574,7 +578,6 @@ gempic_status create_sim(const gempic_config* cfg, gempic_sim** out, bool one_ct
   p.wait_spin_limit = 20000000;
   p.diag = (cfg->flags & GEMPIC_FLAG_DIAG) ? 1 : 0;
   p.snapshot = (cfg->flags & GEMPIC_FLAG_SNAPSHOT) ? 1 : 0;
-  p.gt1 = (cfg->flags & GEMPIC_FLAG_GT1) ? 1 : 0;
 
   e = gempic::configure_kernels(cfg->precision, p.smem_bytes, p.C);
   int maxcl = 1;
@@ -718,7 +721,6 @@ gempic_status create_sim(const gempic_config* cfg, gempic_sim** out, bool one_ct
       if (e != cudaSuccess) goto fail;
       p.hzt = hzt;
       p.zpd = zpd;
-      p.varh = 1;
     }
     // twiddles and shifts in FP64 on the host
     std::vector<double> t(ncx * 2 + nr);

@@ -270,3 +270,29 @@ def test_a_full_device_takes_the_former_depth(G):
     finally:
         del ballast
         torch.cuda.empty_cache()
+
+
+@pytest.mark.parametrize("option", ["refined", "residual"])
+def test_128_options_of_the_generic_kernel(G, option):
+    """Runs whose options the two-CTA march does not have take the generic one for any number of
+    s-steps, and give what single s-steps give."""
+    w = _lwfa(60)
+    w = w.with_(**{"refined": dict(hz=W.refined_h(w.nzeta, w.h, 2.0)),
+                   "residual": dict(residual=True)}[option])
+    with G.Sim(w) as a, G.Sim(w) as b:
+        a.step(14)
+        assert not _two_ctas_per_sm(a)
+        for _ in range(14):
+            b.step(1)
+        _same_bits(a, b)
+        if option == "residual":
+            da, db = a.diagnostics(), b.diagnostics()
+            assert abs(da["gauss_residual"] - db["gauss_residual"]) <= DIAG_RTOL * db["gauss_residual"]
+
+
+def test_128_gt1_takes_the_generic_kernel(G):
+    """(A GT1 run's stops amplify rounding: no comparison of many s-steps.)"""
+    w = _lwfa(60)
+    with G.Sim(w.with_(particle_law="GT1", delta=0.45 * w.nzeta * w.h), bucket_capacity=40000) as s:
+        s.step(8)
+        assert not _two_ctas_per_sm(s) and s.diagnostics()["n_rejoined"] > 0
