@@ -223,7 +223,9 @@ gempic_status gempic_add_particles(struct gempic_sim* sim, int64_t n, const doub
                                    const int32_t* species);
 
 /* Advance n s-steps (persistent device launches: one, or a few where the last wave of s-steps in
- * flight would be nearly empty), then wait and check the device status. */
+ * flight would be nearly empty), then wait and check the device status.  The launch shape follows
+ * n: the same s-steps in other calls agree to rounding (on 128 x 128 and in 2-D in FP32 bit for
+ * bit while no particle is stored; elsewhere sums over bands and CTAs are taken in another order). */
 gempic_status gempic_step(struct gempic_sim* sim, int32_t n);
 
 /* Same, without waiting: launches on the simulation's stream and returns. */
