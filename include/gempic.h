@@ -354,7 +354,9 @@ gempic_status gempic_last_launch(const struct gempic_sim* sim, int32_t* march_ct
 typedef struct gempic_batch gempic_batch;
 
 /* Create n >= 1 instances from cfgs[0..n-1], each validated like gempic_create (GEMPIC_EINVAL
- * also for mixed precisions); cuda_stream and pipeline_depth of the configs are ignored.
+ * also for mixed precisions, and for an instance whose slices do not fit one CTA: 2-D grids and 3-D
+ * ones of up to 32 x 32 do, if their particles leave room, 64 x 64 and larger do not, nor does
+ * cluster_ctas > 1); cuda_stream and pipeline_depth of the configs are ignored.
  * Runs the autotuner (a few s-steps of one throw-away simulation per size class).  On a
  * failure nothing is kept and the first failing status is returned. */
 gempic_status gempic_batch_create(const gempic_config* cfgs, int32_t n, gempic_batch** out);

@@ -215,6 +215,11 @@ gempic_status gempic_batch_create(const gempic_config* cfgs, int32_t n, gempic_b
     gempic_sim* sim = nullptr;
     st = gempic::batch_member(&c, &sim);
     if (st == GEMPIC_OK) b->sims.push_back(sim);
+    // the batch's marches are single CTAs: a slice that needs a cluster would reach for the shared
+    // memory of CTAs that are not there
+    int32_t ctas = 1;
+    if (st == GEMPIC_OK) st = gempic_launch_shape(sim, &ctas, nullptr, nullptr, nullptr);
+    if (st == GEMPIC_OK && ctas != 1) st = GEMPIC_EINVAL;
   }
   if (st == GEMPIC_OK) st = autotune(b, cfgs, n);
   // every simulation at the chosen CTA size; the launch takes the largest shared memory

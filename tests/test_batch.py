@@ -92,3 +92,19 @@ def test_batch_rejects_an_invalid_member():
     ws[1] = ws[1].with_(nx=24)                                 # not a power of two
     with pytest.raises(gempic.GempicError):
         gempic.Batch(ws)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("nx,ny,kw", [(64, 64, {}), (32, 64, {}), (16, 16, dict(cluster_ctas=2))])
+def test_instances_that_need_a_cluster_are_refused(nx, ny, kw):
+    """A batch marches single CTAs; one that fits is taken, alone and beside one that does not."""
+    from paper_2509_16793_gb300 import gempic
+    w = W.small_3d(nx=nx, ny=ny, nzeta=16, ppc=1, precision=32)
+    fits = W.small_3d(nx=16, ny=16, nzeta=16, ppc=1, precision=32)
+    for ws in ([w], [fits, w]):
+        with pytest.raises(gempic.GempicError) as e:
+            gempic.Batch(ws, **kw)
+        assert e.value.status == -1
+    with gempic.Batch([fits, fits]) as b:
+        b.step(2)
+        assert b.sims[0].diagnostics()["step"] == 2
