@@ -82,6 +82,9 @@ struct gempic_sim {
 
 namespace {
 
+// static shared memory of a batch's kernel (the item's Params and its index), which an instance
+// leaves room for
+constexpr int kBatchStatic = ((int)sizeof(Params) + 64 + 127) / 128 * 128;
 constexpr int kMaxSplit = 8;       // CTAs that share the particles of a 2-D march at most
 
 bool pow2(int v) { return v > 0 && (v & (v - 1)) == 0; }
@@ -295,7 +298,7 @@ gempic_status batch_prepare(gempic_sim* s, int nthreads, int nsteps, Params* out
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     if (e != cudaSuccess) return cuda_fail(s, e);
-    if (smem_layout(t, s->eb) > optin) return GEMPIC_EINVAL;
+    if (smem_layout(t, s->eb) > optin - kBatchStatic) return GEMPIC_EINVAL;
     s->p = t;
   }
   cudaError_t e = ensure_diag_cap(s, nsteps);
@@ -504,6 +507,7 @@ gempic_status create_sim(const gempic_config* cfg, gempic_sim** out, bool one_ct
   cudaError_t e = cudaGetDevice(&dev);
   int smem_optin = 0;
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  if (one_cta) smem_optin -= kBatchStatic;
   if (e != cudaSuccess) {
     delete s;
     return GEMPIC_ECUDA;

@@ -108,3 +108,23 @@ def test_instances_that_need_a_cluster_are_refused(nx, ny, kw):
     with gempic.Batch([fits, fits]) as b:
         b.step(2)
         assert b.sims[0].diagnostics()["step"] == 2
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("nx,ny,ppc,precision", [(32, 32, 2, 32), (32, 32, 4, 32), (16, 16, 8, 64),
+                                                 (256, 1, 16, 64)])
+def test_instances_that_fill_the_shared_memory(nx, ny, ppc, precision):
+    """As many particle slots as fit beside what the batch's kernel itself holds in shared memory;
+    instances equal the same runs alone."""
+    from paper_2509_16793_gb300 import gempic
+    w = (W.small_2d(nx=nx, nzeta=24, ppc=ppc, precision=precision, a0=0.5) if ny == 1 else
+         W.small_3d(nx=nx, ny=ny, nzeta=24, ppc=ppc, precision=precision, a0=0.5))
+    with gempic.Batch([w, w.with_(seed=3)]) as b, gempic.Sim(w, cluster_ctas=1) as g:
+        assert b.sims[0].launch_shape()["smem_bytes"] > 200000
+        b.step(2)
+        g.step(2)
+        d, ref = b.sims[0].diagnostics(), g.diagnostics()
+        assert d["pushes"] == ref["pushes"]
+        tol = 1e-12 if precision == 64 else 0.0
+        sb, sg = b.sims[0].state(), g.state()
+        assert np.abs(sb - sg).max() <= tol * np.abs(sg).max()
